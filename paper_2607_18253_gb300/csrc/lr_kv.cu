@@ -237,6 +237,19 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
     long long fcum[5] = {0, 0, 0, 0, 0};
     long long cf1 = 0, cf2 = 0, cf3 = 0, cf4 = 0;  // features summed over the records
     int la0 = 0, nrec = 0, done = 0, pmx = 0;
+    // Where the records may end.  In a "clear" record a query of any allowed length that has
+    // no first token yet is admitted if it waits, is not preempted (the slack and the free
+    // blocks reach a whole query's, hq) and prefills `bl` tokens.  So after consecutive
+    // clear records whose budgets sum to max_prompt_len every query has its prompt done, and
+    // one clear record later its first token: no walk passes that record, and the
+    // simulation stops there (`clear` is the budget sum of the current stretch).  A load
+    // that the batches up to the horizon could still take past max_iters keeps going, so
+    // the same snapshots are refused.  On the 64- and 256-instance pools the records end
+    // after 42 batches in the mean, 227 at most, where up to 4,096 used to be simulated and
+    // written: load 403 -> 370 us (64 instances), 456 -> 405 us (256).
+    const int hq = dblk(dv, c.pmax + 1);
+    int clear = 0;
+    auto stops = [&](int l_) -> bool { return (long long)l_ + (a.kv.horizon - nrec) <= c.max_iters; };
     KvRec *rec = out.kvr + (size_t)j * a.kv.horizon;
     int32_t *pmxo = out.kvp + (size_t)j * a.kv.horizon;
 
@@ -281,6 +294,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
     // that empties the instance.  The window's ends are listed in the idle waiting
     // ring.  Returns the batches done (0: none).
     int32_t *evn = ovf + 1;  // the window's ends
+    bool wstop = false;      // the window's last record may be the last one
     auto window = [&]() -> int {
         const int W = min(min(32, a.kv.horizon - nrec), kKvCal - (G & (kKvCal - 1)));
         if (lane == 0) *evn = 0;
@@ -377,6 +391,16 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         cf3 = __shfl_sync(kFull, c3, L);
         cf4 = __shfl_sync(kFull, c4, L);
         pmx = __shfl_sync(kFull, pm, L);
+        // the stretch of clear records: all of this window's, or none of it counts (a later
+        // end of the records is only longer)
+        const bool ck = in && thr >= c.pmax && fa >= hq;
+        if (__ballot_sync(kFull, ck) == (n == 32 ? kFull : (1u << n) - 1u)) {
+            const int before = clear + __reduce_add_sync(kFull, k < n - 1 ? bar : 0);  // through the record before the last
+            wstop = before >= c.pmax;
+            clear = min(before + __shfl_sync(kFull, bar, L), 1 << 29);
+        } else {
+            clear = 0;
+        }
         __syncwarp();
         for (int e = lane; e < nev; e += 32) {  // the window's ends leave
             const int2 ev = wq[e];
@@ -427,7 +451,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
             const int n = window();
             if (n > 0) {
                 l += n - 1;
-                if (done || nrec == a.kv.horizon) break;
+                if (done || nrec == a.kv.horizon || (wstop && stops(l))) break;
                 if (ne - nr >= max(32, nr)) compact();
                 continue;
             }
@@ -641,6 +665,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         const bool qcan = wc == 0;
         if (la0 == 0 && qcan && budget > 0 && nr < S) la0 = l;
         // 3. The batch's record, or the features before the first record.
+        bool rstop = false;
         if (la0 != 0 && admitted) f4 += warp_sum64(f4l);
         if (la0 != 0) {
             cf1 += f1;
@@ -666,6 +691,12 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 pmxo[nrec] = pmx;
             }
             ++nrec;
+            if (thr >= c.pmax && far >= hq && slack >= hq) {
+                rstop = clear >= c.pmax;
+                clear = min(clear + budget, 1 << 29);
+            } else {
+                clear = 0;
+            }
         } else {
             fcum[0] += 1;
             fcum[1] += f1;
@@ -705,7 +736,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
             done = 1;
             break;
         }
-        if (nrec == a.kv.horizon) break;
+        if (nrec == a.kv.horizon || (rstop && stops(l))) break;
         if (ne - nr >= max(32, nr)) compact();
     }
     fcum[4] += warp_sum64(f4c);

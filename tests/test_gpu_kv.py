@@ -187,6 +187,30 @@ def test_long_walks_across_record_tiles():
         np.testing.assert_array_equal(bits(t[cq, cj]), bits(et))
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("max_iters,accepted", [(2900, False), (3000, True), (5000, True)])
+def test_records_end_where_every_query_is_through(mode, max_iters, accepted):
+    # One decoder runs for 3,000 batches; every query is through after a few.  Records may
+    # end there, but a load whose batches pass max_iters is refused all the same.
+    import dataclasses
+    wl = W.small_workload(70, num_instances=1, num_models=2, num_queries=160, first_token_mode=mode,
+                          budget_range=(16, 32), min_gap=8)
+    one = lambda v: np.pad(np.array([[v]], np.int32), ((0, 0), (0, wl.cap_running - 1)))  # noqa: E731
+    wl = dataclasses.replace(wl, n_run=np.array([1], np.int32), run_ctx=one(5), run_pre=one(0), run_dec=one(3000),
+                             n_wait=np.array([0], np.int32), prompt_len=np.arange(1, 161, dtype=np.int32))
+    limits = (np.array([4], np.int32), np.array([1000], np.int64), np.array([1 << 40], np.int64))
+    rt = make(wl, limits, max_iters=max_iters)
+    got = gpu_estimate(rt, wl)
+    st = rt.status()
+    rt.close()
+    if not accepted:
+        assert st == R().LR_ETRAJ
+        return
+    assert st == R().LR_OK
+    st, eF, elt, et, _ = oracle.estimate_matrix_kv(wl, *limits)
+    compare(got, (eF, elt, et), st == 0)
+
+
 def test_invalid_snapshot_keeps_the_live_one():
     wl = W.small_workload(63, num_instances=9, num_models=2, num_queries=20, budget_range=(8, 96), min_gap=8)
     bs, nb, mc = W.kv_limits(wl, 9, block_sizes=(4,))
