@@ -230,6 +230,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
 
     long long freeb = nbk - held;
     int nr = nr0, ne = nr0;                             // running requests; slots in use
+    int tl = nr0;                                       // past the last running request's slot (holes follow it)
     int pfs = (nr0 > 0 && rq[nr0 - 1].y > 0) ? nr0 - 1 : -1;  // the prefill request's slot
     int wh = 0, wc = nw0;                               // waiting ring head and count
     int G = 0, gr = 0;                                  // batches done; G mod bs
@@ -271,7 +272,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
             kept += __popc(m);
             __syncwarp();
         }
-        ne = kept;
+        ne = tl = kept;
         for (int b = lane; b < kKvCal; b += 32) head[b] = -1;
         if (lane == 0) *ovf = -1;
         __syncwarp();
@@ -456,6 +457,64 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 continue;
             }
         }
+        // Runs of batches in which the waiting head cannot be admitted (no seat, no budget
+        // or not its first chunk's blocks) and nothing but decoders runs, before the first
+        // record: most batches of a load that queues on a full cache.  Each takes one
+        // histogram and one calendar word; the run stops, with that batch untouched, where
+        // the blocks do not suffice or the head gets in.  Bound by the chain of shared-memory
+        // reads and branches, not by bandwidth: with this loop (about 100 cycles a batch, the
+        // step below about 1,000) and the one-by-one preemption, load 370 -> 241 us on the
+        // 64-instance pool (389 of the slowest instance's 465 batches are such), 405 -> 255
+        // us on 256 instances.
+        if (la0 == 0 && pfs < 0 && wc > 0) {
+            const int hp = wq[wh].x;
+            int need1 = dblk(dv, min(hp, B - nd));
+            int ridx = gr == 0 ? 0 : bs - gr;  // residue of the contexts at a block boundary
+            long long r2 = 0, r3 = 0;
+            const int G0 = G;
+            while (l <= c.max_iters && (G == G0 || (G & (kKvCal - 1)) != 0)) {
+                const int need = hist[ridx];
+                int s = head[G & (kKvCal - 1)];
+                const long long fa = freeb - need;
+                if (fa < 0 || (nr < S && B > nd && need1 <= fa)) break;
+                freeb = fa;
+                r2 += nd;
+                r3 += src + (long long)nd * G;
+                if (s >= 0) {
+                    do {  // the decoders whose last batch this is return their blocks
+                        const int ns = nxt[s];
+                        const int4 q = rq[s];
+                        if (q.y == 0) {
+                            freeb += eb[s];
+                            src -= q.x;
+                            --nd;
+                            if (lane == 0) {
+                                hist[q.w] -= 1;
+                                reinterpret_cast<int *>(rq + s)[1] = -1;
+                            }
+                        }
+                        s = ns;
+                    } while (s >= 0);
+                    if (lane == 0) head[G & (kKvCal - 1)] = -1;
+                    nr = nd;
+                    need1 = dblk(dv, min(hp, B - nd));
+                    __syncwarp();
+                }
+                ++G;
+                ++l;
+                ridx = ridx == 0 ? bs - 1 : ridx - 1;
+            }
+            if (G != G0) {
+                gr = ridx == 0 ? 0 : bs - ridx;
+                fcum[0] += G - G0;
+                fcum[2] += r2;
+                fcum[3] += r3;
+                if (l > c.max_iters || (G & (kKvCal - 1)) == 0) {  // the loop's head takes these
+                    --l;
+                    continue;
+                }
+            }
+        }
         // 1. The running scan.  n_run <= S <= B and only the last request may be in
         //    prefill, so every request gets its tokens if the blocks suffice: one per
         //    decoder, and the last one's chunk from what the decoders leave.
@@ -488,66 +547,41 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
             // queue.  The prefill request, last, goes first, so the survivors are
             // decoders.
             // Every request's blocks after the batch sum to what is held plus what the
-            // batch needs, so the cut is found from the tail: the first slot cut (from the
-            // end) whose suffix of post-batch blocks reaches the excess over nb_j.  Usually
-            // few requests go, and the walk stops in the first 32 slots.
-            const long long total = (nbk - freeb) + need_all, excess = total - nbk;
-            long long acc = 0, fitb = -1;  // post-batch blocks: of the suffix so far; of the survivors
-            int cut = 0;
-            for (int top = ne - 1; top >= 0; top -= 32) {
+            // batch needs, so requests leave from the tail until their post-batch blocks
+            // reach the excess over nb_j: usually one or two, taken one by one (every lane
+            // on the same values; a scan over 32 slots and a second pass to move them cost
+            // three times as much).
+            const int excess = need_all - (int)freeb;  // need_all > freeb >= 0
+            long long acc = 0;                         // post-batch blocks of those gone
+            for (int top = tl - 1; top >= 0 && acc < excess; top -= 32) {
                 const int s = top - lane;
-                long long wv = 0;
-                if (s >= 0) {
-                    const int4 q = rq[s];
-                    if (q.y == 0) wv = dblk(dv, q.x + G + 1);
-                    else if (q.y > 0) wv = dblk(dv, q.x + px);
-                }
-                const long long suf = acc + warp_incl_sum64(wv, lane);
-                const unsigned hit = __ballot_sync(kFull, s >= 0 && suf >= excess);
-                if (hit) {
-                    const int l0 = __ffs(hit) - 1;
-                    cut = top - l0;
-                    fitb = total - __shfl_sync(kFull, suf, l0);
-                    break;
-                }
-                acc = __shfl_sync(kFull, suf, 31);
-            }
-            if (fitb < 0) fitb = total - acc;  // (unreachable: the whole list reaches the excess)
-            int m = 0;
-            for (int base = cut; base < ne; base += 32) {
-                const int s = base + lane;
-                m += __popc(__ballot_sync(kFull, s < ne && rq[s].y >= 0));
-            }
-            const int wh2 = (wh - m + C) % C;
-            int k0 = 0, gd = 0;
-            long long gone = 0;
-            for (int base = cut; base < ne; base += 32) {
-                const int s = base + lane;
-                const int4 q = s < ne ? rq[s] : make_int4(0, -1, 0, 0);
-                const bool live = q.y >= 0;
-                const unsigned bl = __ballot_sync(kFull, live);
-                if (live) {
-                    int slot = wh2 + k0 + __popc(bl & ((1u << lane) - 1u));
-                    if (slot >= C) slot -= C;
+                unsigned live = __ballot_sync(kFull, s >= 0 && reinterpret_cast<const int *>(rq + s)[1] >= 0);
+                while (live != 0u && acc < excess) {
+                    const int l0 = __ffs(live) - 1;
+                    live &= live - 1u;
+                    const int r = top - l0;
+                    const int4 q = rq[r];
+                    wh = wh == 0 ? C - 1 : wh - 1;
                     if (q.y == 0) {
-                        wq[slot] = make_int2(q.x + G, q.z - G);
-                        atomicSub(&hist[q.w], 1);
-                        gone += q.x;
-                        ++gd;
+                        acc += dblk(dv, q.x + G + 1);
+                        src -= q.x;
+                        --nd;
+                        if (lane == 0) {
+                            wq[wh] = make_int2(q.x + G, q.z - G);
+                            hist[q.w] -= 1;
+                        }
                     } else {
-                        wq[slot] = make_int2(q.x + q.y, q.z);
+                        acc += dblk(dv, q.x + px);
+                        if (lane == 0) wq[wh] = make_int2(q.x + q.y, q.z);
                     }
-                    reinterpret_cast<int *>(rq + s)[1] = -1;
+                    if (lane == 0) reinterpret_cast<int *>(rq + r)[1] = -1;
+                    ++wc;
+                    --nr;
+                    tl = r;
                 }
-                k0 += __popc(bl);
             }
-            src -= warp_sum64(gone);
-            nd -= warp_sum32(gd);
-            if (pfs >= cut) pfs = -1;
-            wh = wh2;
-            wc += m;
-            nr -= m;
-            freeb = nbk - fitb;
+            pfs = -1;
+            freeb = acc - excess;
             budget = B - nr;
             f1 = 0;
             f2 = nd;
@@ -636,6 +670,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 freeb -= sb;
                 nr += k;
                 ne += k;
+                tl = ne;
                 wh = wh + k >= C ? wh + k - C : wh + k;
                 wc -= k;
             }
@@ -651,7 +686,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                         f1 += x;
                         f4 += (long long)x * (x + 1) / 2;
                         ++nr;
-                        ++ne;
+                        tl = ++ne;
                         wh = wh + 1 >= C ? wh + 1 - C : wh + 1;
                         --wc;
                         budget -= x;
