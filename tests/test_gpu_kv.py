@@ -212,20 +212,21 @@ def test_records_end_where_every_query_is_through(mode, max_iters, accepted):
 
 
 @pytest.mark.parametrize("mode", [0, 1])
-@pytest.mark.parametrize("bs", [1, 3, 16])
+@pytest.mark.parametrize("bs", [3, 1024, 4096])
 def test_long_blocked_queues(mode, bs):
-    # The waiting head stays blocked, by seats (instance 0) or by blocks (1, 2), past the
-    # calendar's re-file boundary at 1,024 batches; instance 2's decoders preempt one another.
+    # The waiting head stays blocked, by seats (instance 0) or by blocks (1 and 2, whose decoders
+    # preempt one another with the smaller blocks), past the calendar's re-file boundary at
+    # 1,024 batches.
     import dataclasses
     wl = W.small_workload(80, num_instances=3, num_models=2, num_queries=6, first_token_mode=mode, cap_running=8,
                           cap_waiting=8, max_prompt_len=60)
     rep = lambda v: np.array([v, v, v], np.int32)  # noqa: E731
     wl = dataclasses.replace(
         wl, max_batched_tokens=rep(64), max_seqs=np.array([4, 8, 8], np.int32), n_run=rep(4),
-        run_ctx=rep([40, 50, 60, 70, 0, 0, 0, 0]), run_pre=rep([0] * 8), run_dec=rep([1500, 1100, 1023, 1400, 0, 0, 0, 0]),
+        run_ctx=rep([400, 500, 600, 700, 0, 0, 0, 0]), run_pre=rep([0] * 8), run_dec=rep([1500, 1100, 1023, 1400, 0, 0, 0, 0]),
         n_wait=rep(4), wait_pre=rep([30, 64, 90, 5, 0, 0, 0, 0]), wait_dec=rep([40, 1, 300, 20, 0, 0, 0, 0]))
-    whole = 220 + 1500 + 1100 + 1023 + 1400
-    nb = np.array([10 * whole, whole // bs + 5, (whole * 2 // 3) // bs], np.int64)
+    nb = np.array([10_000, 2200 // bs + (40 if bs == 3 else 2), 2200 // bs + (8 if bs == 3 else 4)], np.int64)
+    nb[1:] = np.maximum(nb[1:], 4)  # one block a running request at least
     limits = (rep(bs), nb, np.array([1 << 40] * 3, np.int64))
     check(wl, limits)
 
