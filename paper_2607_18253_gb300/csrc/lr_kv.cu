@@ -33,6 +33,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr long long kHuge = 1LL << 62;
+constexpr int kBigKv = 0x7fffffff;
 
 __device__ __forceinline__ long long kv_blocks(long long c, long long bs) { return (c + bs - 1) / bs; }
 // ceil(c / bs) for 0 <= c < 2^31 (32-bit division)
@@ -122,11 +123,11 @@ __device__ __forceinline__ int dres(const Div32 &v, int x) {
 // One instance's residents alone, batch by batch, from the snapshot.  Every lane
 // holds the same scalar state.
 //
-// Running request in slot s: rq[s] = (context, prefill, decode, blocks held) for
-// the prefill request, (context - G, 0, decode + G, context residue mod bs) for a
-// decoder, whose blocks at its end wait in eb[s].  Slots keep the list's order; a
-// request that leaves becomes a hole (prefill -1) until a compaction.  Only the
-// last running request may be in prefill (slot pfs).  The others decode one token
+// Running request in slot s: rq[s] = (context - G, 0, decode + G, context residue mod
+// bs) for a decoder, whose blocks at its end wait in eb[s].  Slots keep the list's
+// order; a request that leaves becomes a hole (second word -1) until a compaction.  Only
+// the last running request may be in prefill (slot pfs, second word 1, its state in
+// registers).  The others decode one token
 // a batch (G = batches done), so no word of theirs changes until they end.  The
 // decoders crossing into a new block in batch G are those whose context is a
 // multiple of bs, counted by a histogram of stored contexts mod bs; their context
@@ -232,9 +233,16 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
     int nr = nr0, ne = nr0;                             // running requests; slots in use
     int tl = nr0;                                       // past the last running request's slot (holes follow it)
     int pfs = (nr0 > 0 && rq[nr0 - 1].y > 0) ? nr0 - 1 : -1;  // the prefill request's slot
+    int pC = 0, pP = 0, pD = 0, pH = 0;                       // its context, prefill, decode and blocks
+    if (pfs >= 0) {
+        const int4 q = rq[pfs];
+        pC = q.x;
+        pP = q.y;
+        pD = q.z;
+        pH = q.w;
+    }
     int wh = 0, wc = nw0;                               // waiting ring head and count
     int G = 0, gr = 0;                                  // batches done; G mod bs
-    long long f4c = 0;                                  // this lane's part of F4 before the first record
     long long fcum[5] = {0, 0, 0, 0, 0};
     long long cf1 = 0, cf2 = 0, cf3 = 0, cf4 = 0;  // features summed over the records
     int la0 = 0, nrec = 0, done = 0, pmx = 0;
@@ -334,14 +342,13 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         // the prefill request's chunk: what the decoders leave, until it finishes
         int x = 0, pneed = 0, ctxp = 0, remk = 0;
         bool pf_ends = false;
-        const int4 pq = pfs >= 0 ? rq[pfs] : make_int4(0, 0, 0, 0);
         if (pfs >= 0) {
             const int avail = B - ndk;
             const int before = warp_incl_sum32(k < W ? avail : 0, lane) - (k < W ? avail : 0);
-            remk = max(0, pq.y - before);
+            remk = max(0, pP - before);
             x = min(remk, avail);
             pf_ends = remk - x == 0;
-            ctxp = pq.x + (pq.y - remk);
+            ctxp = pC + (pP - remk);
             pneed = dblk(dv, ctxp + x) - dblk(dv, ctxp);
         }
         const int need_all = need_d + pneed;
@@ -411,7 +418,11 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
             }
         }
         if (in) head[(G + k) & (kKvCal - 1)] = -1;
-        if (pfs >= 0 && lane == 0) rq[pfs] = make_int4(ctxpL + xL, remL - xL, pq.z, dblk(dv, ctxpL + xL));
+        if (pfs >= 0) {
+            pC = ctxpL + xL;
+            pP = remL - xL;
+            pH = dblk(dv, pC);
+        }
         nd = ndL - cntL;
         nr = nrL - cntL;
         src = srcL - rckL;
@@ -424,7 +435,42 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         return n;
     };
 
-    for (int l = 1;; ++l) {
+    // The batch step, in two forms.  Both are bound by the chain of shared-memory reads,
+    // divisions and branches of one warp (no bandwidth or issue limit is near), and most
+    // batches admit, preempt or end one or two requests, so every lane runs them as scalar
+    // code on the same values and requests are taken one by one: scans over 32 candidates
+    // cost several times what they saved (about 1,900 cycles for a batch with an admission).
+    // The prefill request and the waiting head stay in registers.
+    int ridx = 0;        // residue of the stored contexts at a block boundary in batch G
+    int hp = 0, hd = 0;  // the waiting head (prompt, decode), if any waits
+    if (wc > 0) {
+        hp = wq[wh].x;
+        hd = wq[wh].y;
+    }
+    // a decoder from batch G + 1 on, in slot s, with context ctx (of residue rem) and dec tokens to go
+    auto decode_from_next = [&](int s, int ctx, int rem, int dec) {
+        const int x = ctx - (G + 1), z = dec + (G + 1);
+        int res = rem - (gr + 1);  // x mod bs
+        if (res < 0) res += bs;
+        const int4 q = make_int4(x, 0, z, res);
+        const long long E = kv_end(q, mctx);
+        const int ebv = dblk(dv, (int)(x + E + 1));
+        int32_t *h = E < (long long)G + kKvCal ? &head[E & (kKvCal - 1)] : ovf;
+        if (lane == 0) {
+            rq[s] = q;
+            eb[s] = ebv;
+            nxt[s] = *h;
+            *h = s;
+            hist[res] += 1;
+        }
+        src += x;
+        ++nd;
+    };
+    const int mctx_i = (int)min(mctx, 1LL << 30);  // no context reaches 2^30 tokens
+    const int bB = dblk(dv, B - S + 1);            // the least blocks of a whole batch's budget with a seat free
+    const bool small = nbk < (1LL << 30);
+    for (;;) {
+        int l = G + 1;  // this batch
         if (l > c.max_iters) {
             kv_fail(a.ctl, kETraj, lane);
             return;
@@ -451,41 +497,172 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         if (la0 != 0 && wc == 0) {
             const int n = window();
             if (n > 0) {
-                l += n - 1;
-                if (done || nrec == a.kv.horizon || (wstop && stops(l))) break;
-                if (ne - nr >= max(32, nr)) compact();
+                if (done || nrec == a.kv.horizon || (wstop && stops(G))) break;
+                ridx = gr == 0 ? 0 : bs - gr;
                 continue;
             }
         }
-        // Runs of batches in which the waiting head cannot be admitted (no seat, no budget
-        // or not its first chunk's blocks) and nothing but decoders runs, before the first
-        // record: most batches of a load that queues on a full cache.  Each takes one
-        // histogram and one calendar word; the run stops, with that batch untouched, where
-        // the blocks do not suffice or the head gets in.  Bound by the chain of shared-memory
-        // reads and branches, not by bandwidth: with this loop (about 100 cycles a batch, the
-        // step below about 1,000) and the one-by-one preemption, load 370 -> 241 us on the
-        // 64-instance pool (389 of the slowest instance's 465 batches are such), 405 -> 255
-        // us on 256 instances.
-        if (la0 == 0 && pfs < 0 && wc > 0) {
-            const int hp = wq[wh].x;
-            int need1 = dblk(dv, min(hp, B - nd));
-            int ridx = gr == 0 ? 0 : bs - gr;  // residue of the contexts at a block boundary
-            long long r2 = 0, r3 = 0;
+        int s_end = 0, budget = 0, ndb = 0;  // (ndb: decoders of this batch)
+        int dying = 0;                       // requests leaving after this batch
+        long long back = 0;                  // and their blocks
+        long long slack = 0, far = 0;        // block slack of the running scan; free blocks after it
+        int bar = 0;                         // budget after it
+        long long f1 = 0, f3 = 0, f4 = 0;
+        bool scanned = false;                // the running scan of this batch is done
+        // The lean form, while requests wait and only decoders run: batch after batch until
+        // one needs the general form below (a prompt taken in chunks, the last waiting
+        // request, no slot left: from after its running scan on) or the calendar, the
+        // iteration bound or the horizon is reached.  A batch without any event costs one
+        // histogram and one calendar word: it is told by the free blocks staying below
+        // `hm`, under which the head cannot get in, and no end.  With it, load 241 -> 144 us
+        // on the 64-instance pool (370 before any of this), 255 -> 184 us on 256 instances
+        // (405), whose slowest instance steps 455 batches with 129 admissions and 55
+        // preemptions.
+        if (small && pfs < 0 && wc > 0) {
+            int fb = (int)freeb;
+            int hb = 0, hrem = 0, hfin = 0, hm = 0;  // the head's blocks, residue and last context; the blocks it needs
+            auto derive = [&]() {
+                const int qt = (int)udiv32(dv, (unsigned)hp);
+                hrem = hp - qt * bs;
+                hb = qt + (hrem > 0 ? 1 : 0);
+                hfin = min(hp + hd - (MODE == 1 ? 1 : 0), mctx_i);
+                hm = nr < S ? min(hb, bB) : kBigKv;
+            };
+            derive();
+            int Gstop = (G | (kKvCal - 1)) + 1;  // the next re-file
+            Gstop = min(Gstop, c.max_iters);
+            if (la0 != 0) Gstop = min(Gstop, G + (a.kv.horizon - nrec));
+            long long r1 = 0, r2 = 0, r3 = 0, r4 = 0;  // features summed here
+            long long t3 = src + (long long)nd * G;    // F3 of batch G
             const int G0 = G;
-            while (l <= c.max_iters && (G == G0 || (G & (kKvCal - 1)) != 0)) {
+            auto record = [&](long long sl, int fa_, int bar_, int bl_) {
+                if (lane == 0) {
+                    KvRec R;
+                    R.cf[0] = cf1 + r1;
+                    R.cf[1] = cf2 + r2;
+                    R.cf[2] = cf3 + r3;
+                    R.cf[3] = cf4 + r4;
+                    R.slack = sl;
+                    R.far = fa_;
+                    R.thr = 0;  // requests wait: no query is admitted
+                    R.bar = bar_;
+                    R.bl = bl_;
+                    rec[nrec] = R;
+                    pmxo[nrec] = pmx;
+                }
+                ++nrec;
+            };
+            while (G < Gstop) {
                 const int need = hist[ridx];
                 int s = head[G & (kKvCal - 1)];
-                const long long fa = freeb - need;
-                if (fa < 0 || (nr < S && B > nd && need1 <= fa)) break;
-                freeb = fa;
-                r2 += nd;
-                r3 += src + (long long)nd * G;
-                if (s >= 0) {
-                    do {  // the decoders whose last batch this is return their blocks
+                int fa = fb - need;
+                if ((fa >= 0) & (fa < hm) & (s < 0)) {  // decoding only
+                    fb = fa;
+                    r2 += nd;
+                    r3 += t3;
+                    t3 += nd;
+                    if (la0 != 0) record(fa, fa, B - nd, B - nd);
+                    ++G;
+                    ridx = ridx == 0 ? bs - 1 : ridx - 1;
+                    continue;
+                }
+                slack = nr > 0 ? fa : kHuge;
+                if (fa < 0) {
+                    // preemption from the tail (see the general form)
+                    const int excess = -fa;
+                    int acc = 0;
+                    for (int top = tl - 1; top >= 0 && acc < excess; top -= 32) {
+                        const int s2 = top - lane;
+                        unsigned live = __ballot_sync(kFull, s2 >= 0 && reinterpret_cast<const int *>(rq + s2)[1] >= 0);
+                        while (live != 0u && acc < excess) {
+                            const int r = top - (__ffs(live) - 1);
+                            live &= live - 1u;
+                            const int4 q = rq[r];
+                            wh = wh == 0 ? C - 1 : wh - 1;
+                            hp = q.x + G;
+                            hd = q.z - G;
+                            acc += dblk(dv, hp + 1);
+                            src -= q.x;
+                            if (lane == 0) {
+                                hist[q.w] -= 1;
+                                wq[wh] = make_int2(hp, hd);
+                                reinterpret_cast<int *>(rq + r)[1] = -1;
+                            }
+                            ++wc;
+                            --nr;
+                            tl = r;
+                        }
+                    }
+                    nd = nr;
+                    fa = acc - excess;
+                    slack = -1;
+                    t3 = src + (long long)nd * G;
+                    derive();
+                    __syncwarp();
+                }
+                ndb = nd;
+                budget = B - nd;
+                const int bar_ = budget, far_ = fa;
+                f1 = f4 = 0;
+                if (fa >= hm) {
+                    do {
+                        const int x = min(hp, budget);
+                        if ((x == hp ? hb : dblk(dv, x)) > fa) break;
+                        if (x < hp || wc == 1 || hfin <= hp || ne == C) {
+                            scanned = true;  // the general form admits it
+                            break;
+                        }
+                        // whole: a decoder from the next batch on, ending in batch G + hfin - hp
+                        const int xs = hp - (G + 1), E = G + (hfin - hp);
+                        int res = hrem + ridx - 1;  // xs mod bs
+                        if (res < 0) res += bs;
+                        if (res >= bs) res -= bs;
+                        const int ebv = dblk(dv, hfin), slot = ne++;
+                        int32_t *h = hfin - hp < kKvCal ? &head[E & (kKvCal - 1)] : ovf;
+                        if (lane == 0) {
+                            rq[slot] = make_int4(xs, 0, hd - (MODE == 1 ? 1 : 0) + (G + 1), res);
+                            eb[slot] = ebv;
+                            nxt[slot] = *h;
+                            *h = slot;
+                            hist[res] += 1;
+                        }
+                        tl = ne;
+                        src += xs;
+                        ++nd;
+                        ++nr;
+                        fa -= hb;
+                        budget -= x;
+                        f1 += x;
+                        f4 += (long long)x * (x + 1) / 2;
+                        wh = wh + 1 == C ? 0 : wh + 1;
+                        --wc;
+                        const int2 hv = wq[wh];
+                        hp = hv.x;
+                        hd = hv.y;
+                        derive();
+                    } while (budget > 0 && nr < S);
+                }
+                if (scanned) {  // this batch goes on below
+                    fb = fa;
+                    s_end = s;
+                    f3 = t3;
+                    bar = bar_;
+                    far = far_;
+                    break;
+                }
+                fb = fa;
+                r1 += f1;
+                r2 += ndb;
+                r3 += t3;
+                r4 += f4;
+                if (la0 != 0) record(slack, far_, bar_, budget);
+                if (s >= 0) {  // the decoders whose last batch this is return their blocks
+                    do {
                         const int ns = nxt[s];
                         const int4 q = rq[s];
-                        if (q.y == 0) {
-                            freeb += eb[s];
+                        const int ebs = eb[s];
+                        if (q.y == 0) {  // a hole is a request preempted after it was filed
+                            fb += ebs;
                             src -= q.x;
                             --nd;
                             if (lane == 0) {
@@ -497,214 +674,174 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                     } while (s >= 0);
                     if (lane == 0) head[G & (kKvCal - 1)] = -1;
                     nr = nd;
-                    need1 = dblk(dv, min(hp, B - nd));
-                    __syncwarp();
                 }
+                hm = nr < S ? min(hb, bB) : kBigKv;
                 ++G;
-                ++l;
                 ridx = ridx == 0 ? bs - 1 : ridx - 1;
+                t3 = src + (long long)nd * G;
+                __syncwarp();
             }
-            if (G != G0) {
-                gr = ridx == 0 ? 0 : bs - ridx;
+            if (la0 != 0) {
+                cf1 += r1;
+                cf2 += r2;
+                cf3 += r3;
+                cf4 += r4;
+                if (G != G0) clear = 0;
+            } else {
                 fcum[0] += G - G0;
+                fcum[1] += r1;
                 fcum[2] += r2;
                 fcum[3] += r3;
-                if (l > c.max_iters || (G & (kKvCal - 1)) == 0) {  // the loop's head takes these
-                    --l;
-                    continue;
-                }
+                fcum[4] += r4;
+            }
+            gr = ridx == 0 ? 0 : bs - ridx;
+            freeb = fb;
+            l = G + 1;
+            if (!scanned) {
+                if (la0 != 0 && nrec == a.kv.horizon) break;
+                continue;
             }
         }
         // 1. The running scan.  n_run <= S <= B and only the last request may be in
         //    prefill, so every request gets its tokens if the blocks suffice: one per
         //    decoder, and the last one's chunk from what the decoders leave.
-        const int4 pq = pfs >= 0 ? rq[pfs] : make_int4(0, 0, 0, 0);
-        const int need_d = nd > 0 ? hist[gr == 0 ? 0 : bs - gr] : 0;  // decoders at a block boundary
-        int px = 0, pneed = 0;
-        if (pfs >= 0) {
-            px = min(pq.y, B - nd);
-            pneed = dblk(dv, pq.x + px) - pq.w;
-        }
-        const int need_all = need_d + pneed;
-        long long slack, f1, f2, f3, f4;
-        int budget;
-        bool pf_run = pfs >= 0;  // the prefill request still runs after the scan
-        int dying = 0;           // requests leaving after this batch
-        long long back = 0;      // and their blocks
-        if (need_all <= freeb) {
-            slack = nr > 0 ? freeb - need_all : kHuge;
-            freeb -= need_all;
-            budget = B - nd - px;
+        if (!scanned) {
+            int need_all = hist[ridx];  // decoders at a block boundary
+            s_end = head[G & (kKvCal - 1)];
+            int px = 0, pneed = 0;
+            if (pfs >= 0) {
+                px = min(pP, B - nd);
+                pneed = dblk(dv, pC + px) - pH;
+                need_all += pneed;
+            }
             f1 = px;
-            f2 = nd;
-            f3 = src + (long long)nd * G;
-            f4 = (long long)px * pq.x + (long long)px * (px + 1) / 2;
-        } else {
-            // a request runs out of blocks.  Preempting the tail until each request, in
-            // order, has its blocks leaves the longest prefix of the list whose blocks
-            // after the batch fit in the instance (what the rest held is what was free
-            // to them): those run, the rest go, in order, to the front of the waiting
-            // queue.  The prefill request, last, goes first, so the survivors are
-            // decoders.
-            // Every request's blocks after the batch sum to what is held plus what the
-            // batch needs, so requests leave from the tail until their post-batch blocks
-            // reach the excess over nb_j: usually one or two, taken one by one (every lane
-            // on the same values; a scan over 32 slots and a second pass to move them cost
-            // three times as much).
-            const int excess = need_all - (int)freeb;  // need_all > freeb >= 0
-            long long acc = 0;                         // post-batch blocks of those gone
-            for (int top = tl - 1; top >= 0 && acc < excess; top -= 32) {
-                const int s = top - lane;
-                unsigned live = __ballot_sync(kFull, s >= 0 && reinterpret_cast<const int *>(rq + s)[1] >= 0);
-                while (live != 0u && acc < excess) {
-                    const int l0 = __ffs(live) - 1;
-                    live &= live - 1u;
-                    const int r = top - l0;
-                    const int4 q = rq[r];
-                    wh = wh == 0 ? C - 1 : wh - 1;
-                    if (q.y == 0) {
-                        acc += dblk(dv, q.x + G + 1);
-                        src -= q.x;
-                        --nd;
-                        if (lane == 0) {
-                            wq[wh] = make_int2(q.x + G, q.z - G);
-                            hist[q.w] -= 1;
-                        }
-                    } else {
-                        acc += dblk(dv, q.x + px);
-                        if (lane == 0) wq[wh] = make_int2(q.x + q.y, q.z);
-                    }
-                    if (lane == 0) reinterpret_cast<int *>(rq + r)[1] = -1;
-                    ++wc;
-                    --nr;
-                    tl = r;
-                }
-            }
-            pfs = -1;
-            freeb = acc - excess;
-            budget = B - nr;
-            f1 = 0;
-            f2 = nd;
-            f3 = src + (long long)nd * G;
-            f4 = 0;
-            slack = -1;
-            pf_run = false;
-        }
-        __syncwarp();
-        if (pf_run) {
-            // the prefill request's chunk; at its last chunk it turns decoder
-            const int r = pfs;
-            const int cx = pq.x + px, pre = pq.y - px;
-            int dec = pq.z;
-            if (pre == 0 && MODE == 1) dec -= 1;
-            if (pre > 0) {
-                if (lane == 0) rq[r] = make_int4(cx, pre, dec, pq.w + pneed);
-            } else if (dec <= 0 || (long long)cx >= mctx) {
-                if (lane == 0) reinterpret_cast<int *>(rq + r)[1] = -1;
-                back += pq.w + pneed;
-                ++dying;
-                pfs = -1;
+            f4 = (long long)px * pC + (long long)px * (px + 1) / 2;
+            if (need_all <= freeb) {
+                freeb -= need_all;
+                slack = nr > 0 ? freeb : kHuge;
+                budget = B - nd - px;
             } else {
-                const int4 q = make_int4(cx - (G + 1), 0, dec + (G + 1), dres(dv, cx - (G + 1)));
-                if (lane == 0) {
-                    rq[r] = q;
-                    hist[q.w] += 1;
-                    file(r, q, G);
-                }
-                src += q.x;
-                ++nd;
-                pfs = -1;
-            }
-        }
-        __syncwarp();
-        const int bar = budget;
-        const long long far = freeb;
-        long long f4l = 0;      // this lane's whole admissions' F4 terms
-        bool admitted = false;  // any whole admission this batch
-        // 2. Admission from the waiting front while budget, a seat and the first chunk's
-        //    blocks allow: the prompts that fit whole are a prefix (lane i tests the
-        //    i-th waiting request), then possibly one partial chunk.  An admitted
-        //    request's chunk is applied at once; one that prefills whole decodes from
-        //    the next batch.
-        // FCFS: a head whose first chunk's blocks are not free admits nobody (the
-        // usual case while a queue waits on a full cache)
-        bool adm = budget > 0 && wc > 0 && nr < S;
-        if (adm) adm = dblk(dv, min(wq[wh].x, budget)) <= freeb;
-        while (adm && budget > 0 && wc > 0 && nr < S) {
-            if (ne + 32 > C) compact();
-            const bool in = lane < wc && lane < S - nr;
-            int slot = wh + lane;
-            if (slot >= C) slot -= C;
-            const int2 wv = in ? wq[slot] : make_int2(0, 0);
-            const int hb_i = in ? dblk(dv, wv.x) : 0;
-            const int cp = warp_incl_sum32(wv.x, lane);  // 32 prompts of at most 2^24 tokens
-            const int cb = warp_incl_sum32(hb_i, lane);
-            const bool whole = in && cp <= budget && (long long)cb <= freeb;
-            const int k = __popc(__ballot_sync(kFull, whole));
-            const int dec_a = wv.y - (MODE == 1 ? 1 : 0);
-            const bool ends = whole && (dec_a <= 0 || (long long)wv.x >= mctx);
-            if (whole) {
-                const int s = ne + lane;
-                const int4 q = make_int4(wv.x - (G + 1), ends ? -1 : 0, dec_a + (G + 1), dres(dv, wv.x - (G + 1)));
-                rq[s] = q;
-                if (!ends) {
-                    atomicAdd(&hist[q.w], 1);
-                    file(s, q, G);
-                }
-                f4l += (long long)wv.x * (wv.x + 1) / 2;
-            }
-            const unsigned em = __ballot_sync(kFull, ends);
-            if (k > 0) {
-                const int sp = __shfl_sync(kFull, cp, k - 1), sb = __shfl_sync(kFull, cb, k - 1);
-                f1 += sp;
-                admitted = true;
-                src += sp - (long long)k * (G + 1);
-                nd += k;
-                if (em) {
-                    src -= warp_sum64(ends ? (long long)wv.x - (G + 1) : 0);
-                    back += warp_sum64(ends ? (long long)hb_i : 0);
-                    dying += __popc(em);
-                    nd -= __popc(em);
-                }
-                budget -= sp;
-                freeb -= sb;
-                nr += k;
-                ne += k;
-                tl = ne;
-                wh = wh + k >= C ? wh + k - C : wh + k;
-                wc -= k;
-            }
-            __syncwarp();
-            if (k < 32) {
-                if (budget > 0 && wc > 0 && nr < S) {
-                    const int2 hv = wq[wh];
-                    const int x = min(hv.x, budget);
-                    const int nb1 = dblk(dv, x);
-                    if (x < hv.x && nb1 <= freeb) {
-                        if (lane == 0) rq[ne] = make_int4(x, hv.x - x, hv.y, nb1);
-                        pfs = ne;
-                        f1 += x;
-                        f4 += (long long)x * (x + 1) / 2;
-                        ++nr;
-                        tl = ++ne;
-                        wh = wh + 1 >= C ? wh + 1 - C : wh + 1;
-                        --wc;
-                        budget -= x;
-                        freeb -= nb1;
+                // a request runs out of blocks.  Preempting the tail until each request, in
+                // order, has its blocks leaves the longest prefix of the list whose blocks
+                // after the batch fit in the instance (what the rest held is what was free
+                // to them): those run, the rest go, in order, to the front of the waiting
+                // queue.  The prefill request, last, goes first, so the survivors are
+                // decoders.  Every request's blocks after the batch sum to what is held plus
+                // what the batch needs, so requests leave from the tail until their post-batch
+                // blocks reach the excess over nb_j, usually one or two.
+                const int excess = need_all - (int)freeb;  // need_all > freeb >= 0
+                long long acc = 0;                         // post-batch blocks of those gone
+                for (int top = tl - 1; top >= 0 && acc < excess; top -= 32) {
+                    const int s = top - lane;
+                    unsigned live = __ballot_sync(kFull, s >= 0 && reinterpret_cast<const int *>(rq + s)[1] >= 0);
+                    while (live != 0u && acc < excess) {
+                        const int r = top - (__ffs(live) - 1);
+                        live &= live - 1u;
+                        wh = wh == 0 ? C - 1 : wh - 1;
+                        if (r != pfs) {
+                            const int4 q = rq[r];
+                            acc += dblk(dv, q.x + G + 1);
+                            src -= q.x;
+                            --nd;
+                            hp = q.x + G;
+                            hd = q.z - G;
+                            if (lane == 0) hist[q.w] -= 1;
+                        } else {
+                            acc += dblk(dv, pC + px);
+                            hp = pC + pP;
+                            hd = pD;
+                            pfs = -1;
+                        }
+                        if (lane == 0) {
+                            wq[wh] = make_int2(hp, hd);
+                            reinterpret_cast<int *>(rq + r)[1] = -1;
+                        }
+                        ++wc;
+                        --nr;
+                        tl = r;
                     }
                 }
+                freeb = acc - excess;
+                budget = B - nr;
+                f1 = f4 = 0;
+                slack = -1;
+                __syncwarp();
+            }
+            ndb = nd;
+            f3 = src + (long long)nd * G;
+            if (pfs >= 0) {
+                // the prefill request's chunk; at its last chunk it turns decoder
+                pC += px;
+                pP -= px;
+                pH += pneed;
+                if (pP == 0) {
+                    const int dec = pD - (MODE == 1 ? 1 : 0);
+                    if (dec <= 0 || (long long)pC >= mctx) {
+                        if (lane == 0) reinterpret_cast<int *>(rq + pfs)[1] = -1;
+                        back += pH;
+                        ++dying;
+                    } else {
+                        decode_from_next(pfs, pC, dres(dv, pC), dec);
+                    }
+                    pfs = -1;
+                }
+            }
+            bar = budget;
+            far = freeb;
+        }
+        // slots for every request this batch could admit, those it preempted among them
+        // (residents never outnumber the slots)
+        if (ne + min(wc, S - nr) > C) {
+            __syncwarp();
+            compact();
+            s_end = head[G & (kKvCal - 1)];
+        }
+        // 2. Admission from the waiting front while budget, a seat and the first chunk's
+        //    blocks allow; one that prefills whole decodes from the next batch.
+        while (budget > 0 && wc > 0 && nr < S) {
+            const int x = min(hp, budget);
+            const int qt = (int)udiv32(dv, (unsigned)x), rem = x - qt * bs;
+            const int nb1 = qt + (rem > 0 ? 1 : 0);
+            if (nb1 > freeb) break;
+            const int left = hp - x, dec = hd;
+            budget -= x;
+            freeb -= nb1;
+            f1 += x;
+            f4 += (long long)x * (x + 1) / 2;
+            ++nr;
+            const int s = ne++;
+            tl = ne;
+            wh = wh + 1 == C ? 0 : wh + 1;
+            if (--wc > 0) {
+                const int2 h = wq[wh];
+                hp = h.x;
+                hd = h.y;
+            }
+            if (left > 0) {
+                pfs = s;
+                pC = x;
+                pP = left;
+                pD = dec;
+                pH = nb1;
+                if (lane == 0) rq[s] = make_int4(0, 1, 0, 0);
                 break;
             }
+            const int dec_a = dec - (MODE == 1 ? 1 : 0);
+            if (dec_a <= 0 || (long long)x >= mctx) {
+                if (lane == 0) reinterpret_cast<int *>(rq + s)[1] = -1;
+                back += nb1;
+                ++dying;
+            } else {
+                decode_from_next(s, x, rem, dec_a);
+            }
         }
-        __syncwarp();
         const bool qcan = wc == 0;
         if (la0 == 0 && qcan && budget > 0 && nr < S) la0 = l;
         // 3. The batch's record, or the features before the first record.
         bool rstop = false;
-        if (la0 != 0 && admitted) f4 += warp_sum64(f4l);
         if (la0 != 0) {
             cf1 += f1;
-            cf2 += f2;
+            cf2 += ndb;
             cf3 += f3;
             cf4 += f4;
             // the largest prompt p admitted now: min(p, bl) tokens need at most fa blocks
@@ -735,36 +872,34 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         } else {
             fcum[0] += 1;
             fcum[1] += f1;
-            fcum[2] += f2;
+            fcum[2] += ndb;
             fcum[3] += f3;
             fcum[4] += f4;
-            f4c += f4l;  // summed over the warp at the end
         }
         // 4. The decoders whose last batch this is leave and return their blocks.
-        {
-            int s = head[G & (kKvCal - 1)];
-            while (s >= 0) {
-                const int ns = nxt[s];
-                const int4 q = rq[s];
+        if (s_end >= 0) {
+            do {
+                const int ns = nxt[s_end];
+                const int4 q = rq[s_end];
                 if (q.y == 0) {  // a hole is a request preempted after it was filed
-                    back += eb[s];
+                    back += eb[s_end];
                     ++dying;
                     src -= q.x;
                     --nd;
                     if (lane == 0) {
                         hist[q.w] -= 1;
-                        reinterpret_cast<int *>(rq + s)[1] = -1;
+                        reinterpret_cast<int *>(rq + s_end)[1] = -1;
                     }
                 }
-                s = ns;
-            }
-            __syncwarp();
+                s_end = ns;
+            } while (s_end >= 0);
             if (lane == 0) head[G & (kKvCal - 1)] = -1;
         }
         nr -= dying;
         freeb += back;
-        G = G + 1;
+        ++G;
         gr = gr + 1 == bs ? 0 : gr + 1;
+        ridx = ridx == 0 ? bs - 1 : ridx - 1;
         __syncwarp();
         if (nr == 0 && wc == 0) {  // no resident left: every later batch is empty
             if (la0 == 0) la0 = l + 1;
@@ -772,9 +907,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
             break;
         }
         if (nrec == a.kv.horizon || (rstop && stops(l))) break;
-        if (ne - nr >= max(32, nr)) compact();
     }
-    fcum[4] += warp_sum64(f4c);
     if (lane == 0) {
         KvInst hd;
         for (int k = 0; k < 5; ++k) hd.fcum[k] = fcum[k];
