@@ -54,12 +54,15 @@ struct DevConfig {
 // KV-limited simulation (App. F): one batch of an instance's residents alone, from
 // the first batch in which a query could be admitted (the waiting queue empty after
 // admissions, budget and a seat left).  64 bytes.
+// The walk's fields are clamped to 32 bits, which no comparison with a query's own blocks
+// or prompt (at most 2^20 + 1) can tell.
 struct __align__(16) KvRec {
-    long long cf[4];   // residents' features 1..4 summed from the first record through this one
-    long long slack;   // least (free blocks - blocks needed) over the running scan; < 0: a preemption
-    long long far;     // free blocks after the running scan
-    long long thr;     // a waiting query with prompt p is admitted in this batch iff p <= thr
-    int32_t bar, bl;   // budget left after the running scan, after admissions
+    long long cf[4];             // residents' features 1..4 summed from the first record through this one
+    int32_t slack;               // least (free blocks - blocks needed) over the running scan; < 0: a preemption
+    int32_t far;                 // free blocks after the running scan
+    int32_t thr;                 // a waiting query with prompt p is admitted in this batch iff p <= thr
+    int32_t bar, bl;             // budget left after the running scan, after admissions
+    int32_t pad[3];
 };
 // Per instance: the residents' features before the first record, and the records' extent.
 struct __align__(16) KvInst {

@@ -24,7 +24,8 @@
 // readmissions, to its first token.  A candidate depends only on the instance and
 // the prompt length, so each call first counting-sorts its queries by length
 // (k_kv_count, k_kv_scan, k_kv_scatter), walks once per distinct length, and
-// copies those rows to the other queries of the same length (k_kv_expand).
+// copies those rows to the other queries of the same length (k_kv_expand).  A call of few
+// queries walks each of them directly instead, in the one launch.
 #include "lr_internal.cuh"
 
 namespace lr {
@@ -34,6 +35,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr long long kHuge = 1LL << 62;
 constexpr int kBigKv = 0x7fffffff;
+__device__ __forceinline__ int clamp32(long long x) { return (int)min(x, (long long)kBigKv); }
 
 __device__ __forceinline__ long long kv_blocks(long long c, long long bs) { return (c + bs - 1) / bs; }
 // ceil(c / bs) for 0 <= c < 2^31 (32-bit division)
@@ -380,9 +382,9 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
             R.cf[1] = c2;
             R.cf[2] = c3;
             R.cf[3] = c4;
-            R.slack = fa;  // nrk > 0: the window never starts on an empty instance
-            R.far = fa;
-            R.thr = thr;
+            R.slack = clamp32(fa);  // nrk > 0: the window never starts on an empty instance
+            R.far = clamp32(fa);
+            R.thr = clamp32(thr);
             R.bar = bar;
             R.bl = bar;
             rec[nrec + k] = R;
@@ -542,7 +544,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                     R.cf[1] = cf2 + r2;
                     R.cf[2] = cf3 + r3;
                     R.cf[3] = cf4 + r4;
-                    R.slack = sl;
+                    R.slack = clamp32(sl);
                     R.far = fa_;
                     R.thr = 0;  // requests wait: no query is admitted
                     R.bar = bar_;
@@ -854,9 +856,9 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 R.cf[1] = cf2;
                 R.cf[2] = cf3;
                 R.cf[3] = cf4;
-                R.slack = slack;
-                R.far = far;
-                R.thr = thr;
+                R.slack = clamp32(slack);
+                R.far = clamp32(far);
+                R.thr = clamp32(thr);
                 R.bar = bar;
                 R.bl = budget;
                 rec[nrec] = R;
@@ -948,34 +950,35 @@ __global__ void __launch_bounds__(kKvWarps * 32) k_kv_load(const KvLoad a) {
 }
 
 constexpr float kNaN = __builtin_nanf("");
-constexpr int kEstGroup = 32;   // instances per CTA
 constexpr int kEstWarps = 8;    // warps per CTA
-// leading records of each instance staged in shared memory: on pool256, 99.3% of the
-// candidates reach their first token within 64 records (88% within 16)
-constexpr int kEstStage = 52;
-// the staged fields of the walk: slack, far, thr (8 bytes), bar, bl, admission maximum (4)
-constexpr size_t kEstStageBytes = (size_t)kEstGroup * kEstStage * (3 * 8 + 3 * 4);
-// and each warp's tile of 32 later records (slack, far, thr, bar, bl); three CTAs with
-// their views fit an SM
-constexpr size_t kEstTileBytes = 32 * (3 * 8 + 2 * 4);
-constexpr size_t kEstSmem = kEstStageBytes + kEstWarps * kEstTileBytes;
+// The two shapes of the estimate.  Sorted: 32 instances per CTA, whose leading records'
+// walk fields are staged in shared memory: on pool256, 99.3% of the candidates reach
+// their first token within 64 records (88% within 16).  Direct (few queries): an instance
+// per warp, so that the walks of a call spread over as many warps as it has (instance,
+// 32 queries) units.
+template <bool DIRECT>
+struct EstShape {
+    static constexpr int kGroup = DIRECT ? kEstWarps : 32;  // instances per CTA
+    static constexpr int kStage = DIRECT ? 128 : 78;        // leading records staged
+    // the staged fields of the walk: (slack, far, thr, bar), bl and the admission maximum
+    static constexpr size_t kStageBytes = (size_t)kGroup * kStage * (16 + 2 * 4);
+    // and each warp's tile of 32 later records; sorted, three CTAs with their views fit an SM
+    static constexpr size_t kTileBytes = 32 * (16 + 4);
+    static constexpr size_t kSmem = kStageBytes + kEstWarps * kTileBytes;
+};
 
 // The walk's fields of an instance's leading records, in shared memory.
 struct KvStage {
-    long long *slack, *far, *thr;
-    int32_t *bar, *bl, *pmx;
+    int4 *q;  // slack, far, thr, bar
+    int32_t *bl, *pmx;
 };
+template <typename SH>
 __device__ __forceinline__ KvStage kv_stage(unsigned char *smem, int g) {
+    constexpr int n = SH::kStage;
     KvStage st;
-    long long *b64 = reinterpret_cast<long long *>(smem) + (size_t)g * 3 * kEstStage;
-    st.slack = b64;
-    st.far = b64 + kEstStage;
-    st.thr = b64 + 2 * kEstStage;
-    int32_t *b32 = reinterpret_cast<int32_t *>(reinterpret_cast<long long *>(smem) + (size_t)kEstGroup * 3 * kEstStage) +
-                   (size_t)g * 3 * kEstStage;
-    st.bar = b32;
-    st.bl = b32 + kEstStage;
-    st.pmx = b32 + 2 * kEstStage;
+    st.q = reinterpret_cast<int4 *>(smem) + (size_t)g * n;
+    st.bl = reinterpret_cast<int32_t *>(reinterpret_cast<int4 *>(smem) + (size_t)SH::kGroup * n) + (size_t)g * 2 * n;
+    st.pmx = st.bl + n;
     return st;
 }
 
@@ -994,16 +997,14 @@ struct KvView {
 
 // A warp's tile of 32 consecutive records past the staged ones (the walk's fields).
 struct KvTile {
-    long long *slack, *far, *thr;
-    int32_t *bar, *bl;
+    int4 *q;
+    int32_t *bl;
 };
+template <typename SH>
 __device__ __forceinline__ KvTile kv_tile(unsigned char *smem, int w) {
     KvTile tl;
-    tl.slack = reinterpret_cast<long long *>(smem + kEstStageBytes + (size_t)w * kEstTileBytes);
-    tl.far = tl.slack + 32;
-    tl.thr = tl.far + 32;
-    tl.bar = reinterpret_cast<int32_t *>(tl.thr + 32);
-    tl.bl = tl.bar + 32;
+    tl.q = reinterpret_cast<int4 *>(smem + SH::kStageBytes + (size_t)w * SH::kTileBytes);
+    tl.bl = reinterpret_cast<int32_t *>(tl.q + 32);
     return tl;
 }
 
@@ -1021,64 +1022,45 @@ __device__ __forceinline__ int kv_lower_bound(const int32_t *a, int lo, int n, i
     return lo;
 }
 
-// A candidate's walk: whether it runs, its prefill left, its context, the blocks it
-// holds and its own Eq. 9 features so far.
+// A candidate's walk: whether it runs, its context and the blocks it holds.  Its own Eq. 9
+// features need no sum along the way: the chunks that build a context of c tokens from
+// nothing sum to c prefill tokens and c (c + 1) / 2 attention pairs whatever their sizes,
+// so only what preemptions discard is kept (lost1, lost4), the whole prompt is added at
+// the end, and its one decode token comes at context p.
 struct KvWalk {
     bool run;
-    int pre, ctx, held;
-    long long o1, o2, o3, o4;
+    int ctx, held;
+    long long lost1, lost4;
 };
 
-// One batch (record) of a candidate's walk; true if its first token falls in it.  A
-// running query is preempted if the residents' scan leaves a slack below its blocks,
+// One batch (record) of the walk of a query of p tokens; true if its first token falls in
+// it.  A running query is preempted if the residents' scan leaves a slack below its blocks,
 // or if its own tokens need more blocks than are free to it (it is the last running
-// request: it preempts itself); a preempted query recomputes its whole context and may
-// be readmitted in the same batch.  Token counts stay below p + 2 <= 2^31.
+// request: it preempts itself); a preempted query recomputes its whole context and may be
+// readmitted in the same batch.
 template <int MODE>
-__device__ __forceinline__ bool kv_step(KvWalk &w, const Div32 &dv, long long slack, long long far, long long thr,
-                                        int bar, int bl) {
-    if (w.run) {
-        if (slack < w.held) {  // a resident needs the query's blocks
-            w.pre += w.ctx;
-            w.ctx = 0;
-            w.held = 0;
-            w.run = false;
-        } else if (bar > 0) {
-            const int x = w.pre > 0 ? min(w.pre, bar) : 1;
-            const int nh = dblk(dv, w.ctx + x);
-            if (nh > far) {  // its own tokens do not fit: it preempts itself
-                w.pre += w.ctx;
-                w.ctx = 0;
-                w.held = 0;
-                w.run = false;
-            } else {
-                w.held = nh;
-                if (w.pre > 0) {
-                    w.o1 += x;
-                    w.o4 += (long long)x * w.ctx + (long long)x * (x + 1) / 2;
-                    w.ctx += x;
-                    w.pre -= x;
-                    return w.pre == 0 && MODE == 1;
-                }
-                w.o2 += 1;
-                w.o3 += w.ctx;
-                return true;
-            }
-        } else {
-            return false;  // no budget reached the query this batch
-        }
+__device__ __forceinline__ bool kv_step(KvWalk &w, const Div32 &dv, int p, const int4 &q, int bl) {
+    // Without branches: the lanes of a warp are in different states, a long walk (a query
+    // that is admitted, runs out of blocks and is admitted again, batch after batch) takes
+    // every case in every record, and the two block counts overlap.
+    const int slack = q.x, far = q.y, thr = q.z, bar = q.w;
+    const int rem = p - w.ctx;  // 0 only while it waits for its decode token
+    const int x = rem > 0 ? min(rem, bar) : 1;
+    const int y = min(p, bl);
+    const int nh = dblk(dv, w.ctx + x), hy = dblk(dv, y);
+    const bool stays = w.run & (slack >= w.held) & ((nh <= far) | (bar <= 0));
+    const bool goes = stays & (bar > 0);
+    const bool lost = w.run & !stays;
+    const bool adm = !stays & (p <= thr);
+    if (lost) {
+        w.lost1 += w.ctx;
+        w.lost4 += (long long)w.ctx * (w.ctx + 1) / 2;
     }
-    if (w.pre <= thr) {  // admission (pre == p while waiting)
-        const int x = min(w.pre, bl);
-        w.held = dblk(dv, x);
-        w.o1 += x;
-        w.o4 += (long long)x * (x + 1) / 2;
-        w.ctx = x;
-        w.pre -= x;
-        w.run = true;
-        return w.pre == 0 && MODE == 1;
-    }
-    return false;
+    const bool fin = goes & (MODE == 1 ? x == rem : rem == 0);
+    w.held = adm ? hy : goes ? nh : w.held;
+    w.ctx = adm ? y : goes ? w.ctx + x : w.ctx;
+    w.run = stays | adm;
+    return fin | (MODE == 1 && adm && y == p);
 }
 
 // The (query, instance) candidates of a warp's lanes (one instance, `live`: the lane
@@ -1093,7 +1075,7 @@ template <int MODE>
 __device__ int kv_candidate(const KvView &v, const KvStage &st, const KvTile &tl, int lane, bool live, int p,
                             long long F[5], int &lt) {
     int err = 0, t = 0;
-    KvWalk w = {false, p, 0, 0, 0, 0, 0, 0};
+    KvWalk w = {false, 0, 0, 0, 0};
     bool fin = !live;
     if (live) {
         int lo;
@@ -1104,7 +1086,7 @@ __device__ int kv_candidate(const KvView &v, const KvStage &st, const KvTile &tl
             fin = true;
         }
         for (t = lo; !fin && t < v.ns;) {
-            if (kv_step<MODE>(w, v.dv, st.slack[t], st.far[t], st.thr[t], st.bar[t], st.bl[t])) fin = true;
+            if (kv_step<MODE>(w, v.dv, p, st.q[t], st.bl[t])) fin = true;
             else ++t;
         }
     }
@@ -1116,20 +1098,13 @@ __device__ int kv_candidate(const KvView &v, const KvStage &st, const KvTile &tl
         const int base = __reduce_min_sync(kFull, fin ? 0x7fffffff : t);  // >= ns
         {
             const int r = base + lane;
-            long long sl = kHuge, fa = v.nb, th = kHuge;  // past the records: an empty batch
-            int ba = v.B, bb = v.B;
+            int4 q = make_int4(kBigKv, clamp32(v.nb), kBigKv, v.B);  // past the records: an empty batch
+            int bb = v.B;
             if (r < v.nrec) {
-                const KvRec *rr = v.rec + r;
-                sl = __ldg(&rr->slack);
-                fa = __ldg(&rr->far);
-                th = __ldg(&rr->thr);
-                ba = __ldg(&rr->bar);
-                bb = __ldg(&rr->bl);
+                q = __ldg(reinterpret_cast<const int4 *>(&v.rec[r].slack));
+                bb = __ldg(&v.rec[r].bl);
             }
-            tl.slack[lane] = sl;
-            tl.far[lane] = fa;
-            tl.thr[lane] = th;
-            tl.bar[lane] = ba;
+            tl.q[lane] = q;
             tl.bl[lane] = bb;
         }
         __syncwarp();
@@ -1140,7 +1115,7 @@ __device__ int kv_candidate(const KvView &v, const KvStage &st, const KvTile &tl
                 break;
             }
             const int k = t - base;
-            if (kv_step<MODE>(w, v.dv, tl.slack[k], tl.far[k], tl.thr[k], tl.bar[k], tl.bl[k])) fin = true;
+            if (kv_step<MODE>(w, v.dv, p, tl.q[k], tl.bl[k])) fin = true;
             else ++t;
         }
         __syncwarp();  // the tile is read before the next one is written
@@ -1154,10 +1129,10 @@ __device__ int kv_candidate(const KvView &v, const KvStage &st, const KvTile &tl
         for (int k = 0; k < 4; ++k) cf[k] = __ldg(&r->cf[k]);
     }
     F[0] = v.fcum[0] + t + 1;
-    F[1] = v.fcum[1] + cf[0] + w.o1;
-    F[2] = v.fcum[2] + cf[1] + w.o2;
-    F[3] = v.fcum[3] + cf[2] + w.o3;
-    F[4] = v.fcum[4] + cf[3] + w.o4;
+    F[1] = v.fcum[1] + cf[0] + w.lost1 + p;
+    F[2] = v.fcum[2] + cf[1] + (MODE == 0 ? 1 : 0);
+    F[3] = v.fcum[3] + cf[2] + (MODE == 0 ? p : 0);
+    F[4] = v.fcum[4] + cf[3] + w.lost4 + (long long)p * (p + 1) / 2;
     return 0;
 }
 
@@ -1320,12 +1295,15 @@ __global__ void __launch_bounds__(256) k_kv_expand(const KvEst a) {
     }
 }
 
-// CTA: kEstGroup instances (strided over the pool), the walk's fields of their
-// leading records staged in shared memory.  The CTAs of a group claim units of (32 queries, one instance),
-// the longest prompts first, so the longest walks start first and no warp holds
-// more than one instance's walks of one block.
-template <int MODE>
+// CTA: SH::kGroup instances (strided over the pool), the walk's fields of their leading
+// records staged in shared memory.  Sorted: the CTAs of a group claim units of (32
+// queries, one instance), the longest prompts first, so the longest walks start first and
+// no warp holds more than one instance's walks of one block.  Direct: warp w walks
+// instance w of the group, for the query blocks x, x + gridDim.x, ..., in the call's order.
+template <int MODE, bool DIRECT>
 __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a, bool exact) {
+    using SH = EstShape<DIRECT>;
+    constexpr int kEstGroup = SH::kGroup, kEstStage = SH::kStage;
     extern __shared__ __align__(16) unsigned char est_smem[];
     __shared__ KvView sv[kEstGroup];
     const DevConfig &c = a.cfg;
@@ -1369,18 +1347,15 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
         constexpr int kRound = 4;
         constexpr int kAll = kEstGroup * kEstStage;
         for (int r0 = 0; r0 < kAll; r0 += kRound * kEstWarps * 32) {
-            long long f_sl[kRound], f_fa[kRound], f_th[kRound];
-            int f_ba[kRound], f_bl[kRound], f_pm[kRound];
+            int4 f_q[kRound];
+            int f_bl[kRound], f_pm[kRound];
 #pragma unroll
             for (int k = 0; k < kRound; ++k) {
                 const int idx = r0 + (int)threadIdx.x + k * kEstWarps * 32;
                 const int gw = idx / kEstStage, t = idx - gw * kEstStage;
                 if (gw < ng && t < sv[gw].ns) {
                     const KvRec *r = sv[gw].rec + t;
-                    f_sl[k] = __ldg(&r->slack);
-                    f_fa[k] = __ldg(&r->far);
-                    f_th[k] = __ldg(&r->thr);
-                    f_ba[k] = __ldg(&r->bar);
+                    f_q[k] = __ldg(reinterpret_cast<const int4 *>(&r->slack));
                     f_bl[k] = __ldg(&r->bl);
                     f_pm[k] = __ldg(sv[gw].pmx + t);
                 }
@@ -1390,11 +1365,8 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
                 const int idx = r0 + (int)threadIdx.x + k * kEstWarps * 32;
                 const int gw = idx / kEstStage, t = idx - gw * kEstStage;
                 if (gw < ng && t < sv[gw].ns) {
-                    const KvStage st = kv_stage(est_smem, gw);
-                    st.slack[t] = f_sl[k];
-                    st.far[t] = f_fa[k];
-                    st.thr[t] = f_th[k];
-                    st.bar[t] = f_ba[k];
+                    const KvStage st = kv_stage<SH>(est_smem, gw);
+                    st.q[t] = f_q[k];
                     st.bl[t] = f_bl[k];
                     st.pmx[t] = f_pm[k];
                 }
@@ -1403,12 +1375,18 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
     }
     __syncthreads();
     // the work: one query per distinct prompt length, or every query, by length
-    const int nwork = exact ? *a.nu : a.Q;
+    const int nwork = DIRECT ? a.Q : exact ? *a.nu : a.Q;
     const int32_t *work = exact ? a.leaders : a.order;
-    const int nitems = (nwork + 31) / 32 * ng;
+    const int nitems = DIRECT ? (w < ng ? (nwork + 31) / 32 : 0) : (nwork + 31) / 32 * ng;
     // Software-pipelined: the claim of the next item and its query's prompt are in
     // flight while the current item is walked.
+    int own = blockIdx.x;  // direct: this warp's next query block
     auto claim = [&]() {
+        if (DIRECT) {
+            const int b = own;
+            own += gridDim.x;
+            return b;
+        }
         int v = 0;
         if (lane == 0) v = atomicAdd(&a.claim[blockIdx.y], 1);
         return __shfl_sync(kFull, v, 0);
@@ -1416,7 +1394,13 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
     auto fetch = [&](int it_, int &i_, int &p_) {  // this lane's query of item it_ (i_ < 0: none)
         i_ = -1;
         p_ = 0;
-        if (it_ < nitems) {
+        if (DIRECT && it_ < nitems) {
+            const int pos_ = it_ * 32 + lane;
+            if (pos_ < nwork) {
+                i_ = pos_;
+                p_ = a.prompt[pos_];
+            }
+        } else if (it_ < nitems) {
             const int pos_ = nwork - 1 - ((it_ / ng) * 32 + lane);
             if (pos_ >= 0) {
                 i_ = work[pos_];
@@ -1430,7 +1414,7 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
     for (;;) {
         if (it >= nitems) break;
         const int it_next = claim();
-        const int qb = it / ng, g = it - qb * ng;
+        const int g = DIRECT ? w : it - it / ng * ng;
         const int i = i_cur, p = p_cur;
         int i_nx, p_nx;
         fetch(it_next, i_nx, p_nx);
@@ -1446,7 +1430,7 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
             else if (!(p >= 1 && p <= c.pmax && (long long)p < v.mctx && kv_blocks32(p + 1, v.bs) <= v.nb))
                 err = kEInval;
         }
-        const int werr = kv_candidate<MODE>(v, kv_stage(est_smem, g), kv_tile(est_smem, w), lane,
+        const int werr = kv_candidate<MODE>(v, kv_stage<SH>(est_smem, g), kv_tile<SH>(est_smem, w), lane,
                                             i >= 0 && err == 0, p, F, lt);
         if (err == 0) err = werr;
         if (i >= 0) {
@@ -1484,15 +1468,33 @@ cudaError_t launch_kv_load(const KvLoad &a, int grid, int warps, size_t smem, cu
 cudaError_t set_kv_smem(size_t bytes) {
     cudaError_t e = cudaFuncSetAttribute(k_kv_load<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_kv_load<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_kv_estimate<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEstSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_kv_estimate<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEstSmem);
+    auto est = [&](auto f, size_t n) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+    };
+    est(k_kv_estimate<0, false>, EstShape<false>::kSmem);
+    est(k_kv_estimate<1, false>, EstShape<false>::kSmem);
+    est(k_kv_estimate<0, true>, EstShape<true>::kSmem);
+    est(k_kv_estimate<1, true>, EstShape<true>::kSmem);
     return e;
 }
 
 cudaError_t launch_kv_estimate(const KvEst &a, int sms, cudaStream_t st) {
-    const int gy = (a.cfg.I + kEstGroup - 1) / kEstGroup;
+    constexpr int thr = kEstWarps * 32;
+    // Few queries are walked directly, in one launch.  The sort by prompt length, the walks
+    // of distinct lengths alone and the copies of their rows pay for their five further
+    // launches once a warp would take several units: while the units make one wave (three
+    // CTAs an SM), or up to 1,024 queries at four units a warp, direct is faster.  Event-timed
+    // calls, direct / sorted: 24 instances x 4,096 queries 31 / 58 us, 8,192 54 / 52; 64 x
+    // 1,024 49 / 87, 2,048 88 / 83; 256 x 1,024 31 / 86, 4,096 95 / 68; 64 x 16 13 / 39.
+    const int gd = (a.cfg.I + EstShape<true>::kGroup - 1) / EstShape<true>::kGroup;
+    const int qb = (a.Q + 31) / 32, wave = std::max(1, sms * 3 / gd);
+    if (qb <= std::max(wave, std::min(32, 4 * wave))) {
+        const dim3 grid(std::min(qb, wave), gd);
+        if (a.cfg.mode == 0) k_kv_estimate<0, true><<<grid, thr, EstShape<true>::kSmem, st>>>(a, false);
+        else k_kv_estimate<1, true><<<grid, thr, EstShape<true>::kSmem, st>>>(a, false);
+        return cudaGetLastError();
+    }
+    const int gy = (a.cfg.I + EstShape<false>::kGroup - 1) / EstShape<false>::kGroup;
     const int blocks = (a.Q + 32 * kEstWarps - 1) / (32 * kEstWarps);
     const int gx = std::max(1, std::min(blocks, (sms * 3 + gy - 1) / gy));  // three CTAs fit an SM
     const dim3 grid(gx, gy);
@@ -1506,8 +1508,8 @@ cudaError_t launch_kv_estimate(const KvEst &a, int sms, cudaStream_t st) {
     k_kv_tile_sums<<<tiles, kScanThreads, 0, st>>>(a.cnt, a.tsum, a.claim, gy);
     k_kv_scan<<<tiles, kScanThreads, 0, st>>>(a.cnt, a.start, a.run, a.uid, a.nu, a.tsum);
     k_kv_scatter<<<g1, 256, 0, st>>>(a.prompt, a.Q, a.cfg.pmax, shift, a.run, a.start, a.uid, a.order, a.leaders);
-    if (a.cfg.mode == 0) k_kv_estimate<0><<<grid, kEstWarps * 32, kEstSmem, st>>>(a, exact);
-    else k_kv_estimate<1><<<grid, kEstWarps * 32, kEstSmem, st>>>(a, exact);
+    if (a.cfg.mode == 0) k_kv_estimate<0, false><<<grid, thr, EstShape<false>::kSmem, st>>>(a, exact);
+    else k_kv_estimate<1, false><<<grid, thr, EstShape<false>::kSmem, st>>>(a, exact);
     if (exact) k_kv_expand<<<std::max(1, std::min((a.Q + 7) / 8, sms * 8)), 256, 0, st>>>(a);
     return cudaGetLastError();
 }

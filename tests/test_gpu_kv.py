@@ -231,6 +231,21 @@ def test_long_blocked_queues(mode, bs):
     check(wl, limits)
 
 
+@pytest.mark.parametrize("I,few", [(3, 31), (9, 33), (24, 1000)])
+def test_few_and_many_queries_agree(I, few):
+    # a call of few queries walks each one directly; 20,000 queries are sorted by length and
+    # walked once a length.  Rows agree bit for bit, invalid lengths included.
+    wl = W.small_workload(90 + I, num_instances=I, num_models=2, num_queries=20_000, budget_range=(8, 48), min_gap=8)
+    wl.prompt_len[:3] = (0, 161, 160)
+    limits = W.kv_limits(wl, 13, block_sizes=(2, 8), tightness=(0.0, 0.3))
+    rt = make(wl, limits)
+    many = gpu_estimate(rt, wl)
+    part = gpu_estimate(rt, wl.with_queries(np.arange(few)))
+    rt.close()
+    for a, b in zip(many, part):
+        np.testing.assert_array_equal(a[:few].view(np.uint8), b.view(np.uint8))
+
+
 def test_invalid_snapshot_keeps_the_live_one():
     wl = W.small_workload(63, num_instances=9, num_models=2, num_queries=20, budget_range=(8, 96), min_gap=8)
     bs, nb, mc = W.kv_limits(wl, 9, block_sizes=(4,))
