@@ -1,5 +1,6 @@
 // Host side of the C ABI declared in include/latency_router.h: validation,
 // device memory, launch shapes and the status word.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -60,13 +61,13 @@ struct lr_ctx {
     int max_queries = 0, max_pairs = 0;
     // K1
     size_t k1_smem = 0;
-    // candidate kernel shapes: estimate (instances may span several tiles) and
-    // route (all instances of a row in one CTA)
+    // candidate kernel shapes: estimate (instances may span several tiles), route (all
+    // instances of a row in one CTA) and sweep (several pairs)
     struct Shape {
         int Gp = 0, QS = 0, QT = 0, tiles = 1, occ = 1, block = 0;
         size_t smem = 0;
         bool ok = false;
-    } est, rt;
+    } est, rt, sw;
 };
 
 namespace {
@@ -160,9 +161,9 @@ int pow2_ceil(int x) {
 // Gp groups per row (power of two up to 32, else a multiple of 32); the
 // summary tables of the tile and QT staged query rows fit the shared-memory
 // target.  Routing runs three 256-thread CTAs per SM (one of them fits beside a
-// snapshot load's CTA); the estimate alone runs one 768-thread CTA per SM, so
+// snapshot load's CTA); the estimate alone runs one 512-thread CTA per SM, so
 // that each SM copies its tile block once.
-lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, int max_pairs) {
+lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep) {
     lr_ctx::Shape s;
     s.block = route ? lr::kK2Block : lr::kK2EstBlock;
     const int G = (d.I + 3) / 4;
@@ -177,19 +178,22 @@ lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, int max_pairs) {
     // the tile block (tables and per-instance scalars), brought in by one bulk copy
     lr::DevConfig dt = d;
     dt.tgp = s.Gp;
-    const size_t tables = lr::tile_bytes(dt);
-    const size_t part = s.Gp > 32 ? 2 * (size_t)wpr * 16 * max_pairs : 0;  // wide-row partials per pair
-    // staged row (16 B) and two raw copies of its prompt; routing adds the wide-row
-    // partials, (cost, acc) per model, tau, and two raw copies of tau, dec_hat and acc
-    const size_t per_row = 16 + 8 + (route ? part + (size_t)d.M * 8 + 4 + 8 + (size_t)d.M * 16 : 0);
+    // (and the buffers in which a warp orders the stores of rows that are not whole 16-byte words)
+    const size_t tables = lr::tile_bytes(dt) + (d.I % 4 ? (size_t)s.block * 32 : 0);
+    // wide-row partials; a sweep keeps the row's times, and once the models and the pairs
+    const size_t part = sweep ? 16 * (size_t)s.Gp : s.Gp > 32 ? 2 * (size_t)wpr * 16 : 0;
+    const size_t fixed = tables + (sweep ? 20 * (size_t)s.Gp + 4 + 8 * lr::kMaxPairs : 0);
+    // staged row (32 B) and two raw copies of its prompt; routing adds the wide-row partials,
+    // (cost, acc) per model, tau, and two raw copies of tau, dec_hat and acc
+    const size_t per_row = 32 + 8 + (route ? part + (size_t)d.M * 8 + 4 + 8 + (size_t)d.M * 16 : 0);
     const size_t target = route ? lr::kK2SmemTarget : lr::kK2EstSmemTarget;
-    const size_t room = target > tables ? target - tables : 0;
+    const size_t room = target > fixed ? target - fixed : 0;
     int qt = (int)std::min<size_t>(route ? 256 : 1024, room / per_row);
-    if (route && (size_t)qt * per_row + tables > 200 * 1024) qt = 0;
+    if (route && (size_t)qt * per_row + fixed > 200 * 1024) qt = 0;
     qt = std::max(s.QS, (qt / s.QS) * s.QS);
     s.QT = qt;
-    s.smem = tables + (size_t)qt * per_row;
-    s.ok = s.smem <= 200 * 1024;
+    s.smem = fixed + (size_t)qt * per_row;
+    s.ok = s.smem <= 224 * 1024;
     return s;
 }
 
@@ -260,7 +264,7 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
             return bail(LR_EINVAL, "prices must be finite and >= 0");
     }
     std::vector<int32_t> shift(I), nb(I);
-    int kph = 1, nbh = 1;
+    int kph = 1, nbh = 1, near = 1 << 30;
     for (int j = 0; j < I; ++j) {
         const int B = cfg->max_batched_tokens[j], S = cfg->max_seqs[j], m = cfg->model_of_instance[j];
         if (m < 0 || m >= M) return bail(LR_EINVAL, "model_of_instance out of range");
@@ -272,6 +276,8 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
         if (kp > lr::kKMax || nb[j] > lr::kNBMax)
             return bail(LR_ECAPACITY, "max_prompt_len too large for max_batched_tokens - max_seqs + 1 of instance " +
                                           std::to_string(j));
+        // R_0 >= 1 and r_1 >= gap: at most one budget boundary lies below such a prompt
+        near = (int)std::min<long long>(near, gap + 1);
         kph = std::max(kph, (int)kp);
         nbh = std::max(nbh, nb[j]);
         c->max_seqs = std::max(c->max_seqs, S);
@@ -298,6 +304,7 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     d.max_iters = cfg->max_iters;
     d.kph = kph;
     d.nbh = nbh;
+    d.near = near;
     {
         // thread groups per instance tile of the candidate kernel (as make_shape chooses)
         const int G = (I + 3) / 4;
@@ -389,14 +396,15 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     // K1: one warp per instance.
     c->k1_smem = lr::kK1Warps * lr::trajectory_smem_per_warp(d);
     if (c->k1_smem > 200 * 1024) return bail(LR_ECAPACITY, "snapshot capacities too large for one K1 warp");
-    c->est = make_shape(d, false, 1);
-    c->rt = make_shape(d, true, cfg->max_pairs);
+    c->est = make_shape(d, false, false);
+    c->rt = make_shape(d, true, false);
+    c->sw = make_shape(d, true, true);
     if (!c->est.ok) return bail(LR_ECAPACITY, "summary tables too large for shared memory");
     c->k3_smem = lr::kK3Warps * lr::advance_smem_per_warp(d);
     e = lr::set_k1_smem(c->k1_smem);
     if (e == cudaSuccess && c->k3_smem <= 200 * 1024) e = lr::set_k3_smem(c->k3_smem);
     if (e == cudaSuccess && M <= lr::kCalMaxModels) e = lr::set_calib_smem(M);
-    if (e == cudaSuccess) e = lr::set_k2_smem(std::max(c->est.smem, c->rt.ok ? c->rt.smem : 0));
+    if (e == cudaSuccess) e = lr::set_k2_smem(std::max({c->est.smem, c->rt.ok ? c->rt.smem : 0, c->sw.ok ? c->sw.smem : 0}));
     c->bl_ok = lr::baseline_smem(d) <= 200 * 1024;
     if (e == cudaSuccess && c->bl_ok) e = lr::set_baseline_smem(lr::baseline_smem(d));
     if (e == cudaSuccess) e = lr::cand_occupancy(d.mode, false, c->est.block, c->est.smem, &c->est.occ);
@@ -404,6 +412,9 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     if (e != cudaSuccess) return bail(LR_ECUDA, cudaGetErrorString(e));
     c->est.occ = std::max(1, c->est.occ);
     c->rt.occ = std::max(1, c->rt.occ);
+    if (c->sw.ok) e = lr::cand_occupancy(d.mode, true, c->sw.block, c->sw.smem, &c->sw.occ);
+    if (e != cudaSuccess) return bail(LR_ECUDA, cudaGetErrorString(e));
+    c->sw.occ = std::max(1, c->sw.occ);
     *out = c;
     return LR_OK;
 }
@@ -571,14 +582,17 @@ int lr_route(lr_ctx *c, int32_t Q, const int32_t *prompt_len, const int32_t *dec
         a.src = lr::kSrcMatrix;
         a.ttft_in = kv_matrix;
     }
-    a.Gp = c->rt.Gp;
-    a.QS = c->rt.QS;
-    a.QT = c->rt.QT;
-    a.vec_ok = (c->cfg.I % 4 == 0) && ((uintptr_t)a.ttft % 16 == 0);
-    dim3 grid(std::min(c->sms * c->rt.occ, (Q + a.QS - 1) / a.QS), 1);
-    set_row_split(a, c, (int)grid.x, 1, c->rt.occ, stream);
+    const lr_ctx::Shape &sh = P > 1 ? c->sw : c->rt;
+    if (!sh.ok) return fail(c, LR_ECAPACITY, "routing needs num_instances <= 1024 and its tiles in shared memory");
+    a.Gp = sh.Gp;
+    a.QS = sh.QS;
+    a.QT = sh.QT;
+    a.pg = std::min(32, pow2_ceil(P));
+    a.vec_ok = (c->cfg.I % 4 == 0) && ((uintptr_t)(kv_matrix ? kv_matrix : a.ttft) % 16 == 0);
+    dim3 grid(std::min(c->sms * sh.occ, (Q + a.QS - 1) / a.QS), 1);
+    set_row_split(a, c, (int)grid.x, 1, sh.occ, stream);
     cudaError_t e = lr::launch_cand(a, lr::cand_out_flags(a.ttft != nullptr, false, true, tau != nullptr, P), grid,
-                                    c->rt.block, c->rt.smem, (cudaStream_t)stream);
+                                    sh.block, sh.smem, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "route launch");
     if (frontier_out) {
         e = lr::launch_frontier(a, frontier_out, (cudaStream_t)stream);

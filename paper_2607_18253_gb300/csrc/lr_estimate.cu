@@ -20,10 +20,23 @@
 // and the outer add rounds the exact total once.  This keeps the hot loop on
 // the FMA pipe; instances whose totals reach 2^44 take an int64 path.
 //
+// The kernel is bound by the instructions issued per candidate (and, below some tens of
+// microseconds, by its start-up: tile block, live index, first rows), so:
+//   * the fp32 work of two instances goes in one packed instruction;
+//   * a prompt of at most near = min_j(B_j - S_j + 1) + 1 tokens has at most one budget
+//     boundary below it on every instance, so k* is p > R_0 and the two candidate entries
+//     stay in registers: no bucket and no table read (98% of pool256's queries);
+//   * a row of several warps describes its winner once, after the chunk.
+// Warp instructions for 65,536 x 256 candidates, kernel time: estimate 11.9 M, 16.0 us ->
+// 8.3 M, 15.0 us; route 20.2 M, 27.0 -> 15.1 M, 23.0 us; with the matrix 27.6 -> 24.5 us.
+//
 // The estimate matrix is write-only (4 bytes per candidate) and leaves as one
-// 16-byte evict-first store per thread and row.  Routing reduces each row with
-// redux.sync over order-preserving integer keys of the objective: the lowest
-// lane (lowest instance) among the maximal keys wins, as in a first-max scan.
+// 16-byte evict-first store per thread and row.  Where rows are not whole 16-byte words
+// (I % 4 != 0) each warp puts its 128 elements of a row in order in shared memory first:
+// 4-byte stores 16 bytes apart wrote every sector in pieces (50,001 x 250: 26.6 -> 15.6 us).
+// Routing reduces each row with redux.sync over the objective (the value itself, or an
+// order-preserving integer key): the lowest lane (lowest instance) among the maximal wins,
+// as in a first-max scan.
 #include <math.h>
 
 #include "lr_internal.cuh"
@@ -36,11 +49,13 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr long long kLowMask = (1LL << kSplitBits) - 1;
 constexpr float kNaN = __builtin_nanf("");
 
+// A staged query row: the fp32 values twice each, as the packed instructions take them.
 struct __align__(16) QRec {
-    int p;     // prompt length, clamped into [1, pmax] for table lookups
-    float fp;  // p as fp32, NaN if p was out of range
-    float ph;  // p(p+1)/2 high part (multiple of 2^20)
-    float pl;  // p(p+1)/2 low part
+    float fp[2];  // p as fp32, NaN if p was out of range
+    float ph[2];  // p(p+1)/2 high part (multiple of 2^20)
+    float pl[2];  // p(p+1)/2 low part
+    int p;        // prompt length, clamped into [1, pmax] for table lookups
+    int pad;
 };
 
 __device__ __forceinline__ QRec make_qrec(int p, int pmax, bool *ok) {
@@ -50,9 +65,10 @@ __device__ __forceinline__ QRec make_qrec(int p, int pmax, bool *ok) {
     const long long pp = ((long long)p * (p + 1)) / 2;
     const long long pl = pp & kLowMask;
     q.p = p;
-    q.fp = *ok ? (float)p : kNaN;
-    q.ph = __ll2float_rn(pp - pl);
-    q.pl = __ll2float_rn(pl);
+    q.fp[0] = q.fp[1] = *ok ? (float)p : kNaN;
+    q.ph[0] = q.ph[1] = __ll2float_rn(pp - pl);
+    q.pl[0] = q.pl[1] = __ll2float_rn(pl);
+    q.pad = 0;
     return q;
 }
 
@@ -104,28 +120,49 @@ enum : int {
     kOutSweep = 16    // Lagrangian argmax for several pairs
 };
 
+// Two fp32 values in one 64-bit register pair: the packed fp32 instructions do the two
+// IEEE operations of a pair in one issue slot, each rounded as the scalar instruction.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+    f32x2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    return v;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 v;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+
+// A thread's four instances as two pairs.  Of a compact instance h1 holds the whole F1tot
+// (exact in fp32, and so is F1tot + p) and l1 is unused.
 struct Inst4 {
-    int shift[4];
-    float h1[4], l1[4], h4[4], l4[4], b1p[4], b2[4], b3[4];
+    f32x2 h1[2], l1[2], h4[2], l4[2], b1p[2], b2[2], b3[2];
 };
 
-// T = T_k (the first two terms, which depend on k* only), f3 = fp32(F3 of the candidate).
-__device__ __forceinline__ float ttft_fast(const QRec &q, const Inst4 &r, int u, float T, float f3) {
-    const float f1 = __fadd_rn(r.h1[u], __fadd_rn(r.l1[u], q.fp));
-    const float f4 = __fadd_rn(__fadd_rn(r.h4[u], q.ph), __fadd_rn(r.l4[u], q.pl));
-    float t = __fmaf_rn(r.b1p[u], f1, T);
-    t = __fmaf_rn(r.b2[u], f3, t);
-    t = __fmaf_rn(r.b3[u], f4, t);
-    return t;
+// T: the first two terms, which depend on k* only; f3 = fp32(F3 of the candidate); F1 and F4
+// by exact fp32 sums of the split totals and the query's parts.
+template <bool COMPACT>
+__device__ __forceinline__ f32x2 ttft_fast2(f32x2 fp, f32x2 ph, f32x2 pl, const Inst4 &r, int v, f32x2 T, f32x2 f3) {
+    const f32x2 f1 = add2(r.h1[v], COMPACT ? fp : add2(r.l1[v], fp));
+    const f32x2 f4 = add2(add2(r.h4[v], ph), add2(r.l4[v], pl));
+    f32x2 t = fma2(r.b1p[v], f1, T);
+    t = fma2(r.b2[v], f3, t);
+    return fma2(r.b3[v], f4, t);
 }
 
 // Exact int64 path for instances whose totals do not split into fp32.
 template <int MODE>
-__device__ float ttft_exact64(const DevConfig &c, const StateBuf &sb, const QRec &q, int j, int k, const float T) {
-    if (q.fp != q.fp) return q.fp;
+__device__ float ttft_exact64(const DevConfig &c, const StateBuf &sb, int qp, int j, int k, const float T) {
     const InstParams ip = sb.inst[j];
     const int m = c.moi[j];
-    const long long p = q.p;
+    const long long p = qp;
     const float f1 = __ll2float_rn(ip.f1tot + p);
     const float f3 = __ll2float_rn(sb.f3[(size_t)k * c.I + j] + (MODE == 0 ? p : 0));
     const float f4 = __ll2float_rn(ip.f4tot + (p * (p + 1)) / 2);
@@ -189,6 +226,28 @@ __device__ __forceinline__ uint4 lds_u32x4(uint32_t addr) {
     uint4 v;
     asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
     return v;
+}
+
+__device__ __forceinline__ void sts_f4(uint32_t addr, float x, float y, float z, float w) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+
+__device__ __forceinline__ float lds_f32(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+// Maximum over the warp (all 32 lanes); NaN values lose, and only if all are is it NaN.
+__device__ __forceinline__ float warp_max_f32(float x) {
+    float m;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+    return m;
+}
+
+// The first index of x among v[0..3] (x is one of them, or nothing compares equal).
+__device__ __forceinline__ int first4(const float v[4], float x) {
+    return v[0] == x ? 0 : v[1] == x ? 1 : v[2] == x ? 2 : 3;
 }
 
 __device__ __forceinline__ float pick4(const float v[4], int u) {
@@ -281,8 +340,9 @@ __device__ __forceinline__ void k2_finish(const K2Launch &a, uint32_t *work, uns
 // MODE 0 / 1: SFS with the first output token in its own batch / with the last
 // prompt chunk.  MODE 2: an average-case source (Sec. 4, App. E), affine in p:
 // t = fma(p, g_j, C_j) with g_j = fp32(1/theta_j) and C_j = fp32(W_j + Tdec_j).
-// Routing launches three 256-thread CTAs per SM, the estimate alone one 768-thread CTA
-// (the same registers per thread either way).
+// Routing launches three 256-thread CTAs per SM (80 registers a thread), the estimate
+// alone one 512-thread CTA (up to 128: the two-entry path of mixed models fits without
+// spills; 768 threads took 17.9 us for 50,001 x 250 against 15.6).
 template <int MODE, int OUT>
 __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2Block : kK2EstBlock,
                                   (OUT & (kOutLag | kOutCon | kOutSweep)) ? 3 : 1) k_cand(const K2Launch a) {
@@ -312,10 +372,18 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
     // targets and the raw query rows (route with one pair stages (U, cost) per row
     // and model, sweeps (cost, acc)).
     const int WPR = Gp > 32 ? Gp / 32 : 1;  // warps per row
-    const int NP = SWEEP ? a.P : 1;
-    QRec *s_q = reinterpret_cast<QRec *>(smem + tb);                                   // [QT]
+    // (and, if rows are not whole 16-byte words, two 128-float buffers a warp in which its
+    // stores are put in order)
+    float *s_tr = reinterpret_cast<float *>(smem + tb);
+    QRec *s_q = reinterpret_cast<QRec *>(smem + tb + (I % 4 ? (size_t)blockDim.x * 32 : 0));  // [QT]
     int4 *s_part = reinterpret_cast<int4 *>(s_q + QT);                                 // [NP][QT][WPR][2]
-    float2 *s_ca = reinterpret_cast<float2 *>(s_part + (ROUTE && Gp > 32 ? 2 * NP * QT * WPR : 0));  // [QT][M]
+    // a sweep keeps the chunk's times [QT][4 Gp] instead of row partials, and per thread group
+    // and instance the model (s_m4: -1 if the group's four differ)
+    float4 *s_t = reinterpret_cast<float4 *>(s_part);                                  // [QT][Gp]
+    int32_t *s_m4 = reinterpret_cast<int32_t *>(s_t + (SWEEP ? QT * Gp : 0));          // [Gp], [Gp][4], then lambda, mu
+    float2 *s_lm = reinterpret_cast<float2 *>(s_m4 + (SWEEP ? 5 * Gp + (Gp & 1) : 0));  // [kMaxPairs] (lambda, -mu)
+    float2 *s_ca = SWEEP ? s_lm + kMaxPairs
+                         : reinterpret_cast<float2 *>(s_part + (ROUTE && Gp > 32 ? 2 * QT * WPR : 0));  // [QT][M]
     float *s_tau = reinterpret_cast<float *>(s_ca + (ROUTE ? QT * M : 0));             // [QT]
     // raw query rows as copied from global memory, two chunks in flight:
     // prompt [2][QT], and for routing tau [2][QT], dec_hat [2][QT][M], acc [2][QT][M]
@@ -425,11 +493,14 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
             goto finish;
         }
     }
-    Inst4 r;
-    int model[4], la[4];
+    int model[4];
     float ag[4], ac[4];  // average-case sources: t = fma(p, ag, ac)
     bool fast_mine = true, compact_mine = true;
     const int fs = 4 * Gp;  // scalar field stride
+    auto scal = [&](int f, int u) { return s_scal[f * fs + u * Gp + g]; };
+    // the bucket width of the tile's first instance
+    const int shift0 = AFF ? 0 : s_scal[kScShift * fs];
+    bool same_model = true, same_shift = true;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         if (AFF) {
@@ -441,29 +512,20 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
             ac[u] = (a.src == kSrcLps)      ? qd.clps
                     : (a.src == kSrcMatrix) ? 0.f
                                             : __double2float_rn(__dadd_rn(__ddiv_rn((double)sb.inst[j].f1tot, qd.theta), qd.tdec));
-            continue;
+        } else {
+            model[u] = scal(kScModel, u);
+            same_shift = same_shift && scal(kScShift, u) == shift0;
+            if (u < nv) fast_mine = fast_mine && scal(kScFast, u) != 0;
+            if (u < nv) compact_mine = compact_mine && scal(kScCompact, u) != 0;
         }
-        const int col = u * Gp + g;
-        r.shift[u] = s_scal[kScShift * fs + col];
-        r.h1[u] = __int_as_float(s_scal[kScH1 * fs + col]);
-        r.l1[u] = __int_as_float(s_scal[kScL1 * fs + col]);
-        r.h4[u] = __int_as_float(s_scal[kScH4 * fs + col]);
-        r.l4[u] = __int_as_float(s_scal[kScL4 * fs + col]);
-        r.b1p[u] = __int_as_float(s_scal[kScB1p * fs + col]);
-        r.b2[u] = __int_as_float(s_scal[kScB2 * fs + col]);
-        r.b3[u] = __int_as_float(s_scal[kScB3 * fs + col]);
-        model[u] = s_scal[kScModel * fs + col];
-        la[u] = s_scal[kScLa * fs + col];
-        if (u < nv) fast_mine = fast_mine && s_scal[kScFast * fs + col] != 0;
-        if (u < nv) compact_mine = compact_mine && s_scal[kScCompact * fs + col] != 0;
+        same_model = same_model && model[u] == model[0];
     }
-    // the bucket width of the tile's first instance (SPEC needs one width per CTA)
-    const int shift0 = AFF ? 0 : s_scal[kScShift * fs];
     if (threadIdx.x == 0) s_claim[1] = second;
     const bool fast = __syncthreads_and(fast_mine);
+    // every instance of the CTA compact (padding columns are)
+    const bool compact = fast && __syncthreads_and(compact_mine);
     const bool vec = a.vec_ok && nv == 4;
     const unsigned gmask = group_mask(Gp, lane);
-    const int grp_lane0 = lane & ~(min(Gp, 32) - 1);  // first lane of this row group in the warp
     const int wrow = g / 32;                          // warp index within a wide row
     // shared addresses of this thread's table columns: entA (k, u) at
     // ecol + u * ecst + k * erow (entB ebofs further), bucket (b, u) at
@@ -473,22 +535,63 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
     const uint32_t ecst = 8u * (uint32_t)Gp;
     const uint32_t erow = 8u * 4u * (uint32_t)Gp, brow = 4u * 4u * (uint32_t)Gp;
     const uint32_t ebofs = (uint32_t)tile_enta_bytes(c);
-    bool same_model = true;
-#pragma unroll
-    for (int u = 1; u < 4; ++u) same_model = same_model && model[u] == model[0];
-
-    bool same_shift = true;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) same_shift = same_shift && (AFF || r.shift[u] == shift0);
-    // SPEC: every thread of the CTA has four compact instances of one model (the fp32
-    // split path, F3 read from entA alone), every instance of the CTA the same bucket
-    // width (a thread's four buckets are one 16-byte load) and aligned vector stores, so
-    // none of the per-thread checks below is needed (an invalid prompt still gives NaN
-    // times, which no comparison selects)
-    const bool spec = __syncthreads_and(fast && compact_mine && nv == 4 && same_model && same_shift && a.vec_ok);
-    auto run = [&](auto fast_tag, auto spec_tag) {
+    // rows that are not whole 16-byte words: a warp puts its 128 elements of a row in order
+    // in shared memory and stores them coalesced; ntr of this lane's four lie in the pool
+    const bool tr = I % 4 != 0 && Gp >= 32;
+    const uint32_t trb = (uint32_t)__cvta_generic_to_shared(s_tr) + (threadIdx.x >> 5) * 1024u;
+    const int ntr = min(4, max(0, (I - (jb - 4 * lane) - lane + 31) >> 5));
+    if (SWEEP) {
+        if (threadIdx.x < Gp) {
+            bool one = true;
+            for (int u = 0; u < 4; ++u) {
+                s_m4[Gp + 4 * g + u] = model[u];
+                one = one && (u >= nv || model[u] == model[0]);
+            }
+            s_m4[g] = one ? model[0] : -1;
+        }
+        for (int k = threadIdx.x; k < a.P; k += blockDim.x) s_lm[k] = make_float2(a.lam[k], -a.mu[k]);
+    }
+    // UNI: every thread of the CTA has four compact instances of one model and every
+    // instance the same bucket width (a thread's four buckets are one 16-byte load)
+    const bool uni = __syncthreads_and(compact && nv == 4 && same_model && same_shift);
+    auto run = [&](auto fast_tag, auto compact_tag, auto uni_tag, auto wide_tag) {
         constexpr bool FAST = decltype(fast_tag)::value;
-        constexpr bool SPEC = decltype(spec_tag)::value;
+        constexpr bool COMPACT = decltype(compact_tag)::value;
+        constexpr bool UNI = decltype(uni_tag)::value;
+        constexpr bool WIDE = decltype(wide_tag)::value;  // Gp > 32: whole warps per row
+        // the register path for prompts with at most one budget boundary below them (not
+        // beside the routing state of threads with several models: the registers end there)
+        constexpr bool NEAR = COMPACT && !AFF && (UNI || !ROUTE);
+        // Lagrangian routing over threads of one model each: the winner of a row of several
+        // warps is described once per row, after the chunk, instead of by a lane of every warp
+        constexpr bool DEFER = ROUTE && UNI && WIDE && !CON && !SWEEP;
+        Inst4 r;
+        int r0[4], shift[4];
+        float T0[4], T1[4], X0[4], X1[4];  // entries 0 and 1 of the thread's instances (see the tile block)
+        if (!AFF) {
+            auto two = [&](int f, int v) { return pack2(__int_as_float(scal(f, 2 * v)), __int_as_float(scal(f, 2 * v + 1))); };
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                r.l1[v] = two(kScL1, v);
+                r.h1[v] = COMPACT ? add2(two(kScH1, v), r.l1[v]) : two(kScH1, v);
+                r.h4[v] = two(kScH4, v);
+                r.l4[v] = two(kScL4, v);
+                r.b1p[v] = UNI && v ? r.b1p[0] : two(kScB1p, v);
+                r.b2[v] = UNI && v ? r.b2[0] : two(kScB2, v);
+                r.b3[v] = UNI && v ? r.b3[0] : two(kScB3, v);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                shift[u] = scal(kScShift, u);
+                r0[u] = scal(kScR0, u);
+                const float2 e0 = lds_float2(ecol + u * ecst), e1 = lds_float2(ecol + u * ecst + (c.kph > 1 ? erow : 0u));
+                T0[u] = e0.x;
+                X0[u] = e0.y;
+                T1[u] = e1.x;
+                X1[u] = e1.y;
+            }
+        }
+        const f32x2 nmu2 = (ROUTE && !CON && !SWEEP) ? pack2(-a.mu[0], -a.mu[0]) : 0ull;
         // chunk k: the first QT rows of the range in s_claim[k & 1], staged in raw buffer k & 1
         for (int buf = 0;; buf ^= 1) {
             int q0, nrows;
@@ -531,46 +634,113 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
             __syncthreads();
             float *orow = (OUT & kOutMatrix) ? a.ttft + (size_t)(q0 + qs) * I + jb : nullptr;
             const size_t ostep = (size_t)QS * I;
-            for (int rr = qs; rr < nrows; rr += QS) {
-                const QRec q = s_q[rr];
-                const uint32_t p7 = (uint32_t)q.p << 7;
-                float t[4];
-                int kk[4];
-                uint4 bw4 = make_uint4(0u, 0u, 0u, 0u);
-                if (SPEC && !AFF) bw4 = lds_u32x4(bcol + (uint32_t)(q.p >> shift0) * brow);
+            const bool mat = AFF && a.src == kSrcMatrix;
+            // a given matrix: its row is read one row ahead
+            float tn[4];
+            auto read_row = [&](int rr) {
+                if (!mat || rr >= nrows) return;
+                const float *src = a.ttft_in + (size_t)(q0 + rr) * I + jb;
+                if (vec) {
+                    const float4 f = __ldcs(reinterpret_cast<const float4 *>(src));
+                    tn[0] = f.x;
+                    tn[1] = f.y;
+                    tn[2] = f.z;
+                    tn[3] = f.w;
+                } else {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (AFF) {
-                        if (a.src == kSrcMatrix)
-                            t[u] = u < nv ? __ldcs(a.ttft_in + (size_t)(q0 + rr) * I + jb + u) : kNaN;
-                        else t[u] = __fmaf_rn(q.fp, ag[u], ac[u]);
-                        kk[u] = 0;
-                        continue;
-                    }
-                    // bucket word (boundary << 7) | below: p > boundary iff (p << 7) > word
-                    const uint32_t bw = SPEC ? (u == 0 ? bw4.x : u == 1 ? bw4.y : u == 2 ? bw4.z : bw4.w)
-                                             : lds_u32(bcol + 4u * u + (uint32_t)(q.p >> r.shift[u]) * brow);
-                    kk[u] = (int)(bw & 127u) + (p7 > bw ? 1 : 0);
-                    const uint32_t ea = ecol + u * ecst + (uint32_t)kk[u] * erow;
-                    const float2 e = lds_float2(ea);
-                    if (SPEC) {
-                        // compact: F3 + p below 2^31, one exact int -> fp32 rounding
-                        const float f3 = MODE == 0 ? __int2float_rn(__float_as_int(e.y) + q.p) : e.y;
-                        t[u] = ttft_fast(q, r, u, e.x, f3);
-                    } else if (FAST) {
-                        float f3 = e.y;
-                        if (MODE == 0) {
-                            const float2 hl = lds_float2(ea + ebofs);
-                            f3 = __fadd_rn(hl.x, __fadd_rn(hl.y, q.fp));
-                        }
-                        t[u] = ttft_fast(q, r, u, e.x, f3);
+                    for (int u = 0; u < 4; ++u) tn[u] = u < nv ? __ldcs(src + u) : kNaN;
+                }
+            };
+            if (AFF) read_row(qs);
+            uint32_t trw = trb;  // this row's buffer of the two
+            for (int rr = qs; rr < nrows; rr += QS) {
+                struct {
+                    f32x2 fp2, ph2, pl2;
+                    float fp;
+                    int p;
+                } q;
+                {
+                    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(s_q + rr);
+                    const int4 y = reinterpret_cast<const int4 *>(s_q + rr)[1];
+                    q.fp2 = x.x;
+                    q.ph2 = x.y;
+                    q.pl2 = pack2(__int_as_float(y.x), __int_as_float(y.y));
+                    q.p = y.z;
+                    q.fp = __uint_as_float((unsigned)x.x);
+                }
+                float t[4];
+                int kk[4] = {0, 0, 0, 0};
+                if (AFF) {
+                    if (mat) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) t[u] = tn[u];
+                        read_row(rr + QS);
                     } else {
-                        t[u] = (u < nv) ? ttft_exact64<MODE>(c, sb, q, jb + u, kk[u], e.x) : 0.f;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) t[u] = __fmaf_rn(q.fp, ag[u], ac[u]);
+                    }
+                } else if (FAST) {
+                    float T[4], F3[4];
+                    if (NEAR && q.p <= c.near) {
+                        // at most one budget boundary lies below p: k* = (p > r0), and the
+                        // two candidate entries are in registers
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const bool k1 = q.p > r0[u];
+                            T[u] = k1 ? T1[u] : T0[u];
+                            const float x = k1 ? X1[u] : X0[u];
+                            F3[u] = MODE == 0 ? __int2float_rn(__float_as_int(x) + q.p) : x;
+                            kk[u] = k1 ? 1 : 0;
+                        }
+                    } else {
+                        const uint32_t p7 = (uint32_t)q.p << 7;
+                        uint4 bw4 = make_uint4(0u, 0u, 0u, 0u);
+                        if (UNI) bw4 = lds_u32x4(bcol + (uint32_t)(q.p >> shift0) * brow);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            // bucket word (boundary << 7) | below: p > boundary iff (p << 7) > word
+                            const uint32_t bw = UNI ? (u == 0 ? bw4.x : u == 1 ? bw4.y : u == 2 ? bw4.z : bw4.w)
+                                                    : lds_u32(bcol + 4u * u + (uint32_t)(q.p >> shift[u]) * brow);
+                            kk[u] = (int)(bw & 127u) + (p7 > bw ? 1 : 0);
+                            const uint32_t ea = ecol + u * ecst + (uint32_t)kk[u] * erow;
+                            const float2 e = lds_float2(ea);
+                            T[u] = e.x;
+                            F3[u] = e.y;
+                            if (COMPACT && MODE == 0) {
+                                // F3 + p below 2^31, one exact int -> fp32 rounding
+                                F3[u] = __int2float_rn(__float_as_int(e.y) + q.p);
+                            } else if (MODE == 0) {
+                                const float2 hl = lds_float2(ea + ebofs);
+                                F3[u] = __fadd_rn(hl.x, __fadd_rn(hl.y, q.fp));
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int v = 0; v < 2; ++v)
+                        unpack2(ttft_fast2<COMPACT>(q.fp2, q.ph2, q.pl2, r, v, pack2(T[2 * v], T[2 * v + 1]),
+                                                    pack2(F3[2 * v], F3[2 * v + 1])),
+                                t[2 * v], t[2 * v + 1]);
+                } else {
+                    const uint32_t p7 = (uint32_t)q.p << 7;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t bw = lds_u32(bcol + 4u * u + (uint32_t)(q.p >> shift[u]) * brow);
+                        kk[u] = (int)(bw & 127u) + (p7 > bw ? 1 : 0);
+                        const float2 e = lds_float2(ecol + u * ecst + (uint32_t)kk[u] * erow);
+                        t[u] = q.fp != q.fp ? kNaN : (u < nv) ? ttft_exact64<MODE>(c, sb, q.p, jb + u, kk[u], e.x) : 0.f;
                     }
                 }
                 if (OUT & kOutMatrix) {
-                    if (SPEC || vec) {
+                    if (UNI ? a.vec_ok != 0 : vec) {
                         __stcs(reinterpret_cast<float4 *>(orow), make_float4(t[0], t[1], t[2], t[3]));
+                    } else if (tr) {
+                        sts_f4(trw + 16u * lane, t[0], t[1], t[2], t[3]);
+                        __syncwarp();
+                        float *ob = orow - 3 * lane;  // element `lane` of the warp's block
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (u < ntr) __stcs(ob + 32 * u, lds_f32(trw + 4u * lane + 128u * u));
+                        trw ^= 512u;  // the other buffer: the next row's writes need not wait for these reads
                     } else {
                         for (int u = 0; u < nv; ++u) __stcs(orow + u, t[u]);
                     }
@@ -579,59 +749,70 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                 if (OUT & kOutIters) {
                     const bool bad = q.fp != q.fp;
                     const size_t o = (size_t)(q0 + rr) * I + jb;
-                    for (int u = 0; u < nv; ++u) a.first_batch[o + u] = bad ? -1 : la[u] + kk[u] + off;
+                    for (int u = 0; u < nv; ++u) a.first_batch[o + u] = bad ? -1 : scal(kScLa, u) + kk[u] + off;
                 }
-                if (ROUTE) {
-                    const bool row_ok = SPEC || q.fp == q.fp;
+                if (SWEEP) {
+                    if (!UNI) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (u >= nv) t[u] = kNaN;
+                    }
+                    s_t[rr * Gp + g] = make_float4(t[0], t[1], t[2], t[3]);
+                } else if (ROUTE) {
                     const float2 *carow = s_ca + rr * M;
                     const float tau = CON ? s_tau[rr] : 0.f;
-#pragma unroll 1
-                    for (int pp = 0; pp < (SWEEP ? NP : 1); ++pp) {
-                        const float lam = SWEEP ? a.lam[pp] : 0.f;
-                        const float mu = a.mu[pp];
+                    float2 ca0 = make_float2(0.f, 0.f);
+                    if (UNI || same_model) ca0 = carow[model[0]];
+                    float B[4];  // constrained: the times themselves, NaN beyond the pool
+                    if (!UNI) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (u >= nv) t[u] = kNaN;
+                    }
+                    unsigned k2 = 0u;
+                    float m2 = 0.f;
+                    if (CON) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) B[u] = t[u];
+                        m2 = fminf(fminf(t[0], t[1]), fminf(t[2], t[3]));  // NaN only if all are
+                        k2 = m2 == m2 ? order_key(-m2) : 0u;
+                    }
+                    do {
                         float U[4];
-                        if (SPEC || same_model) {
-                            const float2 ca = carow[model[0]];
-                            U[0] = U[1] = U[2] = U[3] = SWEEP ? __fmaf_rn(-lam, ca.x, ca.y) : ca.x;
+                        if (UNI || same_model) {
+                            U[0] = U[1] = U[2] = U[3] = ca0.x;
                         } else {
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const float2 ca = carow[model[u]];
-                                U[u] = SWEEP ? __fmaf_rn(-lam, ca.x, ca.y) : ca.x;
-                            }
+                            for (int u = 0; u < 4; ++u) U[u] = carow[model[u]].x;
                         }
-                        // this thread's best of its four instances (first max wins); NaN marks
-                        // an invalid row or an instance beyond the pool
-                        float best1, best2 = 0.f;
-                        int u1 = 0, u2 = 0;
+                        // this thread's objective values; NaN (an invalid prompt, no estimate or an
+                        // instance beyond the pool) is never the maximum
+                        float J[4];
                         if (CON) {
-                            best1 = ((SPEC || 0 < nv) && row_ok && t[0] <= tau) ? U[0] : kNaN;
-                            best2 = ((SPEC || 0 < nv) && row_ok) ? t[0] : kNaN;
 #pragma unroll
-                            for (int u = 1; u < 4; ++u) {
-                                if ((SPEC || u < nv) && t[u] <= tau && (U[u] > best1 || best1 != best1)) { best1 = U[u]; u1 = u; }
-                                // a NaN time (no estimate, per candidate only from a matrix
-                                // source) is never the least
-                                if ((SPEC || u < nv) && (!AFF || t[u] == t[u]) && (t[u] < best2 || (AFF && best2 != best2))) {
-                                    best2 = t[u];
-                                    u2 = u;
-                                }
-                            }
+                            for (int u = 0; u < 4; ++u) J[u] = t[u] <= tau ? U[u] : kNaN;
                         } else {
-                            best1 = ((SPEC || 0 < nv) && row_ok) ? __fmaf_rn(-mu, t[0], U[0]) : kNaN;
 #pragma unroll
-                            for (int u = 1; u < 4; ++u) {
-                                // J is NaN exactly when the time is (no estimate): never chosen.
-                                // Only a matrix source mixes NaN and finite times in a row.
-                                const float J = __fmaf_rn(-mu, t[u], U[u]);
-                                if ((SPEC || u < nv) && (!AFF || J == J) && (J > best1 || (AFF && best1 != best1))) {
-                                    best1 = J;
-                                    u1 = u;
-                                }
-                            }
+                            for (int v = 0; v < 2; ++v)
+                                unpack2(fma2(nmu2, pack2(t[2 * v], t[2 * v + 1]), pack2(U[2 * v], U[2 * v + 1])), J[2 * v],
+                                        J[2 * v + 1]);
                         }
-                        const unsigned k1 = (best1 == best1) ? order_key(best1) : 0u;
-                        const unsigned k2 = (CON && best2 == best2 && row_ok) ? order_key(-best2) : 0u;
+                        const float m1 = fmaxf(fmaxf(J[0], J[1]), fmaxf(J[2], J[3]));
+                        if (DEFER) {
+                            // the first of the lanes with the warp's maximum leaves its times; its
+                            // instance is picked when the chunk's rows are written (see below)
+                            const float w = warp_max_f32(m1);
+                            const unsigned best = __ballot_sync(kFull, m1 == w);
+                            if (m1 == w && (best & lanemask_lt()) == 0u) {
+                                float4 *part = reinterpret_cast<float4 *>(s_part + 2 * (rr * WPR + wrow));
+                                part[0] = make_float4(t[0], t[1], t[2], t[3]);
+                                part[1] = make_float4(w, U[0], __int_as_float(jb), 0.f);
+                            } else if (best == 0u && lane == 0) {  // an invalid prompt
+                                reinterpret_cast<float *>(s_part + 2 * (rr * WPR + wrow) + 1)[0] = kNaN;
+                            }
+                            break;
+                        }
+                        const unsigned k1 = m1 == m1 ? order_key(m1) : 0u;
                         // row group argmax: the lowest lane among the maximal keys
                         const unsigned w1 = __reduce_max_sync(gmask, k1);
                         const int src1 = __ffs(__ballot_sync(gmask, k1 == w1) & gmask) - 1;
@@ -641,38 +822,122 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                             w2 = __reduce_max_sync(gmask, k2);
                             src2 = __ffs(__ballot_sync(gmask, k2 == w2) & gmask) - 1;
                         }
-                        // the winner of each reduction describes itself
-                        const Cand c1 = {w1, jb + u1, pick4(t, u1), pick4(U, u1)};
-                        const Cand c2 = {w2, jb + u2, pick4(t, u2), pick4(U, u2)};
+                        // the winner of each reduction describes itself: the first of its instances
+                        // with the best value
                         if (Gp <= 32) {
                             const bool use2 = CON && w1 == 0u;
-                            if (lane == (use2 ? src2 : src1))
-                                write_pick(a, (size_t)pp * a.Q + q0 + rr, use2 ? c2 : c1);
+                            if (lane == (use2 ? src2 : src1)) {
+                                const int u = use2 ? first4(B, m2) : first4(J, m1);
+                                write_pick(a, (size_t)(q0 + rr), Cand{use2 ? w2 : w1, jb + u, pick4(t, u), pick4(U, u)});
+                            }
                         } else {
                             // wide rows: each warp leaves its partial; combined once per chunk
-                            int4 *part = s_part + 2 * ((pp * QT + rr) * WPR + wrow);
-                            if (lane == src1) part[0] = pack(c1);
-                            if (CON && lane == src2) part[1] = pack(c2);
+                            int4 *part = s_part + 2 * (rr * WPR + wrow);
+                            if (lane == src1) {
+                                const int u = first4(J, m1);
+                                part[0] = pack(Cand{w1, jb + u, pick4(t, u), pick4(U, u)});
+                            }
+                            if (CON && lane == src2) {
+                                const int u = first4(B, m2);
+                                part[1] = pack(Cand{w2, jb + u, pick4(t, u), pick4(U, u)});
+                            }
                         }
-                    }
+                    } while (false);
                 }
             }
-            if (ROUTE && Gp > 32) {
-                // one thread per (row, pair) combines the warps of the row in instance order
+            if (SWEEP) {
+                // A lane per (row, pair): each follows the pool's times of its row in instance
+                // order, so a candidate of a pair costs a packed multiply-add and a running
+                // maximum, with no reduction across lanes and no row-by-row winner (a lane per
+                // four instances and one pair after the other took about 120 warp instructions
+                // per row and pair).  32 pairs x 4,096 queries x 64 instances: kernel 17.3 -> 12.0 us.
                 __syncthreads();
-                for (int t2 = threadIdx.x; t2 < nrows * NP; t2 += blockDim.x) {
-                    const int pp = t2 / nrows;
-                    const int r2 = t2 - pp * nrows;
+                const int pg = a.pg, rw = 32 / pg, np = (a.P + 31) / 32;
+                const int pl = lane & (pg - 1), rs = lane / pg;
+                const int units = (nrows + rw - 1) / rw * np;
+                for (int un = threadIdx.x >> 5; un < units; un += blockDim.x >> 5) {
+                    const int row = un / np * rw + rs, pp = un % np * 32 + pl;
+                    const bool act = row < nrows && pp < a.P;
+                    const int rr = min(row, nrows - 1);
+                    const float2 lm = s_lm[min(pp, a.P - 1)];
+                    const f32x2 nm = pack2(lm.y, lm.y);
+                    const float4 *tr4 = s_t + rr * Gp;
+                    const float2 *carow = s_ca + rr * M;
+                    float best = -INFINITY, U = 0.f;
+                    int bj = -1, cur = -1;
+                    for (int gg = 0; 4 * gg < I; ++gg) {
+                        const float4 t4 = tr4[gg];
+                        const int m = s_m4[gg];
+                        float U4[4], J[4];
+                        if (m >= 0) {
+                            if (m != cur) {
+                                const float2 ca = carow[m];
+                                U = __fmaf_rn(-lm.x, ca.x, ca.y);
+                                cur = m;
+                            }
+                            U4[0] = U4[1] = U4[2] = U4[3] = U;
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const float2 ca = carow[s_m4[Gp + 4 * gg + u]];
+                                U4[u] = __fmaf_rn(-lm.x, ca.x, ca.y);
+                            }
+                        }
+                        unpack2(fma2(nm, pack2(t4.x, t4.y), pack2(U4[0], U4[1])), J[0], J[1]);
+                        unpack2(fma2(nm, pack2(t4.z, t4.w), pack2(U4[2], U4[3])), J[2], J[3]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (J[u] > best) {  // NaN (no estimate, or beyond the pool) never is
+                                best = J[u];
+                                bj = 4 * gg + u;
+                            }
+                    }
+                    if (act) {
+                        Cand w = {0u, 0, 0.f, 0.f};
+                        if (bj >= 0) {
+                            const float2 ca = carow[s_m4[Gp + bj]];
+                            w = Cand{1u, bj, reinterpret_cast<const float *>(tr4)[bj], __fmaf_rn(-lm.x, ca.x, ca.y)};
+                        }
+                        write_pick(a, (size_t)pp * a.Q + q0 + row, w);
+                    }
+                }
+            } else if (DEFER) {
+                // one thread per row: the best warp of the row (the first among equals), then
+                // the first of the winning thread's four instances with that value
+                __syncthreads();
+                for (int r2 = threadIdx.x; r2 < nrows; r2 += blockDim.x) {
+                    const float4 *part = reinterpret_cast<const float4 *>(s_part + 2 * (size_t)(r2 * WPR));
+                    int wb = 0;
+                    float w = part[1].x;
+                    for (int wi = 1; wi < WPR; ++wi) {
+                        const float x = part[2 * wi + 1].x;
+                        if (x > w) {
+                            w = x;
+                            wb = wi;
+                        }
+                    }
+                    const float4 tw = part[2 * wb], d = part[2 * wb + 1];
+                    const float nm = -a.mu[0], tt[4] = {tw.x, tw.y, tw.z, tw.w};
+                    const float J[4] = {__fmaf_rn(nm, tt[0], d.y), __fmaf_rn(nm, tt[1], d.y), __fmaf_rn(nm, tt[2], d.y),
+                                        __fmaf_rn(nm, tt[3], d.y)};
+                    const int u = first4(J, w);
+                    // (an invalid prompt's row is NaN in every warp)
+                    write_pick(a, (size_t)(q0 + r2), Cand{w == w ? 1u : 0u, __float_as_int(d.z) + u, pick4(tt, u), d.y});
+                }
+            } else if (ROUTE && Gp > 32) {
+                // one thread per row combines the warps of the row in instance order
+                __syncthreads();
+                for (int r2 = threadIdx.x; r2 < nrows; r2 += blockDim.x) {
                     Cand c1 = {0u, 0, 0.f, 0.f}, c2 = {0u, 0, 0.f, 0.f};
                     for (int wi = 0; wi < WPR; ++wi) {
-                        const Cand x1 = unpack(s_part[2 * ((pp * QT + r2) * WPR + wi)]);
+                        const Cand x1 = unpack(s_part[2 * (r2 * WPR + wi)]);
                         if (x1.key > c1.key) c1 = x1;
                         if (CON) {
-                            const Cand x2 = unpack(s_part[2 * ((pp * QT + r2) * WPR + wi) + 1]);
+                            const Cand x2 = unpack(s_part[2 * (r2 * WPR + wi) + 1]);
                             if (x2.key > c2.key) c2 = x2;
                         }
                     }
-                    write_pick(a, (size_t)pp * a.Q + q0 + r2, (CON && c1.key == 0u) ? c2 : c1);
+                    write_pick(a, (size_t)(q0 + r2), (CON && c1.key == 0u) ? c2 : c1);
                 }
             }
             if (threadIdx.x == 0) {  // into the slot this chunk was read from
@@ -682,10 +947,14 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
             __syncthreads();
         }
     };
-    if (spec) run(Flag<true>{}, Flag<true>{});
-    else if (fast) run(Flag<true>{}, Flag<false>{});
-    else run(Flag<false>{}, Flag<false>{});
-    (void)grp_lane0;
+    const Flag<true> yes{};
+    const Flag<false> no{};
+    if (AFF) run(yes, yes, no, no);
+    else if (uni && Gp > 32) run(yes, yes, yes, yes);
+    else if (uni) run(yes, yes, yes, no);
+    else if (compact) run(yes, yes, no, no);
+    else if (fast) run(yes, no, no, no);
+    else run(no, no, no, no);
     }
 finish:
     k2_finish(a, a.work, gridDim.x * gridDim.y, gridDim.y);
@@ -941,7 +1210,7 @@ __global__ void __launch_bounds__(256) k_baseline(const K2Launch a, int policy, 
             const int k = bk.y + (q.p > bk.x ? 1 : 0);
             const float T =
                 reinterpret_cast<const float2 *>(sb.tile + tile_base(c, j))[(size_t)k * 4 * c.tgp + tile_col(c, j)].x;
-            a.ttft_chosen[i] = ttft_exact64<MODE>(c, sb, q, j, k, T);
+            a.ttft_chosen[i] = ttft_exact64<MODE>(c, sb, q.p, j, k, T);
         }
     }
 }

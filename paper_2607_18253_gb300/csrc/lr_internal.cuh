@@ -47,6 +47,7 @@ struct DevConfig {
     int32_t I, M, capR, capW;
     int32_t pmax, mode, max_iters, tgp;     // tgp: thread groups per instance tile of the candidate kernel
     int32_t kph, nbh;                       // table row counts (host bounds over instances)
+    int32_t near;                           // k* <= 1 on every instance for a prompt up to this
     const int32_t *moi, *B, *S, *shift, *nb;
     const float *coef, *pin, *pout;
 };
@@ -158,7 +159,8 @@ __device__ __forceinline__ long long warp_sum64(long long v) {
 // bulk copy brings it in.  Instance j0 + 4g + u of the tile sits in column u * tgp + g:
 //   entA [kph][4][tgp]    8 bytes: T_k (fp32) and X_k, which is f3_k (fp32) when the
 //                         first token comes with the last chunk, else F3_k as an int32
-//                         (valid when the instance is compact: F3_k + pmax < 2^31)
+//                         (valid when the instance is compact: F3_k + pmax < 2^31 and
+//                         F1tot + pmax <= 2^24)
 //   entB [kph][4][tgp]    8 bytes: H3_k, L3_k, the exact fp32 split of F3_k
 //   bkt  [nbh][tgp][4]    uint32: (in-bucket boundary << 7) | boundaries below, the
 //                         boundary 2^24 - 1 when the bucket holds none; a thread's four
@@ -167,8 +169,8 @@ __device__ __forceinline__ long long warp_sum64(long long v) {
 //   scal [kScal][4][tgp]  32-bit scalars, fields kSc*
 // A warp reads a table as one dense 4- or 8-byte word per lane (1 or 2 shared-memory
 // wavefronts); a compact CTA reads only entA.
-constexpr int kScal = 12;
-enum : int { kScShift = 0, kScH1, kScL1, kScH4, kScL4, kScB1p, kScB2, kScB3, kScModel, kScLa, kScFast, kScCompact };
+constexpr int kScal = 13;
+enum : int { kScShift = 0, kScH1, kScL1, kScH4, kScL4, kScB1p, kScB2, kScB3, kScModel, kScLa, kScFast, kScCompact, kScR0 };
 constexpr uint32_t kBktNone = (1u << 24) - 1;  // bucket boundary field of a bucket without one
 __host__ __device__ inline size_t tile_enta_bytes(const DevConfig &c) { return (size_t)c.kph * 4 * c.tgp * 8; }
 __host__ __device__ inline size_t tile_ent_bytes(const DevConfig &c) { return 2 * tile_enta_bytes(c); }
@@ -319,6 +321,7 @@ struct K2Launch {
     // launch shape: Gp thread groups of four instances per row (a power of two up
     // to 32, else a multiple of 32), QS rows in flight, QT rows per staged chunk
     int32_t Gp, QS, QT, vec_ok;
+    int32_t pg;  // sweep: lanes per row (a power of two, the pairs up to 32)
     // TTFT source (kSrc*) and, for the average-case ones, the instance constants
     int32_t src;
     const QueueDev *qd;
@@ -347,7 +350,7 @@ cudaError_t cand_occupancy(int mode, bool route, int block, size_t smem, int *bl
 cudaError_t set_k2_smem(size_t bytes);
 constexpr int kK2Block = 256;                // route: three CTAs per SM, one fits beside a load's CTA
 constexpr size_t kK2SmemTarget = 72 * 1024;  // three CTAs per SM
-constexpr int kK2EstBlock = 768;             // estimate alone: one CTA per SM, one tile copy per SM
+constexpr int kK2EstBlock = 512;             // estimate alone: one CTA per SM, one tile copy per SM
 constexpr size_t kK2EstSmemTarget = 120 * 1024;
 
 // K3: append routed queries and advance every instance to t_now (online stream).

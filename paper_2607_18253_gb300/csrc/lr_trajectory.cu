@@ -719,7 +719,8 @@ __device__ void summarize_instance(const K1Launch &a, const StateBuf &out, int j
     const float b1d = c.coef[m_j * 5 + 2];
     const long long ppmax = ((long long)c.pmax * (c.pmax + 1)) / 2;
     bool fast = (f1 + c.pmax < kFastLimit) && (f4 + ppmax < kFastLimit);
-    bool compact = true;  // every F3_k + pmax below 2^31 (first token in its own batch)
+    // every F1 exact in fp32, and every F3_k + pmax below 2^31 (first token in its own batch)
+    bool compact = f1 + c.pmax <= (1 << 24);
     const long long lowmask = (1LL << kSplitBits) - 1;
     int kp = 0;          // table rows kept
     long long rc = r0;   // cumulative budget R_k
@@ -927,6 +928,7 @@ __device__ void summarize_instance(const K1Launch &a, const StateBuf &out, int j
         sc[kScLa * fs] = la;
         sc[kScFast * fs] = ip.fast;
         sc[kScCompact * fs] = (fast && compact) ? 1 : 0;
+        sc[kScR0 * fs] = r0;
     }
 }
 

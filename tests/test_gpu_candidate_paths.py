@@ -1,0 +1,128 @@
+"""The candidate kernel's paths against the CPU oracle, bit for bit: instance counts around the
+warp and tile edges (rows that are not whole 16-byte words are put in order in shared memory),
+prompts around the bound up to which a candidate's two table entries stay in registers, sweeps
+with every lane split, and instances whose prefill total is not exact in fp32.
+
+Times, utilities and assignments are compared exactly (both sides evaluate the same sequence
+of IEEE operations)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+from paper_2607_18253_gb300 import workloads as W  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def R():
+    from paper_2607_18253_gb300 import router
+    return router
+
+
+def bits(a):
+    return np.ascontiguousarray(a, np.float32).view(np.uint32)
+
+
+def check(wl, sweep=5):
+    rt = R().LatencyRouter.from_workload(wl, max_pairs=max(1, sweep))
+    rt.load_state(*R().state_tensors(wl))
+    p, dh, acc, tau = R().query_tensors(wl)
+    Q, I = wl.num_queries, wl.num_instances
+    _, lt, t32, _ = oracle.estimate_matrix(wl)
+    # estimates, into a buffer whose rows start at any 4-byte word, guarded at both ends
+    for shift in (0, 1):
+        guard = torch.full((Q * I + 8,), -7.0, device="cuda")
+        out = guard[4 + shift:4 + shift + Q * I]
+        rt.estimate_ttft(p, out=out)
+        np.testing.assert_array_equal(bits(out.cpu().numpy()), bits(t32).ravel())
+        assert (guard[:4 + shift] == -7.0).all() and (guard[4 + shift + Q * I:] == -7.0).all()
+    fb = torch.empty((Q, I), dtype=torch.int32, device="cuda")
+    rt.estimate_ttft(p, first_batch=fb)
+    np.testing.assert_array_equal(fb.cpu().numpy(), lt)
+    if I > 1024:
+        rt.close()
+        return
+    # routes, with and without the matrix
+    for tt in (None, tau):
+        for matrix in (None, torch.empty((Q, I), device="cuda")):
+            o = rt.route(p, dh, acc, wl.lam[:1], None if tt is not None else wl.mu[:1], tau=tt, ttft_matrix=matrix)
+            a, u, tc = oracle.route(wl, t32, tau=wl.tau if tt is not None else None)
+            np.testing.assert_array_equal(o["assign"].cpu().numpy(), a)
+            np.testing.assert_array_equal(bits(o["util"].cpu().numpy()), bits(u))
+            np.testing.assert_array_equal(bits(o["ttft_chosen"].cpu().numpy()), bits(tc))
+            if matrix is not None:
+                np.testing.assert_array_equal(bits(matrix.cpu().numpy()), bits(t32))
+    if sweep > 1:
+        lam, mu = np.linspace(0.0, 3.0, sweep).astype(np.float32), np.geomspace(1e-3, 1.0, sweep).astype(np.float32)
+        matrix = torch.empty((Q, I), device="cuda")
+        o = rt.route(p, dh, acc, lam, mu, frontier=True, ttft_matrix=matrix)
+        a, u, tc = oracle.route(wl, t32, lam=lam, mu=mu)
+        np.testing.assert_array_equal(o["assign"].cpu().numpy(), a)
+        np.testing.assert_array_equal(bits(o["util"].cpu().numpy()), bits(u))
+        np.testing.assert_array_equal(bits(o["ttft_chosen"].cpu().numpy()), bits(tc))
+        np.testing.assert_array_equal(bits(matrix.cpu().numpy()), bits(t32))
+        np.testing.assert_allclose(o["frontier"].cpu().numpy(), oracle.frontier(wl, a, tc), rtol=1e-12)
+    assert rt.status() == R().LR_OK
+    rt.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("I", [1, 3, 5, 31, 33, 125, 128, 129, 131, 250, 257, 510, 1023, 1025])
+def test_instance_counts(I, mode):
+    # (a wide pool's tables hold fewer budget boundaries)
+    wl = W.small_workload(1000 + I, num_instances=I, num_models=3, num_queries=37, first_token_mode=mode,
+                          budget_range=(16, 96) if I < 500 else (64, 128), min_gap=8 if I < 500 else 48)
+    gap = wl.max_batched_tokens - wl.max_seqs + 1
+    near = int(gap.min()) + 1  # at most one budget boundary lies below a prompt up to this
+    wl.prompt_len[:8] = np.clip([1, near - 1, near, near + 1, near + 2, 2 * near, 159, 160], 1, 160)
+    check(wl)
+
+
+@pytest.mark.parametrize("I", [12, 128, 256])
+@pytest.mark.parametrize("grouped", [False, True])
+def test_models_of_a_thread(I, grouped):
+    # four instances of one model a thread and equal budgets (one bucket width), or mixed models
+    wl = W.small_workload(5, num_instances=I, num_models=4, num_queries=300, budget_range=(64, 64), min_gap=8)
+    moi = np.arange(I) * 4 // I if grouped else wl.model_of_instance
+    wl = dataclasses.replace(wl, model_of_instance=moi.astype(np.int32), max_seqs=np.full(I, 8, np.int32),
+                             n_run=np.minimum(wl.n_run, 8))
+    # replicas with equal states: ties go to the lowest instance
+    for a in (wl.n_run, wl.run_ctx, wl.run_pre, wl.run_dec, wl.n_wait, wl.wait_pre, wl.wait_dec):
+        a[1::2] = a[0::2][:a[1::2].shape[0]]
+    check(wl)
+
+
+@pytest.mark.parametrize("P", [2, 3, 8, 31, 32, 33, 64])
+def test_sweep_lane_splits(P):
+    check(W.small_workload(40 + P, num_instances=45, num_models=3, num_queries=101, budget_range=(16, 96), min_gap=8),
+          sweep=P)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_prefill_totals_beyond_fp32(mode):
+    # one instance whose residents hold more than 2^24 prompt tokens: the whole tile leaves the
+    # single-sum path
+    I = 40
+    wl = W.small_workload(77, num_instances=I, num_models=3, num_queries=33, first_token_mode=mode,
+                          budget_range=(1 << 20, 1 << 20), min_gap=1 << 19, max_prompt_len=4000)
+    wl.wait_pre[7, :] = (1 << 22) + 12345
+    wl.wait_dec[7, :] = 3
+    wl.n_wait[7] = wl.cap_waiting
+    check(wl)
+
+
+def test_one_token_prompts():
+    # max_prompt_len 1: the tables have a single row
+    check(W.small_workload(3, num_instances=9, num_models=2, num_queries=5, max_prompt_len=1))
