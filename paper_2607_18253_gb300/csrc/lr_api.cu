@@ -595,7 +595,7 @@ int lr_route(lr_ctx *c, int32_t Q, const int32_t *prompt_len, const int32_t *dec
                                     sh.block, sh.smem, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "route launch");
     if (frontier_out) {
-        e = lr::launch_frontier(a, frontier_out, (cudaStream_t)stream);
+        e = lr::launch_frontier(a, frontier_out, c->sms, (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "frontier launch");
     }
     return LR_OK;

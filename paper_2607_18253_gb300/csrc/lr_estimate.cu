@@ -37,6 +37,7 @@
 // Routing reduces each row with redux.sync over the objective (the value itself, or an
 // order-preserving integer key): the lowest lane (lowest instance) among the maximal wins,
 // as in a first-max scan.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "lr_internal.cuh"
@@ -960,37 +961,74 @@ finish:
     k2_finish(a, a.work, gridDim.x * gridDim.y, gridDim.y);
 }
 
-// Per-pair means of (accuracy, cost, TTFT) of the chosen instances, fp64, fixed
-// reduction order (one CTA per pair).
-__global__ void __launch_bounds__(256) k_frontier(const K2Launch a, double *out) {
-    __shared__ double red[3][256];
-    const int pp = blockIdx.x;
+// Per-pair means of (accuracy, cost, TTFT) of the chosen instances, fp64, in a fixed
+// reduction order: a cluster of CTAs per pair, each over a contiguous range of queries, its
+// rank 0 adding the ranks' sums in order.  Bound by the SM's narrow fp64 unit (six
+// operations a query: three conversions, three additions, about 16 cycles per warp
+// instruction) and the three dependent loads of a query, so the pairs spread over the SMs
+// and a thread has four queries' loads in flight.  32 pairs x 4,096 queries: 17.1 us (one
+// CTA per pair, one query at a time) -> 7.3 us.
+constexpr int kFrontierThreads = 256;
+__global__ void __launch_bounds__(kFrontierThreads) k_frontier(const K2Launch a, double *out) {
+    __shared__ double red[3][kFrontierThreads];
+    __shared__ double part[8][3];  // rank 0: the ranks' sums
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    cluster.sync();  // every CTA of the cluster runs before one writes into another's shared memory
+    const int pp = blockIdx.y, cs = gridDim.x, rank = blockIdx.x;
     const DevConfig &c = a.cfg;
+    const double nan = __longlong_as_double(0x7ff8000000000000LL);
+    const int per = (a.Q + cs - 1) / cs, lo = rank * per, hi = min(a.Q, lo + per);
     double sa = 0.0, sc = 0.0, st = 0.0;
-    for (int i = threadIdx.x; i < a.Q; i += blockDim.x) {
-        const size_t o = (size_t)pp * a.Q + i;
-        const int jj = a.assign[o];
-        if (jj < 0 || jj >= c.I) {
-            sa = sc = st = __longlong_as_double(0x7ff8000000000000LL);
-            continue;
+    constexpr int kU = 4;
+    for (int i0 = lo + threadIdx.x; i0 < hi; i0 += kU * kFrontierThreads) {
+        int jj[kU], m[kU], d[kU], p[kU];
+        float t[kU], ac[kU];
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+            const int i = i0 + k * kFrontierThreads;
+            const size_t o = (size_t)pp * a.Q + i;
+            jj[k] = i < hi ? a.assign[o] : 0;
+            t[k] = i < hi ? a.ttft_chosen[o] : 0.f;
+            p[k] = i < hi ? a.prompt[i] : 0;
         }
-        const int m = c.moi[jj];
-        const size_t g = (size_t)i * c.M + m;
-        const float cost = __fmaf_rn((float)a.dec_hat[g], c.pout[m], __fmul_rn((float)a.prompt[i], c.pin[m]));
-        sa += (double)a.acc[g];
-        sc += (double)cost;
-        st += (double)a.ttft_chosen[o];
+#pragma unroll
+        for (int k = 0; k < kU; ++k) m[k] = (jj[k] >= 0 && jj[k] < c.I) ? c.moi[jj[k]] : 0;
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+            const int i = i0 + k * kFrontierThreads;
+            const size_t g = (size_t)i * c.M + m[k];
+            d[k] = i < hi ? a.dec_hat[g] : 0;
+            ac[k] = i < hi ? a.acc[g] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+            if (i0 + k * kFrontierThreads >= hi) break;
+            if (jj[k] < 0 || jj[k] >= c.I) {  // no instance: the means are undefined
+                sa = sc = st = nan;
+                continue;
+            }
+            const float cost = __fmaf_rn((float)d[k], c.pout[m[k]], __fmul_rn((float)p[k], c.pin[m[k]]));
+            sa += (double)ac[k];
+            sc += (double)cost;
+            st += (double)t[k];
+        }
     }
     red[0][threadIdx.x] = sa;
     red[1][threadIdx.x] = sc;
     red[2][threadIdx.x] = st;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+    for (int s = kFrontierThreads / 2; s > 0; s >>= 1) {
         if ((int)threadIdx.x < s)
             for (int f = 0; f < 3; ++f) red[f][threadIdx.x] += red[f][threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x < 3) out[pp * 3 + threadIdx.x] = red[threadIdx.x][0] / (double)a.Q;
+    if (threadIdx.x < 3) cluster.map_shared_rank(&part[0][0], 0)[rank * 3 + threadIdx.x] = red[threadIdx.x][0];
+    cluster.sync();
+    if (rank == 0 && threadIdx.x < 3) {
+        double v = part[0][threadIdx.x];
+        for (int r = 1; r < cs; ++r) v += part[r][threadIdx.x];
+        out[pp * 3 + threadIdx.x] = v / (double)a.Q;
+    }
 }
 
 template <int MODE>
@@ -1273,9 +1311,23 @@ cudaError_t launch_features(const K2Launch &a, int sms, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_frontier(const K2Launch &a, double *out, cudaStream_t st) {
-    k_frontier<<<a.P, 256, 0, st>>>(a, out);
-    return cudaGetLastError();
+cudaError_t launch_frontier(const K2Launch &a, double *out, int sms, cudaStream_t st) {
+    // CTAs per pair: a power of two up to 8 (the portable cluster size), while the pairs
+    // leave SMs free and each CTA still has 512 queries
+    int cs = 1;
+    while (cs < 8 && 2 * cs * a.P <= sms && 512 * cs < a.Q) cs *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cs, a.P);
+    cfg.blockDim = dim3(kFrontierThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cs;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_frontier, a, out);
 }
 
 size_t baseline_smem(const DevConfig &c) {

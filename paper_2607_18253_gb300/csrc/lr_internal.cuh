@@ -337,7 +337,7 @@ inline int k2_work_words(int I) { return (I + 1023) / 1024 + 2; }
 int cand_out_flags(bool matrix, bool iters, bool route, bool constrained, int P);
 cudaError_t launch_cand(const K2Launch &a, int out, dim3 grid, int block, size_t smem, cudaStream_t st);
 cudaError_t launch_features(const K2Launch &a, int sms, cudaStream_t st);
-cudaError_t launch_frontier(const K2Launch &a, double *out, cudaStream_t st);
+cudaError_t launch_frontier(const K2Launch &a, double *out, int sms, cudaStream_t st);
 // Baseline routing policies (0 Round Robin, 1 Shortest Queue, 2 Latency-Agnostic) and
 // the stream metrics (OnTimeUtility, SLO attainment) over routed queries.
 size_t baseline_smem(const DevConfig &c);

@@ -126,3 +126,23 @@ def test_prefill_totals_beyond_fp32(mode):
 def test_one_token_prompts():
     # max_prompt_len 1: the tables have a single row
     check(W.small_workload(3, num_instances=9, num_models=2, num_queries=5, max_prompt_len=1))
+
+
+@pytest.mark.parametrize("P,Q", [(1, 1), (1, 511), (1, 513), (1, 5000), (3, 2048), (19, 2049), (64, 1025)])
+def test_frontier_splits(P, Q):
+    # one to eight CTAs per pair, ranges that end inside a thread's four queries, and queries
+    # without an instance
+    wl = W.small_workload(60, num_instances=11, num_models=3, num_queries=Q, budget_range=(16, 64), min_gap=8)
+    rt = R().LatencyRouter.from_workload(wl, max_pairs=P)
+    rt.load_state(*R().state_tensors(wl))
+    p, dh, acc, _ = R().query_tensors(wl)
+    lam, mu = np.linspace(0.5, 2.0, P).astype(np.float32), np.geomspace(1e-2, 1.0, P).astype(np.float32)
+    o = rt.route(p, dh, acc, lam, mu, frontier=True)
+    want = oracle.frontier(wl, o["assign"].cpu().numpy(), o["ttft_chosen"].cpu().numpy())
+    np.testing.assert_allclose(o["frontier"].cpu().numpy(), want, rtol=1e-12)
+    again = rt.route(p, dh, acc, lam, mu, frontier=True)
+    assert torch.equal(o["frontier"].view(torch.int64), again["frontier"].view(torch.int64))
+    p[Q // 2] = 0
+    bad = rt.route(p, dh, acc, lam, mu, frontier=True)
+    assert torch.isnan(bad["frontier"]).all() and rt.status() == R().LR_EINVAL
+    rt.close()
