@@ -31,6 +31,7 @@ struct lr_ctx {
     lr::DevCtl *ctl = nullptr;
     int max_seqs = 0;
     size_t k3_smem = 0;
+    bool k3_ok = false;  // the queue capacities are within what lr_advance takes
     float *scratch_tch = nullptr;
     uint32_t *k2_work = nullptr;  // the candidate kernel's row counters
     double *ontime_part = nullptr;  // per-CTA partial sums of lr_on_time_utility
@@ -401,8 +402,11 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     c->sw = make_shape(d, true, true);
     if (!c->est.ok) return bail(LR_ECAPACITY, "summary tables too large for shared memory");
     c->k3_smem = lr::kK3Warps * lr::advance_smem_per_warp(d);
+    // capacities lr_advance takes: 32 B a running and 12 B a waiting request within 200 KB
+    // for four instances (it needs less)
+    c->k3_ok = lr::kK3Warps * sizeof(int32_t) * ((size_t)8 * d.capR + (size_t)3 * d.capW + 32) <= 200 * 1024;
     e = lr::set_k1_smem(c->k1_smem);
-    if (e == cudaSuccess && c->k3_smem <= 200 * 1024) e = lr::set_k3_smem(c->k3_smem);
+    if (e == cudaSuccess && c->k3_ok) e = lr::set_k3_smem(c->k3_smem);
     if (e == cudaSuccess && M <= lr::kCalMaxModels) e = lr::set_calib_smem(M);
     if (e == cudaSuccess) e = lr::set_k2_smem(std::max({c->est.smem, c->rt.ok ? c->rt.smem : 0, c->sw.ok ? c->sw.smem : 0}));
     c->bl_ok = lr::baseline_smem(d) <= 200 * 1024;
@@ -853,7 +857,7 @@ int lr_advance_tracked(lr_ctx *c, int32_t Q, const int32_t *assign, const int32_
     if (dec_cols != 1 && dec_cols != c->cfg.M) return fail(c, LR_EINVAL, "dec_cols must be 1 or num_models");
     if (!std::isfinite(t_now)) return fail(c, LR_EINVAL, "t_now must be finite");
     if (c->cfg.capR < c->max_seqs) return fail(c, LR_ECAPACITY, "advancing needs cap_running >= every max_seqs");
-    if ((c->kv_on ? c->k3_kv_smem : c->k3_smem) > 200 * 1024)
+    if (c->kv_on ? c->k3_kv_smem > 200 * 1024 : !c->k3_ok)
         return fail(c, LR_ECAPACITY, "queue capacities too large for one advance warp");
     lr::K3Launch k;
     std::memset(&k, 0, sizeof(k));

@@ -371,11 +371,10 @@ struct K3Launch {
     KvLimits kv;  // the KV stream step (launch_advance_kv) only
 };
 constexpr int kK3Warps = 4;
-// Shared memory of one K3 warp: the running list twice (ctx, pre, dec, id; the
-// batch's survivors are compacted into the other copy) and the waiting queue (pre,
-// dec, id).
+// Shared memory of one K3 warp: a window's ends by batch, the decoders (context and decode
+// offsets, id) and the waiting queue (prompt, decode, id); 16-byte aligned.
 __host__ __device__ inline size_t advance_smem_per_warp(const DevConfig &c) {
-    return sizeof(int32_t) * ((size_t)8 * c.capR + (size_t)3 * c.capW + 32);
+    return (sizeof(int32_t) * ((size_t)3 * c.capR + (size_t)3 * c.capW + 96) + 15) & ~(size_t)15;
 }
 // The KV stream step's waiting queue is a ring of capW + capR entries: preempted
 // requests return to its front.

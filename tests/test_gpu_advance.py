@@ -107,6 +107,43 @@ def test_advance_small_pools(mode):
 
 
 @pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("scale", [1.0, 0.13, 1e-13, 0.0])
+def test_decode_windows(mode, scale):
+    # long decode-only stretches, with requests ending inside them, seats that hold a queue
+    # back, clocks that pass powers of two and arrivals exactly at a batch's end; batch times
+    # down to ones that leave the clock's last bit (and to zero) take the one-batch path
+    I, cap = 13, 64
+    rng = np.random.default_rng(77)
+    wl = W.small_workload(5, num_instances=I, num_models=3, num_queries=8, cap_running=cap, cap_waiting=64,
+                          first_token_mode=mode, wait_max=20, budget_range=(64, 300), min_gap=8)
+    S = rng.integers(3, 50, I).astype(np.int32)
+    n_run = np.minimum(S, rng.integers(0, 50, I)).astype(np.int32)
+    col = np.arange(cap)[None, :] < n_run[:, None]
+    import dataclasses
+    wl = dataclasses.replace(
+        wl, max_seqs=S, n_run=n_run, run_pre=np.zeros((I, cap), np.int32),
+        run_ctx=np.where(col, rng.integers(0, 3000, (I, cap)), 0).astype(np.int32),
+        run_dec=np.where(col, rng.integers(1, 400, (I, cap)), 0).astype(np.int32), coef=(wl.coef * np.float32(scale)))
+    rt = make_router(wl)
+    N = 64
+    ftt = torch.full((N,), float("nan"), dtype=torch.float64, device="cuda")
+    rt.track_first_tokens(ftt)
+    track = oracle.new_track(wl, N)
+    clk = np.zeros(I)
+    for step, t_now in enumerate((0.011, 0.9, -1.0, 2.1, 65.0, 3e5)):
+        a = rng.integers(-1, I, 8).astype(np.int32)
+        p, d = rng.integers(1, 160, 8).astype(np.int32), rng.integers(1, 60, 8).astype(np.int32)
+        if t_now < 0:  # exactly where some instance's batch ends
+            t_now = float(np.median(oracle.advance(wl, clk, a, p, d, 1.5)[1]))
+        rt.advance(dev(a), dev(p), dev(d), t_now, id_base=8 * step)
+        wl, clk, track = oracle.advance(wl, clk, a, p, d, t_now, track=track, id_base=8 * step)
+        check_state(read(rt), wl, clk)
+        assert rt.status() == R().LR_OK, step
+        np.testing.assert_array_equal(ftt.cpu().numpy().view(np.uint64), track["first_token_time"].view(np.uint64))
+    rt.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
 def test_route_advance_loop_pool64(mode):
     # the online loop of Sec. 5: route a micro-batch on the live snapshot, append it
     # to the chosen instances, advance the pool; assignments and states stay identical
