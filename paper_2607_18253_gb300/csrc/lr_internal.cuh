@@ -125,12 +125,33 @@ __device__ __forceinline__ int32_t load_acquire(const int32_t *p) {
     return v;
 }
 
-// Publish a new live buffer (after a __threadfence of the writes that made it): the
-// index and its copies, which readers take with acquire loads.
-__device__ __forceinline__ void publish_live(DevCtl *ctl, int32_t v) {
-    atomicExch(&ctl->active, v);
-    for (int r = 0; r < kLiveReps; ++r)
-        asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(&ctl->live[r][0]), "r"(v) : "memory");
+// The end of a load's CTA (every thread calls it): the last CTA to finish publishes the
+// new live buffer if every instance succeeded -- the index and its copies, which readers
+// take with acquire loads -- and resets the load's control words.  One fence and one
+// atomic a CTA; the copies are stored by a warp, two a lane (one thread storing 64 words
+// between four atomics cost a load about a microsecond).
+__device__ __forceinline__ void finish_load(DevCtl *ctl, int dst, unsigned ctas) {
+    __shared__ int s_publish;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        int v = -1;
+        if (atomicAdd(&ctl->done_ctas, 1u) == ctas - 1) {
+            __threadfence();
+            if (*(volatile int32_t *)&ctl->load_err == 0) v = dst;
+            *(volatile int32_t *)&ctl->load_err = 0;
+            *(volatile uint32_t *)&ctl->done_ctas = 0u;
+        }
+        s_publish = v;
+    }
+    __syncthreads();
+    const int v = s_publish;
+    if (v >= 0 && threadIdx.x < 32) {
+        __threadfence();  // what this CTA's thread 0 acquired precedes the stores
+        if (threadIdx.x == 0) asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(&ctl->active), "r"(v) : "memory");
+        for (int r = threadIdx.x; r < kLiveReps; r += 32)
+            asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(&ctl->live[r][0]), "r"(v) : "memory");
+    }
 }
 
 // The live-buffer index from this CTA's copy, with acquire ordering.
@@ -148,10 +169,14 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+// Sum over the warp, modulo 2^64, on every lane: three reductions of 22-bit pieces (each
+// sum stays below 2^32) instead of five rounds of two shuffles and a 64-bit addition.
 __device__ __forceinline__ long long warp_sum64(long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    const unsigned long long u = (unsigned long long)v;
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)u & 0x3fffffu);
+    const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 22) & 0x3fffffu);
+    const unsigned s2 = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 44));
+    return (long long)(s0 + ((unsigned long long)s1 << 22) + ((unsigned long long)s2 << 44));
 }
 
 // Candidate-kernel tile block: everything one CTA of the candidate kernel needs about

@@ -66,16 +66,7 @@ __device__ __forceinline__ int warp_incl_sum32(int x, int lane) {
     }
     return x;
 }
-__device__ __forceinline__ long long warp_sum64(long long x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-    return x;
-}
-__device__ __forceinline__ int warp_sum32(int x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-    return x;
-}
+__device__ __forceinline__ int warp_sum32(int x) { return __reduce_add_sync(kFull, x); }
 
 // End calendar of the KV load: a decoder that ends in batch E (>= the current
 // batch G) waits in list E mod kKvCal if E < G + kKvCal, else in the overflow list,
@@ -934,19 +925,7 @@ __global__ void __launch_bounds__(kKvWarps * 32) k_kv_load(const KvLoad a) {
     const StateBuf out = dst ? a.buf1 : a.buf0;
     const size_t per_warp = kv_smem_per_warp(a.cfg, a.kv.hist) / sizeof(int32_t);
     if (j < a.cfg.I) kv_instance<MODE>(a, out, j, lane, kv_smem + wid * per_warp);
-    // the last CTA to finish publishes the new snapshot if every instance succeeded
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned prev = atomicAdd(&a.ctl->done_ctas, 1u);
-        if (prev == gridDim.x - 1) {
-            __threadfence();
-            const int err = atomicExch(&a.ctl->load_err, 0);
-            if (err == 0) publish_live(a.ctl, dst);
-            atomicExch(&a.ctl->done_ctas, 0u);
-            __threadfence();
-        }
-    }
+    finish_load(a.ctl, dst, gridDim.x);
 }
 
 constexpr float kNaN = __builtin_nanf("");
