@@ -440,6 +440,11 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         hp = wq[wh].x;
         hd = wq[wh].y;
     }
+    // Counts change by reductions that return nothing: a load, an addition and a store by one
+    // lane would hold the whole (in-order) warp for a shared-memory round trip.
+    auto hist_add = [&](int res, int d) {
+        if (lane == 0) asm volatile("red.shared.add.s32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(hist + res)), "r"(d) : "memory");
+    };
     // a decoder from batch G + 1 on, in slot s, with context ctx (of residue rem) and dec tokens to go
     auto decode_from_next = [&](int s, int ctx, int rem, int dec) {
         const int x = ctx - (G + 1), z = dec + (G + 1);
@@ -449,13 +454,15 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         const long long E = kv_end(q, mctx);
         const int ebv = dblk(dv, (int)(x + E + 1));
         int32_t *h = E < (long long)G + kKvCal ? &head[E & (kKvCal - 1)] : ovf;
+        const int hv = *h;
         if (lane == 0) {
             rq[s] = q;
             eb[s] = ebv;
-            nxt[s] = *h;
+            nxt[s] = hv;
             *h = s;
-            hist[res] += 1;
         }
+        hist_add(res, 1);
+        __syncwarp();  // the next filing of this batch reads the list's head
         src += x;
         ++nd;
     };
@@ -546,19 +553,25 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 ++nrec;
             };
             while (G < Gstop) {
-                const int need = hist[ridx];
+                int need = hist[ridx];
                 int s = head[G & (kKvCal - 1)];
                 int fa = fb - need;
-                if ((fa >= 0) & (fa < hm) & (s < 0)) {  // decoding only
+                // decoding only: the next batch's words are read while this one is judged
+                while (G < Gstop) {
+                    const int rn = ridx == 0 ? bs - 1 : ridx - 1;
+                    const int need_n = hist[rn], s_n = head[(G + 1) & (kKvCal - 1)];
+                    if (__any_sync(kFull, (fa < 0) | (fa >= hm) | (s >= 0))) break;
                     fb = fa;
                     r2 += nd;
                     r3 += t3;
                     t3 += nd;
                     if (la0 != 0) record(fa, fa, B - nd, B - nd);
                     ++G;
-                    ridx = ridx == 0 ? bs - 1 : ridx - 1;
-                    continue;
+                    ridx = rn;
+                    s = s_n;
+                    fa = fb - need_n;
                 }
+                if (G >= Gstop) break;
                 slack = nr > 0 ? fa : kHuge;
                 if (fa < 0) {
                     // preemption from the tail (see the general form)
@@ -576,8 +589,8 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                             hd = q.z - G;
                             acc += dblk(dv, hp + 1);
                             src -= q.x;
+                            hist_add(q.w, -1);
                             if (lane == 0) {
-                                hist[q.w] -= 1;
                                 wq[wh] = make_int2(hp, hd);
                                 reinterpret_cast<int *>(rq + r)[1] = -1;
                             }
@@ -610,15 +623,19 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                         int res = hrem + ridx - 1;  // xs mod bs
                         if (res < 0) res += bs;
                         if (res >= bs) res -= bs;
-                        const int ebv = dblk(dv, hfin), slot = ne++;
                         int32_t *h = hfin - hp < kKvCal ? &head[E & (kKvCal - 1)] : ovf;
+                        const int hv = *h;
+                        wh = wh + 1 == C ? 0 : wh + 1;
+                        const int2 wv = wq[wh];  // the next head
+                        const int ebv = dblk(dv, hfin), slot = ne++;
                         if (lane == 0) {
                             rq[slot] = make_int4(xs, 0, hd - (MODE == 1 ? 1 : 0) + (G + 1), res);
                             eb[slot] = ebv;
-                            nxt[slot] = *h;
+                            nxt[slot] = hv;
                             *h = slot;
-                            hist[res] += 1;
                         }
+                        hist_add(res, 1);
+                        __syncwarp();  // a further admission reads the list's head
                         tl = ne;
                         src += xs;
                         ++nd;
@@ -627,11 +644,9 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                         budget -= x;
                         f1 += x;
                         f4 += (long long)x * (x + 1) / 2;
-                        wh = wh + 1 == C ? 0 : wh + 1;
                         --wc;
-                        const int2 hv = wq[wh];
-                        hp = hv.x;
-                        hd = hv.y;
+                        hp = wv.x;
+                        hd = wv.y;
                         derive();
                     } while (budget > 0 && nr < S);
                 }
@@ -658,10 +673,8 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                             fb += ebs;
                             src -= q.x;
                             --nd;
-                            if (lane == 0) {
-                                hist[q.w] -= 1;
-                                reinterpret_cast<int *>(rq + s)[1] = -1;
-                            }
+                            hist_add(q.w, -1);
+                            if (lane == 0) reinterpret_cast<int *>(rq + s)[1] = -1;
                         }
                         s = ns;
                     } while (s >= 0);
@@ -738,7 +751,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                             --nd;
                             hp = q.x + G;
                             hd = q.z - G;
-                            if (lane == 0) hist[q.w] -= 1;
+                            hist_add(q.w, -1);
                         } else {
                             acc += dblk(dv, pC + px);
                             hp = pC + pP;
@@ -879,10 +892,8 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                     ++dying;
                     src -= q.x;
                     --nd;
-                    if (lane == 0) {
-                        hist[q.w] -= 1;
-                        reinterpret_cast<int *>(rq + s_end)[1] = -1;
-                    }
+                    hist_add(q.w, -1);
+                    if (lane == 0) reinterpret_cast<int *>(rq + s_end)[1] = -1;
                 }
                 s_end = ns;
             } while (s_end >= 0);
