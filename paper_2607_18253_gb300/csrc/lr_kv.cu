@@ -708,6 +708,75 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 continue;
             }
         }
+        // A prompt that outruns the free blocks: its first chunk takes a batch's whole budget,
+        // the next batch's chunk does not fit, so the request is preempted and, first in the
+        // queue again, admitted with the same chunk -- batch after batch, until enough blocks
+        // are free or a decoder ends.  Such a batch changes the free blocks alone, and costs
+        // the words of a batch without events (the general form took 1,200 cycles; on the
+        // 64-instance pool, where 8% of the prompts exceed the budget, half of the slowest
+        // instance's time: load 138 -> 80 us).
+        if (small && !scanned && pfs >= 0 && pC == B - nd && pP > 0) {
+            int F = (int)freeb + pH;                        // the blocks free without this request
+            const int more = dblk(dv, pC + min(pP, B - nd));  // what its second chunk would hold
+            int Gstop = min((G | (kKvCal - 1)) + 1, c.max_iters);
+            if (la0 != 0) Gstop = min(Gstop, G + (a.kv.horizon - nrec));
+            const int G0 = G;
+            long long t3 = src + (long long)nd * G, r3 = 0;
+            const long long tri = (long long)pC * (pC + 1) / 2;
+            int s = head[G & (kKvCal - 1)];
+            int F1 = F - hist[ridx];
+            while (G < Gstop) {
+                const int rn = ridx == 0 ? bs - 1 : ridx - 1;
+                const int need_n = hist[rn], s_n = head[(G + 1) & (kKvCal - 1)];
+                if (__any_sync(kFull, (F1 < pH) | (F1 >= more) | (s >= 0))) break;
+                F = F1;
+                r3 += t3;
+                if (la0 != 0) {
+                    if (lane == 0) {
+                        const long long k = G - G0 + 1;
+                        KvRec R;
+                        R.cf[0] = cf1 + k * pC;
+                        R.cf[1] = cf2 + k * nd;
+                        R.cf[2] = cf3 + r3;
+                        R.cf[3] = cf4 + k * tri;
+                        R.slack = -1;
+                        R.far = F;
+                        R.thr = 0;  // no budget is left
+                        R.bar = B - nd;
+                        R.bl = 0;
+                        rec[nrec] = R;
+                        pmxo[nrec] = pmx;
+                    }
+                    ++nrec;
+                }
+                t3 += nd;
+                ++G;
+                ridx = rn;
+                s = s_n;
+                F1 = F - need_n;
+            }
+            if (G != G0) {
+                const long long k = G - G0;
+                if (la0 != 0) {
+                    cf1 += k * pC;
+                    cf2 += k * nd;
+                    cf3 += r3;
+                    cf4 += k * tri;
+                    clear = 0;
+                } else {
+                    fcum[0] += k;
+                    fcum[1] += k * pC;
+                    fcum[2] += k * nd;
+                    fcum[3] += r3;
+                    fcum[4] += k * tri;
+                }
+                gr = ridx == 0 ? 0 : bs - ridx;
+                freeb = F - pH;
+                l = G + 1;
+                if (la0 != 0 && nrec == a.kv.horizon) break;
+                if (G >= Gstop) continue;
+            }
+        }
         // 1. The running scan.  n_run <= S <= B and only the last request may be in
         //    prefill, so every request gets its tokens if the blocks suffice: one per
         //    decoder, and the last one's chunk from what the decoders leave.

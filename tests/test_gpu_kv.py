@@ -231,6 +231,28 @@ def test_long_blocked_queues(mode, bs):
     check(wl, limits)
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("bs,slack", [(1, 50), (4, 12), (16, 3)])
+@pytest.mark.parametrize("queue", [1, 3])
+def test_prompt_outruns_the_blocks(mode, bs, slack, queue):
+    # the waiting head's first chunk is a whole batch's budget and fits, its second does not: it
+    # is preempted and admitted again in batch after batch while the decoders run on, with and
+    # without requests behind it (before the first record, and after it)
+    import dataclasses
+    wl = W.small_workload(95, num_instances=4, num_models=2, num_queries=40, first_token_mode=mode, cap_running=8,
+                          cap_waiting=8, max_prompt_len=70)
+    I = 4
+    rep = lambda v: np.tile(np.array(v, np.int32), (I, 1) if np.ndim(v) else I)  # noqa: E731
+    dec = rep([300, 280, 0, 0, 0, 0, 0, 0])
+    dec[1:, :2] -= np.array([[290, 0], [296, 275], [0, 274]], np.int32)
+    wl = dataclasses.replace(
+        wl, max_batched_tokens=rep(32), max_seqs=rep(8), n_run=rep(2), run_ctx=rep([600, 613, 0, 0, 0, 0, 0, 0]),
+        run_pre=rep([0] * 8), run_dec=dec, n_wait=rep(queue), wait_pre=rep([64, 50, 31, 0, 0, 0, 0, 0]),
+        wait_dec=rep([20, 9, 5, 0, 0, 0, 0, 0]))
+    nb = (-(-600 // bs) + -(-613 // bs) + slack + np.arange(I)).astype(np.int64)
+    check(wl, (rep(bs), nb, np.array([1 << 40] * I, np.int64)))
+
+
 @pytest.mark.parametrize("I,few", [(3, 31), (9, 33), (24, 1000)])
 def test_few_and_many_queries_agree(I, few):
     # a call of few queries walks each one directly; 20,000 queries are sorted by length and
