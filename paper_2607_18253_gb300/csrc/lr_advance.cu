@@ -751,6 +751,7 @@ __global__ void __launch_bounds__(kK3Warps * 32) k_advance(const K3Launch a) {
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     const int j = blockIdx.x * kK3Warps + wid;
+    chain_wait();
     const int active = *((volatile int32_t *)&a.ctl->active);
     if (j >= a.cfg.I) return;
     if (active < 0) {
@@ -762,6 +763,7 @@ __global__ void __launch_bounds__(kK3Warps * 32) k_advance(const K3Launch a) {
     const StateBuf idst = active ? a.buf0 : a.buf1;
     const size_t per_warp = advance_smem_per_warp(a.cfg) / sizeof(int32_t);
     advance_instance(a, src, idst, j, lane, k3_smem + wid * per_warp);
+    chain_next();
 }
 
 __global__ void __launch_bounds__(kK3Warps * 32) k_advance_kv(const K3Launch a) {
@@ -769,6 +771,7 @@ __global__ void __launch_bounds__(kK3Warps * 32) k_advance_kv(const K3Launch a) 
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     const int j = blockIdx.x * kK3Warps + wid;
+    chain_wait();
     const int active = *((volatile int32_t *)&a.ctl->active);
     if (j >= a.cfg.I) return;
     if (active < 0) {
@@ -780,12 +783,14 @@ __global__ void __launch_bounds__(kK3Warps * 32) k_advance_kv(const K3Launch a) 
     const StateBuf idst = active ? a.buf0 : a.buf1;
     const size_t per_warp = advance_kv_smem_per_warp(a.cfg) / sizeof(int32_t);
     advance_instance_kv(a, src, idst, j, lane, k3_smem + wid * per_warp);
+    chain_next();
 }
 
 // Copy of the live snapshot into caller arrays (the live buffer is known only on
 // the device).
 __global__ void k_read_state(const DevConfig c, const StateBuf b0, const StateBuf b1, const DevCtl *ctl,
                              const StateOut o) {
+    chain_wait();
     const int active = *((volatile const int32_t *)&ctl->active);
     const StateBuf s = active == 1 ? b1 : b0;
     const size_t R = (size_t)c.I * c.capR, W = (size_t)c.I * c.capW;
@@ -811,13 +816,11 @@ __global__ void k_read_state(const DevConfig c, const StateBuf b0, const StateBu
 
 cudaError_t launch_read_state(const DevConfig &c, const StateBuf &b0, const StateBuf &b1, DevCtl *ctl,
                               const StateOut &o, cudaStream_t st) {
-    k_read_state<<<128, 256, 0, st>>>(c, b0, b1, ctl, o);
-    return cudaGetLastError();
+    return launch_chained(k_read_state, 128, 256, 0, st, c, b0, b1, (const DevCtl *)ctl, o);
 }
 
 cudaError_t launch_advance(const K3Launch &a, int grid, size_t smem, cudaStream_t st) {
-    k_advance<<<grid, kK3Warps * 32, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_advance, grid, kK3Warps * 32, smem, st, a);
 }
 
 cudaError_t set_k3_smem(size_t bytes) {
@@ -825,8 +828,7 @@ cudaError_t set_k3_smem(size_t bytes) {
 }
 
 cudaError_t launch_advance_kv(const K3Launch &a, int grid, size_t smem, cudaStream_t st) {
-    k_advance_kv<<<grid, kK3Warps * 32, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_advance_kv, grid, kK3Warps * 32, smem, st, a);
 }
 
 cudaError_t set_k3_kv_smem(size_t bytes) {

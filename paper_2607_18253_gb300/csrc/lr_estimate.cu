@@ -423,13 +423,12 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
         for (int it = 0; it < (1 << 22) && !landed; ++it) landed = mbar_test(mbar);
         return landed;
     };
-    if (threadIdx.x == 0) {
-        if (!AFF) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        s_claim[0] = first_range(a);
+    if (threadIdx.x == 0 && !AFF) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    chain_wait();
+    if (threadIdx.x == 0) s_claim[0] = first_range(a);
     __syncthreads();
     const int2 first = s_claim[0];
     // the first chunk of query rows travels while the live index is read and the tile
@@ -958,6 +957,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
     else run(no, no, no, no);
     }
 finish:
+    chain_next();
     k2_finish(a, a.work, gridDim.x * gridDim.y, gridDim.y);
 }
 
@@ -972,6 +972,7 @@ constexpr int kFrontierThreads = 256;
 __global__ void __launch_bounds__(kFrontierThreads) k_frontier(const K2Launch a, double *out) {
     __shared__ double red[3][kFrontierThreads];
     __shared__ double part[8][3];  // rank 0: the ranks' sums
+    chain_wait();
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     cluster.sync();  // every CTA of the cluster runs before one writes into another's shared memory
     const int pp = blockIdx.y, cs = gridDim.x, rank = blockIdx.x;
@@ -1033,21 +1034,20 @@ __global__ void __launch_bounds__(kFrontierThreads) k_frontier(const K2Launch a,
 
 template <int MODE>
 cudaError_t launch_cand_mode(const K2Launch &a, int out, dim3 grid, int block, size_t smem, cudaStream_t st) {
+    auto go = [&](void (*k)(K2Launch)) { return launch_chained(k, grid, block, smem, st, a); };
     switch (out) {
-        case kOutMatrix: k_cand<MODE, kOutMatrix><<<grid, block, smem, st>>>(a); break;
+        case kOutMatrix: return go(k_cand<MODE, kOutMatrix>);
         case kOutMatrix | kOutIters:
             if (MODE == 2) return cudaErrorInvalidValue;  // the batch index exists only for SFS
-            k_cand<(MODE == 2 ? 0 : MODE), kOutMatrix | kOutIters><<<grid, block, smem, st>>>(a);
-            break;
-        case kOutLag: k_cand<MODE, kOutLag><<<grid, block, smem, st>>>(a); break;
-        case kOutLag | kOutMatrix: k_cand<MODE, kOutLag | kOutMatrix><<<grid, block, smem, st>>>(a); break;
-        case kOutCon: k_cand<MODE, kOutCon><<<grid, block, smem, st>>>(a); break;
-        case kOutCon | kOutMatrix: k_cand<MODE, kOutCon | kOutMatrix><<<grid, block, smem, st>>>(a); break;
-        case kOutSweep: k_cand<MODE, kOutSweep><<<grid, block, smem, st>>>(a); break;
-        case kOutSweep | kOutMatrix: k_cand<MODE, kOutSweep | kOutMatrix><<<grid, block, smem, st>>>(a); break;
+            return go(k_cand<(MODE == 2 ? 0 : MODE), kOutMatrix | kOutIters>);
+        case kOutLag: return go(k_cand<MODE, kOutLag>);
+        case kOutLag | kOutMatrix: return go(k_cand<MODE, kOutLag | kOutMatrix>);
+        case kOutCon: return go(k_cand<MODE, kOutCon>);
+        case kOutCon | kOutMatrix: return go(k_cand<MODE, kOutCon | kOutMatrix>);
+        case kOutSweep: return go(k_cand<MODE, kOutSweep>);
+        case kOutSweep | kOutMatrix: return go(k_cand<MODE, kOutSweep | kOutMatrix>);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template <typename F>
@@ -1136,6 +1136,7 @@ __global__ void __launch_bounds__(256) k_baseline(const K2Launch a, int policy, 
     extern __shared__ __align__(16) unsigned char bsm[];
     const DevConfig &c = a.cfg;
     const int I = c.I, M = c.M;
+    chain_wait();
     __shared__ int s_active;
     if (threadIdx.x == 0) s_active = load_live(a.ctl);
     __syncthreads();
@@ -1320,13 +1321,15 @@ cudaError_t launch_frontier(const K2Launch &a, double *out, int sms, cudaStream_
     cfg.gridDim = dim3(cs, a.P);
     cfg.blockDim = dim3(kFrontierThreads);
     cfg.stream = st;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cs;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cs;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_frontier, a, out);
 }
 
@@ -1339,9 +1342,7 @@ size_t baseline_smem(const DevConfig &c) {
 cudaError_t launch_baseline(const K2Launch &a, int policy, long long rr_start, float lam, int sms, cudaStream_t st) {
     const size_t smem = baseline_smem(a.cfg);
     const int grid = std::max(1, std::min((a.Q + 255) / 256, sms * 4));
-    if (a.cfg.mode == 0) k_baseline<0><<<grid, 256, smem, st>>>(a, policy, rr_start, lam);
-    else k_baseline<1><<<grid, 256, smem, st>>>(a, policy, rr_start, lam);
-    return cudaGetLastError();
+    return launch_chained(a.cfg.mode == 0 ? k_baseline<0> : k_baseline<1>, grid, 256, smem, st, a, policy, rr_start, lam);
 }
 
 cudaError_t launch_on_time(int Q, const float *util, const float *ttft, const float *tau, const float *delay,

@@ -998,6 +998,7 @@ __global__ void __launch_bounds__(kKvWarps * 32) k_kv_load(const KvLoad a) {
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     const int j = blockIdx.x * (int)(blockDim.x >> 5) + wid;
+    chain_wait();
     __shared__ int s_active;
     if (threadIdx.x == 0) s_active = load_acquire(&a.ctl->active);
     __syncthreads();
@@ -1207,6 +1208,8 @@ __device__ __forceinline__ int kv_bucket(int p, int pmax, int shift) {
 }
 
 __global__ void __launch_bounds__(256) k_kv_count(const int32_t *prompt, int Q, int pmax, int shift, int32_t *cnt) {
+    chain_wait();
+    chain_next();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x) {
         const int b = kv_bucket(prompt[i], pmax, shift);
         const unsigned m = __match_any_sync(__activemask(), b);
@@ -1225,6 +1228,8 @@ static_assert(kKvBuckets == kKvScanTiles * 4 * kScanThreads, "scan tiles cover t
 // the tiles before it.  (One CTA over every bucket was bound by one SM's bandwidth.)
 __global__ void __launch_bounds__(kScanThreads) k_kv_tile_sums(const int32_t *cnt, int32_t *tsum, int32_t *claim,
                                                                int groups) {
+    chain_wait();
+    chain_next();
     __shared__ int ws[2][kScanThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     if (blockIdx.x == 0)
@@ -1252,6 +1257,8 @@ __global__ void __launch_bounds__(kScanThreads) k_kv_scan(int32_t *cnt, int32_t 
                                                           int32_t *nu, const int32_t *tsum) {
     __shared__ int ws[2][kScanThreads / 32];
     __shared__ int base[2];
+    chain_wait();
+    chain_next();
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     if (tid == 0) {  // the tiles before this one
         int c = 0, u = 0;
@@ -1305,6 +1312,8 @@ __global__ void __launch_bounds__(kScanThreads) k_kv_scan(int32_t *cnt, int32_t 
 __global__ void __launch_bounds__(256) k_kv_scatter(const int32_t *prompt, int Q, int pmax, int shift, int32_t *run,
                                                     const int32_t *start, const int32_t *uid, int32_t *order,
                                                     int32_t *leaders) {
+    chain_wait();
+    chain_next();
     const int lane = threadIdx.x & 31;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x) {
         const int b = kv_bucket(prompt[i], pmax, shift);
@@ -1323,6 +1332,7 @@ __global__ void __launch_bounds__(256) k_kv_scatter(const int32_t *prompt, int Q
 // One warp per query row: a query that is not its bucket's leader copies the
 // leader's rows (times, and first batches and features if asked for).
 __global__ void __launch_bounds__(256) k_kv_expand(const KvEst a) {
+    chain_wait();
     const int I = a.cfg.I, lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
     const bool v4 = I % 4 == 0 && (reinterpret_cast<uintptr_t>(a.ttft) & 15) == 0;
@@ -1371,6 +1381,7 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
     // pool's models, whose walks differ in length, so the groups' work is alike
     const int gy = gridDim.y;
     const int ng = min(kEstGroup, (c.I - (int)blockIdx.y + gy - 1) / gy);
+    chain_wait();
     const int active = load_acquire(&a.ctl->active);
     // the group's views, a thread each
     if ((int)threadIdx.x < ng) {
@@ -1514,14 +1525,13 @@ __global__ void __launch_bounds__(kEstWarps * 32, 3) k_kv_estimate(const KvEst a
         i_cur = i_nx;
         p_cur = p_nx;
     }
+    chain_next();
 }
 
 }  // namespace
 
 cudaError_t launch_kv_load(const KvLoad &a, int grid, int warps, size_t smem, cudaStream_t st) {
-    if (a.cfg.mode == 0) k_kv_load<0><<<grid, warps * 32, smem, st>>>(a);
-    else k_kv_load<1><<<grid, warps * 32, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(a.cfg.mode == 0 ? k_kv_load<0> : k_kv_load<1>, grid, warps * 32, smem, st, a);
 }
 
 cudaError_t set_kv_smem(size_t bytes) {
@@ -1549,9 +1559,8 @@ cudaError_t launch_kv_estimate(const KvEst &a, int sms, cudaStream_t st) {
     const int qb = (a.Q + 31) / 32, wave = std::max(1, sms * 3 / gd);
     if (qb <= std::max(wave, std::min(32, 4 * wave))) {
         const dim3 grid(std::min(qb, wave), gd);
-        if (a.cfg.mode == 0) k_kv_estimate<0, true><<<grid, thr, EstShape<true>::kSmem, st>>>(a, false);
-        else k_kv_estimate<1, true><<<grid, thr, EstShape<true>::kSmem, st>>>(a, false);
-        return cudaGetLastError();
+        return launch_chained(a.cfg.mode == 0 ? k_kv_estimate<0, true> : k_kv_estimate<1, true>, grid, thr,
+                              EstShape<true>::kSmem, st, a, false);
     }
     const int gy = (a.cfg.I + EstShape<false>::kGroup - 1) / EstShape<false>::kGroup;
     const int blocks = (a.Q + 32 * kEstWarps - 1) / (32 * kEstWarps);
@@ -1562,15 +1571,21 @@ cudaError_t launch_kv_estimate(const KvEst &a, int sms, cudaStream_t st) {
     const int nbk = 2 + ((a.cfg.pmax - 1) >> shift);
     const bool exact = shift == 0;
     const int g1 = std::max(1, std::min((a.Q + 255) / 256, sms * 4));
-    k_kv_count<<<g1, 256, 0, st>>>(a.prompt, a.Q, a.cfg.pmax, shift, a.cnt);
     const int tiles = (nbk + 4095) / 4096;
-    k_kv_tile_sums<<<tiles, kScanThreads, 0, st>>>(a.cnt, a.tsum, a.claim, gy);
-    k_kv_scan<<<tiles, kScanThreads, 0, st>>>(a.cnt, a.start, a.run, a.uid, a.nu, a.tsum);
-    k_kv_scatter<<<g1, 256, 0, st>>>(a.prompt, a.Q, a.cfg.pmax, shift, a.run, a.start, a.uid, a.order, a.leaders);
-    if (a.cfg.mode == 0) k_kv_estimate<0, false><<<grid, thr, EstShape<false>::kSmem, st>>>(a, exact);
-    else k_kv_estimate<1, false><<<grid, thr, EstShape<false>::kSmem, st>>>(a, exact);
-    if (exact) k_kv_expand<<<std::max(1, std::min((a.Q + 7) / 8, sms * 8)), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = launch_chained(k_kv_count, g1, 256, 0, st, a.prompt, a.Q, a.cfg.pmax, shift, a.cnt);
+    if (e == cudaSuccess)
+        e = launch_chained(k_kv_tile_sums, tiles, kScanThreads, 0, st, (const int32_t *)a.cnt, a.tsum, a.claim, gy);
+    if (e == cudaSuccess)
+        e = launch_chained(k_kv_scan, tiles, kScanThreads, 0, st, a.cnt, a.start, a.run, a.uid, a.nu, (const int32_t *)a.tsum);
+    if (e == cudaSuccess)
+        e = launch_chained(k_kv_scatter, g1, 256, 0, st, a.prompt, a.Q, a.cfg.pmax, shift, a.run, (const int32_t *)a.start,
+                           (const int32_t *)a.uid, a.order, a.leaders);
+    if (e == cudaSuccess)
+        e = launch_chained(a.cfg.mode == 0 ? k_kv_estimate<0, false> : k_kv_estimate<1, false>, grid, thr,
+                           EstShape<false>::kSmem, st, a, exact);
+    if (e == cudaSuccess && exact)
+        e = launch_chained(k_kv_expand, std::max(1, std::min((a.Q + 7) / 8, sms * 8)), 256, 0, st, a);
+    return e;
 }
 
 }  // namespace lr

@@ -954,6 +954,7 @@ __global__ void __launch_bounds__(kK1Warps * 32) k_trajectory(const K1Launch a) 
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     const int j = blockIdx.x * kK1Warps + wid;
+    chain_wait();
     __shared__ int s_active;
     const size_t per_warp = trajectory_smem_per_warp(a.cfg) / sizeof(int32_t);
     int dst = 0;
@@ -995,9 +996,7 @@ cudaError_t launch_tile_pad(const DevConfig &c, unsigned char *tile, cudaStream_
 }
 
 cudaError_t launch_trajectory(const K1Launch &a, int grid, int block, size_t smem, cudaStream_t st) {
-    if (a.cfg.mode == 0) k_trajectory<0><<<grid, block, smem, st>>>(a);
-    else k_trajectory<1><<<grid, block, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(a.cfg.mode == 0 ? k_trajectory<0> : k_trajectory<1>, grid, block, smem, st, a);
 }
 
 cudaError_t set_k1_smem(size_t bytes) {
