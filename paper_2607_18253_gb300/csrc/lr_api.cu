@@ -34,7 +34,7 @@ struct lr_ctx {
     bool k3_ok = false;  // the queue capacities are within what lr_advance takes
     float *scratch_tch = nullptr;
     uint32_t *k2_work = nullptr;  // the candidate kernel's row counters
-    double *ontime_part = nullptr;  // per-CTA partial sums of lr_on_time_utility
+    double *ontime_part = nullptr;  // per-CTA partial sums of lr_on_time_utility, and their count
     bool bl_ok = false;             // the baseline policies' shared memory fits
     // stream of the last snapshot load (lr_load_state or lr_advance): a candidate-kernel
     // call on another stream may run beside it
@@ -363,7 +363,7 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     LR_ALLOC(c->ctl, 1);
     LR_ALLOC(c->scratch_tch, (size_t)cfg->max_pairs * cfg->max_queries);
     LR_ALLOC(c->k2_work, lr::k2_work_words(I));
-    LR_ALLOC(c->ontime_part, 2 * (size_t)lr::kOnTimeParts);
+    LR_ALLOC(c->ontime_part, 2 * (size_t)lr::kOnTimeParts + 1);  // and the CTA count (zero between calls)
     LR_ALLOC(c->qraw, I);
     LR_ALLOC(c->qd, I);
     LR_ALLOC(c->cal_acc, lr::cal_acc_words(M));
