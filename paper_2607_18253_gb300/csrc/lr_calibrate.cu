@@ -416,6 +416,7 @@ __global__ void __launch_bounds__(kCalThreads, 1) k_calibrate(long long N, const
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();  // the sums are zero and the barriers ready
+    chain_wait();
     if (TMA && c0 < c1) {
         // The last warp produces (its lane 0 issues each tile once the consumers have
         // released the stage), the others consume at their own pace: no CTA barrier in
@@ -498,6 +499,7 @@ __global__ void __launch_bounds__(kCalThreads, 1) k_calibrate(long long N, const
             const bool in = i < c1;
             row(in, true, in ? model[i] : 0, in ? time[i] : 0.0, F + (in ? i : 0) * kCalCols);
         }
+    chain_next();
     flush();
     if (__any_sync(kFull, bad) && lane == 0) record_status(ctl, kEInval);
     if (!ok && threadIdx.x == 0) record_status(ctl, kECuda);
@@ -569,13 +571,9 @@ cudaError_t launch_calibrate(long long N, const long long *F, const int32_t *mod
     const bool tma = ((uintptr_t)F | (uintptr_t)model | (uintptr_t)time) % 16 == 0;
     if (N <= 0) grid = 1;
     // the ring also holds the solve's scaled entries (kCalSolveWords doubles a model)
-    if (tma)
-        k_calibrate<true><<<grid, kCalThreads, fixed + kCalStageBytes * nst, st>>>(N, F, model, time, M, D, nst, acc,
-                                                                                  coef, ctl);
-    else
-        k_calibrate<false><<<grid, kCalThreads, fixed + solve_bytes(M), st>>>(N, F, model, time, M, D, nst, acc, coef,
-                                                                               ctl);
-    return cudaGetLastError();
+    return launch_chained(tma ? k_calibrate<true> : k_calibrate<false>, grid, kCalThreads,
+                          fixed + (tma ? kCalStageBytes * nst : solve_bytes(M)), st, N, F, model, time, M, D, nst, acc, coef,
+                          ctl);
 }
 
 cudaError_t set_calib_smem(int M) {

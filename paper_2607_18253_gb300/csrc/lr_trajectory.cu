@@ -214,6 +214,16 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
     // before any of them is used; the first block's loads go out before anything
     // waits on the counts, so that one memory round trip covers both.
     constexpr int kBlk = 8;  // entries per lane and block
+    // What lr_create set is read, and the calendar cleared, before the predecessor is done.
+    const int B = c.B[j];
+    const int S = c.S[j];
+    const int m_j = c.moi[j], sh = c.shift[j], nb = c.nb[j];
+    const float b0 = c.coef[m_j * 5 + 0], b1p = c.coef[m_j * 5 + 1], b1d = c.coef[m_j * 5 + 2],
+                b2 = c.coef[m_j * 5 + 3], b3 = c.coef[m_j * 5 + 4];
+    WarpSmem m = carve(wbase, c);
+    for (int i = lane; i < kCalendar / 4; i += 32) reinterpret_cast<int4 *>(m.cal)[i] = make_int4(0, 0, 0, 0);
+    for (int i = lane; i < kCalendar / 32; i += 32) m.bm[i] = 0u;
+    chain_wait();
     int xc[kBlk], xp[kBlk], xd[kBlk], yp[kBlk], yd[kBlk];
     auto load_block = [&](int base) {
 #pragma unroll
@@ -227,14 +237,8 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
         }
     };
     load_block(0);
-    const int B = c.B[j];
-    const int S = c.S[j];
     const int nr = a.in.n_run[j];
     const int nw = a.in.n_wait[j];
-    // used after the step loop, requested here so that no memory round trip is left there
-    const int m_j = c.moi[j], sh = c.shift[j], nb = c.nb[j];
-    const float b0 = c.coef[m_j * 5 + 0], b1p = c.coef[m_j * 5 + 1], b1d = c.coef[m_j * 5 + 2],
-                b2 = c.coef[m_j * 5 + 3], b3 = c.coef[m_j * 5 + 4];
     // one read of the live-buffer index per CTA (every thread reading the same word would
     // queue them all on one L2 line), behind the snapshot's loads
     if (threadIdx.x == 0) *s_active = load_acquire(&a.ctl->active);
@@ -247,10 +251,6 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
         out.n_wait[j] = nw;
         out.clock[j] = a.in.clock ? a.in.clock[j] : 0.0;
     }
-    WarpSmem m = carve(wbase, c);
-    // Clear the calendar.
-    for (int i = lane; i < kCalendar / 4; i += 32) reinterpret_cast<int4 *>(m.cal)[i] = make_int4(0, 0, 0, 0);
-    for (int i = lane; i < kCalendar / 32; i += 32) m.bm[i] = 0u;
     if (!(nr >= 0 && nr <= c.capR && nr <= S && nw >= 0 && nw <= c.capW)) {
         fail(a.ctl, kEState, lane);
         return;
@@ -954,7 +954,6 @@ __global__ void __launch_bounds__(kK1Warps * 32) k_trajectory(const K1Launch a) 
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     const int j = blockIdx.x * kK1Warps + wid;
-    chain_wait();
     __shared__ int s_active;
     const size_t per_warp = trajectory_smem_per_warp(a.cfg) / sizeof(int32_t);
     int dst = 0;
