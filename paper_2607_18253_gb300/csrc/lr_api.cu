@@ -473,8 +473,10 @@ int lr_load_state(lr_ctx *c, const lr_state_view *v, void *stream) {
     return LR_OK;
 }
 
+// `leaders` (KV limits only): null if every query's row is to be written; else set if only the
+// rows of the first query of each length were.
 static int estimate_common(lr_ctx *c, int32_t Q, const int32_t *p, float *ttft, int32_t *iters, int64_t *feat,
-                           void *stream) {
+                           void *stream, bool *leaders = nullptr) {
     if (!c) return LR_EINVAL;
     c->err.clear();
     if (Q < 0) return fail(c, LR_EINVAL, "Q < 0");
@@ -505,7 +507,9 @@ static int estimate_common(lr_ctx *c, int32_t Q, const int32_t *p, float *ttft, 
         k.nu = k.uid + lr::kKvBuckets;
         k.tsum = k.nu + 4;
         k.claim = k.tsum + 2 * lr::kKvScanTiles;
-        cudaError_t e = lr::launch_kv_estimate(k, c->sms, (cudaStream_t)stream);
+        bool lead = false;
+        cudaError_t e = lr::launch_kv_estimate(k, c->sms, leaders == nullptr, &lead, (cudaStream_t)stream);
+        if (leaders) *leaders = lead;
         return e == cudaSuccess ? LR_OK : cuda_fail(c, e, "KV estimate launch");
     }
     lr::K2Launch a = k2_base(c);
@@ -560,11 +564,14 @@ int lr_route(lr_ctx *c, int32_t Q, const int32_t *prompt_len, const int32_t *dec
     if (Q == 0) return LR_OK;
     if (!prompt_len || !dec_hat || !acc || !assign_out || !util_out) return fail(c, LR_EINVAL, "null array");
     float *kv_matrix = nullptr;
+    bool leaders = false;
     if (c->kv_on) {
         // KV limits: the estimate matrix first (into the caller's matrix if asked
-        // for, else library memory), then utility and argmax over it
+        // for, else library memory, where a row per distinct length will do), then
+        // utility and argmax over it
         kv_matrix = ttft_matrix_out ? ttft_matrix_out : c->kv_mat;
-        const int rc = estimate_common(c, Q, prompt_len, kv_matrix, nullptr, nullptr, stream);
+        const int rc = estimate_common(c, Q, prompt_len, kv_matrix, nullptr, nullptr, stream,
+                                       ttft_matrix_out ? nullptr : &leaders);
         if (rc != LR_OK) return rc;
     }
     lr::K2Launch a = k2_base(c);
@@ -585,6 +592,10 @@ int lr_route(lr_ctx *c, int32_t Q, const int32_t *prompt_len, const int32_t *dec
     if (kv_matrix) {
         a.src = lr::kSrcMatrix;
         a.ttft_in = kv_matrix;
+        if (leaders) {
+            a.lead_start = c->kv_sort + lr::kKvBuckets;
+            a.lead_order = c->kv_order;
+        }
     }
     const lr_ctx::Shape &sh = P > 1 ? c->sw : c->rt;
     if (!sh.ok) return fail(c, LR_ECAPACITY, "routing needs num_instances <= 1024 and its tiles in shared memory");

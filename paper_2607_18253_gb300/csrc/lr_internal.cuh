@@ -317,7 +317,9 @@ struct KvEst {
 };
 constexpr int kKvBuckets = 1 << 16;
 constexpr int kKvScanTiles = kKvBuckets / 4096;  // the bucket scan's tiles, one CTA each
-cudaError_t launch_kv_estimate(const KvEst &a, int sms, cudaStream_t st);
+// expand: every query's row is written; else, when the call is sorted (*leaders set), only the
+// row of the first query of each length, order[start[p]]
+cudaError_t launch_kv_estimate(const KvEst &a, int sms, bool expand, bool *leaders, cudaStream_t st);
 
 // Batches covered by K1's completion calendar; decoders ending later are
 // tracked by scanning the decoder list.
@@ -378,6 +380,9 @@ struct K2Launch {
     int32_t src;
     const QueueDev *qd;
     const float *ttft_in;  // kSrcMatrix: [Q][I]
+    // kSrcMatrix, or null: the row of a query of p tokens is lead_order[lead_start[p]] (0 for an
+    // invalid length), not its own
+    const int32_t *lead_start, *lead_order;
     // [0]: CTAs finished; [1 + tile]: query rows of the tile claimed past the static
     // ones.  Zero before a launch; the last CTA to finish clears them for the next.
     uint32_t *work;

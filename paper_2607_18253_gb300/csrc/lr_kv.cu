@@ -24,7 +24,8 @@
 // readmissions, to its first token.  A candidate depends only on the instance and
 // the prompt length, so each call first counting-sorts its queries by length
 // (k_kv_count, k_kv_scan, k_kv_scatter), walks once per distinct length, and
-// copies those rows to the other queries of the same length (k_kv_expand).  A call of few
+// copies those rows to the other queries of the same length (k_kv_expand; a route that
+// returns no matrix reads the first query's row instead).  A call of few
 // queries walks each of them directly instead, in the one launch.
 #include "lr_internal.cuh"
 
@@ -1185,8 +1186,12 @@ __device__ int kv_candidate(const KvView &v, const KvStage &st, const KvTile &tl
     const int tc = min(t, v.nrec - 1);
     long long cf[4] = {0, 0, 0, 0};
     if (tc >= 0) {
-        const KvRec *r = v.rec + tc;
-        for (int k = 0; k < 4; ++k) cf[k] = __ldg(&r->cf[k]);
+        const longlong2 *r = reinterpret_cast<const longlong2 *>(v.rec[tc].cf);
+        const longlong2 x = __ldg(r), y = __ldg(r + 1);
+        cf[0] = x.x;
+        cf[1] = x.y;
+        cf[2] = y.x;
+        cf[3] = y.y;
     }
     F[0] = v.fcum[0] + t + 1;
     F[1] = v.fcum[1] + cf[0] + w.lost1 + p;
@@ -1547,7 +1552,8 @@ cudaError_t set_kv_smem(size_t bytes) {
     return e;
 }
 
-cudaError_t launch_kv_estimate(const KvEst &a, int sms, cudaStream_t st) {
+cudaError_t launch_kv_estimate(const KvEst &a, int sms, bool expand, bool *leaders, cudaStream_t st) {
+    *leaders = false;
     constexpr int thr = kEstWarps * 32;
     // Few queries are walked directly, in one launch.  The sort by prompt length, the walks
     // of distinct lengths alone and the copies of their rows pay for their five further
@@ -1583,7 +1589,8 @@ cudaError_t launch_kv_estimate(const KvEst &a, int sms, cudaStream_t st) {
     if (e == cudaSuccess)
         e = launch_chained(a.cfg.mode == 0 ? k_kv_estimate<0, false> : k_kv_estimate<1, false>, grid, thr,
                            EstShape<false>::kSmem, st, a, exact);
-    if (e == cudaSuccess && exact)
+    *leaders = exact && !expand;
+    if (e == cudaSuccess && exact && expand)
         e = launch_chained(k_kv_expand, std::max(1, std::min((a.Q + 7) / 8, sms * 8)), 256, 0, st, a);
     return e;
 }
