@@ -421,18 +421,15 @@ __device__ void advance_instance(const K3Launch &a, const StateBuf &src, const S
 // ---- The stream step under KV-cache limits (App. F: KV-cache allocation, context
 // limits and preemption; the same step rule as the KV estimate) ----
 //
-// One warp per instance, every batch planned in two warp passes: the running list in
-// order (each request's tokens within the budget, its new blocks, the blocks it holds),
-// then FCFS admission from the waiting head while the budget, a seat and the first
-// chunk's blocks allow.  When the running scan's new blocks exceed the free ones, lane
-// 0 replays the scan request by request, preempting the last running request (possibly
-// the one being served) until each finds its blocks; that case is rare and keeps the
-// exact order of the rule.  A preempted request returns its blocks, its whole context
-// becomes prefill again and it goes to the front of the waiting ring, in running order.
-// A request whose context reaches the limit ends.  Each batch takes the Eq. 9 time of
-// its own composition in the estimator's fp32 order, and runs only if it ends by t_now.
-
-__device__ __forceinline__ int kv_blk(int c, int bs) { return (int)(((unsigned)c + (unsigned)bs - 1u) / (unsigned)bs); }
+// One warp per instance, as above: the decoders are held by offsets, the prefill request in
+// registers, the waiting queue in a ring to whose front preempted requests return.  The
+// free blocks are a running total; a batch needs a block for each decoder whose context is
+// a multiple of the block size.  If they do not suffice, requests leave from the list's
+// tail until what the leavers would hold after the batch reaches the excess (which leaves
+// the longest prefix of the list that fits, as serving it in order does); their whole
+// context becomes prefill again.  A request whose context reaches the limit ends.  Each
+// batch takes the Eq. 9 time of its own composition in the estimator's fp32 order, and runs
+// only if it ends by t_now: a plan touches no state but free ring slots until then.
 
 __device__ void advance_instance_kv(const K3Launch &a, const StateBuf &src, const StateBuf &idst, int j, int lane,
                                     int32_t *wbase) {
@@ -444,20 +441,43 @@ __device__ void advance_instance_kv(const K3Launch &a, const StateBuf &src, cons
     const long long nbk = a.kv.nb[j], mctx = a.kv.mctx[j];
     const int capR = c.capR, capW = c.capW;
     const int Wc = capW + capR;  // the waiting ring
-    int32_t *rc0 = wbase, *rp0 = rc0 + capR, *rd0 = rp0 + capR;
-    int32_t *rc1 = rd0 + capR, *rp1 = rc1 + capR, *rd1 = rp1 + capR;
-    int32_t *ri0 = rd1 + capR, *ri1 = ri0 + capR;
-    int32_t *wp = ri1 + capR, *wd = wp + Wc, *wi = wd + Wc;
+    const Div32 dv = make_div32(bs);
+    long long *wsx = reinterpret_cast<long long *>(wbase);  // [32] a window's ends: offsets summed,
+    int32_t *wcnt = wbase + 64, *weblk = wcnt + 32;         // [32] counted, and their blocks;
+    int32_t *wneed = weblk + 32;                            // [32] and the blocks its batches need
+    int32_t *rx = wneed + 32, *rz = rx + capR, *ri = rz + capR;  // decoders: context - G, decode + G, id
+    int32_t *wp = ri + capR, *wd = wp + Wc, *wi = wd + Wc;
     const bool track = a.track != 0;
     const size_t rrow = (size_t)j * capR, wrow = (size_t)j * capW;
-    int nr = src.n_run[j];
+    const int nr0 = src.n_run[j];
     int nw = src.n_wait[j];
-    for (int t = lane; t < nr; t += 32) {
-        rc0[t] = src.run_ctx[rrow + t];
-        rp0[t] = src.run_pre[rrow + t];
-        rd0[t] = src.run_dec[rrow + t];
-        ri0[t] = track ? src.run_id[rrow + t] : -1;
+    // the request in prefill, if any, is the last running one
+    int pP = 0, pC = 0, pD = 0, pI = -1;
+    if (nr0 > 0) {
+        pP = src.run_pre[rrow + nr0 - 1];
+        pC = src.run_ctx[rrow + nr0 - 1];
+        pD = src.run_dec[rrow + nr0 - 1];
+        if (track) pI = src.run_id[rrow + nr0 - 1];
     }
+    bool pf = pP > 0;
+    int nd = nr0 - (pf ? 1 : 0);  // decoders
+    // a decoder's last batch: its decode count or the context limit
+    auto last_batch = [&](int x, int z) { return (int)min((long long)z - 1, mctx - 1 - x); };
+    long long csx = 0, freeb = 0;  // the decoders' context offsets summed; free blocks
+    int emin = kBig;               // the first last batch
+    for (int t = lane; t < nd; t += 32) {
+        const int x = src.run_ctx[rrow + t], z = src.run_dec[rrow + t];
+        rx[t] = x;
+        rz[t] = z;
+        ri[t] = track ? src.run_id[rrow + t] : -1;
+        csx += x;
+        freeb -= dblk(dv, x);
+        emin = min(emin, last_batch(x, z));
+    }
+    csx = warp_sum64(csx);
+    int pH = pf ? dblk(dv, pC) : 0;  // the prefill request's blocks
+    freeb = nbk + warp_sum64(freeb) - pH;
+    emin = __reduce_min_sync(kFull, emin);
     for (int t = lane; t < nw; t += 32) {
         wp[t] = src.wait_pre[wrow + t];
         wd[t] = src.wait_dec[wrow + t];
@@ -497,226 +517,286 @@ __device__ void advance_instance_kv(const K3Launch &a, const StateBuf &src, cons
     __syncwarp();
 
     const float *cf = c.coef + 5 * c.moi[j];
-    const float b0 = cf[0], b1p = cf[1], b1d = cf[2], b2 = cf[3], b3 = cf[4];
+    const BatchTime bt = {cf[0], cf[1], cf[2], cf[3], cf[4]};
     double t = src.clock[j];
     int wh = 0, iters = 0;  // the waiting ring holds nw requests from wh on
+    int G = 0, fresh = 0;   // batches executed; decoders from `fresh` on may owe their first token's time
     int err = kOk;
-    int32_t *rc = rc0, *rp = rp0, *rd = rd0, *ri = ri0, *nc = rc1, *np = rp1, *nd = rd1, *ni = ri1;
+    const int off = c.mode == 1 ? 1 : 0;  // the first token comes with the last chunk
+    auto emit_fresh = [&](double t_end) {
+        if (!track) return;
+        if (c.mode == 0)
+            for (int r = fresh + lane; r < nd; r += 32) ri[r] = emit_first(a, ri[r], true, t_end);
+        __syncwarp();
+        fresh = nd;
+    };
+    // the decoders whose last batch is g or before leave, in place; returns the blocks they held
+    auto drop_ended = [&](int g) -> long long {
+        int kept = 0, em = kBig;
+        long long cs = 0, back = 0;
+        for (int base = 0; base < nd; base += 32) {
+            const int r = base + lane;
+            const bool live = r < nd;
+            const int x = live ? rx[r] : 0, z = live ? rz[r] : 0, id = live ? ri[r] : -1;
+            const int E = live ? last_batch(x, z) : -1;
+            const bool keep = live && E > g;
+            const unsigned bal = __ballot_sync(kFull, keep);
+            __syncwarp();
+            if (keep) {
+                const int pos = kept + __popc(bal & lanemask_lt());
+                rx[pos] = x;
+                rz[pos] = z;
+                ri[pos] = id;
+                cs += x;
+                em = min(em, E);
+            } else if (live) {
+                back += dblk(dv, x + E + 1);
+            }
+            kept += __popc(bal);
+        }
+        nd = kept;
+        csx = warp_sum64(cs);
+        emin = __reduce_min_sync(kFull, em);
+        fresh = min(fresh, nd);
+        __syncwarp();
+        return warp_sum64(back);
+    };
     while (true) {
-        if (nr == 0 && nw == 0) {  // nothing to run: idle until t_now (never backwards)
+        if (nd == 0 && !pf && nw == 0) {  // nothing to run: idle until t_now (never backwards)
             t = fmax(t, a.t_now);
             break;
         }
-        if (++iters > c.max_iters) {
+        if (iters >= c.max_iters) {
             err = kETraj;
             break;
         }
-        // 1. the running scan: each request's tokens within the budget (a prefix of the
-        //    list is served), the new blocks they need and the blocks every request holds
-        long long used = 0, held = 0, nblk = 0;
-        long long f1 = 0, f2 = 0, f3 = 0, f4 = 0;
-        int rend = 0;
-        for (int base = 0; base < nr; base += 32) {
-            const int r = base + lane;
-            const bool live = r < nr;
-            const int ctx = live ? rc[r] : 0, pre = live ? rp[r] : 0;
-            const int need = live ? (pre > 0 ? pre : 1) : 0;
-            const long long incl = used + warp_incl_sum64(need, lane);
-            const long long x = live ? max(0LL, min((long long)need, (long long)B - (incl - need))) : 0;
-            if (live) held += kv_blk(ctx, bs);
-            if (x > 0) {
-                nblk += kv_blk(ctx + (int)x, bs) - kv_blk(ctx, bs);
-                if (pre > 0) {
-                    f1 += x;
-                    f4 += x * ctx + x * (x + 1) / 2;
-                } else {
-                    f2 += 1;
-                    f3 += ctx;
+        // 1. the running scan: every decoder one token, the prefill request its chunk
+        int need_d = 0;
+        for (int r = lane; r < nd; r += 32) need_d += dres(dv, rx[r] + G) == 0 ? 1 : 0;
+        need_d = __reduce_add_sync(kFull, need_d);
+        const int hp = nw > 0 ? wp[wh] : 0;
+        if (!pf && nd > 0 && need_d <= freeb &&
+            (nw == 0 || nd >= S || B <= nd || dblk(dv, min(hp, B - nd)) > freeb - need_d)) {
+            // Only decoding: up to 32 batches, lane k taking batch G + k, as in the plain step.
+            // Batch k runs if the blocks suffice -- those its decoders need, and those the
+            // window's ends return, are counted by batch -- and the head, if one waits, still
+            // cannot be admitted.  With the list held by offsets, 16-query micro-batches on 64
+            // instances: kernel 42 -> 32 us.
+            wsx[lane] = 0;
+            wcnt[lane] = weblk[lane] = wneed[lane] = 0;
+            __syncwarp();
+            for (int r = lane; r < nd; r += 32) {
+                const int x = rx[r];
+                const int e = last_batch(x, rz[r]) - G;  // its last batch of the window
+                const int g = dres(dv, x + G);
+                for (int k = g == 0 ? 0 : bs - g; k < 32 && k <= e; k += bs) atomicAdd(&wneed[k], 1);
+                if (e < 32) {
+                    atomicAdd(&wcnt[e], 1);
+                    atomicAdd(reinterpret_cast<unsigned long long *>(&wsx[e]), (unsigned long long)(long long)x);
+                    atomicAdd(&weblk[e], dblk(dv, x + G + e + 1));
                 }
             }
-            rend += __popc(__ballot_sync(kFull, x > 0));
-            used = __shfl_sync(kFull, incl, 31);
+            __syncwarp();
+            const int cnt = wcnt[lane], eb = weblk[lane], need = wneed[lane];
+            const long long sx = wsx[lane];
+            __syncwarp();  // read before the next window clears them
+            const int ndk = nd - (warp_incl_sum32(cnt, lane) - cnt);
+            const long long csk = csx - (warp_incl_sum64(sx, lane) - sx);
+            const long long gain = warp_incl_sum64((long long)eb - need, lane);  // through batch k
+            const long long fb = freeb + gain - eb;                              // after its scan
+            const float T = bt(0, ndk, csk + (long long)ndk * (G + lane), 0);
+            const ClockScan cs = clock_scan(t, T, lane);
+            const double te = cs.time();
+            const bool blocked = nw == 0 || ndk >= S || B <= ndk || dblk(dv, min(hp, B - ndk)) > fb;
+            const int W = min(32, c.max_iters - iters);
+            const unsigned in = W == 32 ? kFull : (1u << W) - 1u;
+            const unsigned bad = ~__ballot_sync(kFull, ndk > 0 && fb >= 0 && blocked);
+            const unsigned can = (bad ? (1u << (__ffs(bad) - 1)) - 1u : kFull) & in;  // (lane 0 always)
+            const unsigned run = __ballot_sync(kFull, te <= a.t_now) & can & cs.exact;
+            const int n = run == kFull ? 32 : __ffs(~run) - 1;
+            double t_first;
+            int done = n;
+            if (n > 0) {
+                t_first = __shfl_sync(kFull, te, 0);
+                t = __shfl_sync(kFull, te, n - 1);
+            } else if (!(cs.exact & 1u)) {
+                const double t1 = t + (double)__shfl_sync(kFull, T, 0);
+                if (t1 > a.t_now) break;  // still running at t_now
+                t = t_first = t1;
+                done = 1;
+            } else {
+                break;  // the next batch would end after t_now
+            }
+            emit_fresh(t_first);
+            freeb += __shfl_sync(kFull, gain, done - 1);  // less what the batches needed, and the ends' blocks
+            iters += done;
+            G += done;
+            if (emin < G) drop_ended(G - 1);
+            // an admissible exact batch that does not end by t_now ends the step
+            if (n > 0 && n < 32 && ((can & cs.exact) >> n & 1u)) break;
+            continue;
         }
-        held = warp_sum64(held);
-        nblk = warp_sum64(nblk);
-        long long freeb = nbk - held;
-        long long budget = max(0LL, (long long)B - used);
-        int pnr = nr;  // running requests left after preemptions
-        if (nblk > freeb) {
-            // Not every served request finds its blocks: lane 0 replays the scan in the
-            // rule's order, preempting from the tail, and the served prefix's features
-            // are summed again.
-            long long pf = freeb, bud = B;
-            int r = 0, n = nr;
-            if (lane == 0) {
-                while (r < n && bud > 0) {
-                    const long long x = rp[r] > 0 ? min((long long)rp[r], bud) : 1LL;
-                    const int nb1 = kv_blk(rc[r] + (int)x, bs) - kv_blk(rc[r], bs);
-                    while (pf < nb1 && n - 1 >= r) {
-                        --n;
-                        pf += kv_blk(rc[n], bs);
-                    }
-                    if (r >= n) break;  // r preempted itself
-                    pf -= nb1;
-                    bud -= x;
-                    ++r;
-                }
+        ++iters;
+        const int px = pf ? min(pP, B - nd) : 0;
+        const int pnew = pf ? dblk(dv, pC + px) : 0;
+        const int need_all = need_d + (pnew - pH);
+        // the plan: what the batch would leave of the list and of the blocks
+        int pnd = nd, kq = 0;  // decoders left, requests preempted
+        bool ppf = pf;
+        long long pcsx = csx, fb = freeb - need_all;
+        if (fb < 0) {
+            long long acc = 0;  // post-batch blocks of those gone
+            const long long excess = -fb;
+            if (pf) {
+                acc = pnew;
+                ppf = false;
+                kq = 1;
             }
-            rend = __shfl_sync(kFull, r, 0);
-            pnr = __shfl_sync(kFull, n, 0);
-            freeb = __shfl_sync(kFull, pf, 0);
-            budget = __shfl_sync(kFull, bud, 0);
-            f1 = f2 = f3 = f4 = 0;
-            used = 0;
-            for (int base = 0; base < rend; base += 32) {
-                const int r2 = base + lane;
-                const bool live = r2 < rend;
-                const int ctx = live ? rc[r2] : 0, pre = live ? rp[r2] : 0;
-                const int need = live ? (pre > 0 ? pre : 1) : 0;
-                const long long incl = used + warp_incl_sum64(need, lane);
-                const long long x = live ? max(0LL, min((long long)need, (long long)B - (incl - need))) : 0;
-                if (x > 0) {
-                    if (pre > 0) {
-                        f1 += x;
-                        f4 += x * ctx + x * (x + 1) / 2;
-                    } else {
-                        f2 += 1;
-                        f3 += ctx;
-                    }
-                }
-                used = __shfl_sync(kFull, incl, 31);
+            while (acc < excess && pnd > 0) {
+                const int x = rx[--pnd];
+                acc += dblk(dv, x + G + 1);
+                pcsx -= x;
+                ++kq;
             }
-        } else {
-            freeb -= nblk;
+            fb = acc - excess;
         }
-        // the preempted tail [pnr, nr) goes to the ring's front in running order, its
-        // whole context prefill again (the slots before the head are free; the head
-        // moves only if the batch runs)
-        const int k = nr - pnr;
-        int wh2 = wh - k;
+        int wh2 = wh - kq;
         if (wh2 < 0) wh2 += Wc;
-        for (int i = lane; i < k; i += 32) {
+        // (in running order, before the head: decoders, then the prefill request)
+        for (int i = lane; i < nd - pnd; i += 32) {
             int pos = wh2 + i;
             if (pos >= Wc) pos -= Wc;
-            wp[pos] = rc[pnr + i] + rp[pnr + i];
-            wd[pos] = rd[pnr + i];
-            wi[pos] = ri[pnr + i];
+            wp[pos] = rx[pnd + i] + G;
+            wd[pos] = rz[pnd + i] - G;
+            wi[pos] = ri[pnd + i];
+        }
+        if (pf && !ppf && lane == 0) {
+            int pos = wh2 + kq - 1;
+            if (pos >= Wc) pos -= Wc;
+            wp[pos] = pC + pP;
+            wd[pos] = pD;
+            wi[pos] = pI;
         }
         __syncwarp();
-        const int nw2 = nw + k;
-        // 2. admission from the ring's head while the budget, a seat and the first
-        //    chunk's blocks allow (each condition holds for a prefix of the queue)
-        int na = 0;
-        long long wused = 0, bused = 0;
+        const int nw2 = nw + kq, qx = ppf ? px : 0;
+        const int pnr = pnd + (ppf ? 1 : 0);
+        const int budget = B - pnd - qx;
+        long long f1 = qx, f4 = (long long)qx * pC + (long long)qx * (qx + 1) / 2;
+        const long long f3 = pcsx + (long long)pnd * G;
+        // 2. admission from the ring's head while the budget, a seat and the first chunk's
+        //    blocks allow (each condition holds for a prefix of the queue)
+        int na = 0, wused = 0;
+        long long bused = 0, ablk = 0;  // blocks up to the round; of the admitted
         for (int base = 0; budget - wused > 0 && base < nw2 && pnr + base < S; base += 32) {
             const int q = base + lane;
             int pos = wh2 + q;
             if (pos >= Wc) pos -= Wc;
             const bool in = q < nw2 && pnr + q < S;
             const int p = in ? wp[pos] : 0;
+            // (a preempted context can reach 2^28 tokens)
             const long long incl = wused + warp_incl_sum64(p, lane);
             const long long st = incl - p;
             const bool cand = in && st < budget;
             const long long x = cand ? min((long long)p, budget - st) : 0;
-            const int nb1 = cand ? kv_blk((int)x, bs) : 0;
+            const int nb1 = cand ? dblk(dv, (int)x) : 0;
             const long long binc = bused + warp_incl_sum64(nb1, lane);
-            const bool adm = cand && binc <= freeb;
-            if (adm) {
-                f1 += x;
-                f4 += x * (x + 1) / 2;
-            }
+            const bool adm = cand && binc <= fb;
+            f1 += warp_sum64(adm ? x : 0);
+            f4 += warp_sum64(adm ? x * (x + 1) / 2 : 0);
+            ablk += warp_sum64(adm ? (long long)nb1 : 0);
             const int nadm = __popc(__ballot_sync(kFull, adm));
             na += nadm;
-            wused = __shfl_sync(kFull, incl, 31);
-            bused = __shfl_sync(kFull, binc, 31);
             if (nadm < 32) break;
+            wused = (int)__shfl_sync(kFull, incl, 31);  // all admitted: below the budget, or the last
+            bused = __shfl_sync(kFull, binc, 31);
         }
-        f1 = warp_sum64(f1);
-        f2 = warp_sum64(f2);
-        f3 = warp_sum64(f3);
-        f4 = warp_sum64(f4);
-        // Eq. 9 for this batch, in the estimator's fp32 order
-        float T = __fmul_rn(b0, 1.0f);
-        T = __fmaf_rn(b1d, __ll2float_rn(f2), T);
-        T = __fmaf_rn(b1p, __ll2float_rn(f1), T);
-        T = __fmaf_rn(b2, __ll2float_rn(f3), T);
-        T = __fmaf_rn(b3, __ll2float_rn(f4), T);
-        if (t + (double)T > a.t_now) break;  // still running at t_now
+        const float T = bt(f1, pnd, f3, f4);
+        const double t1 = t + (double)T;
+        if (t1 > a.t_now) break;  // still running at t_now
         if (pnr + na > capR) {
             err = kETraj;
             break;
         }
-        // 3. execute it: the served prefix and the admitted requests advance; a request
-        //    with no decode token left, or whose context reached the limit, ends
-        int kept = 0;
-        long long rused = 0, wst = 0;
-        const int total = pnr + na;
-        for (int base = 0; base < total; base += 32) {
-            const int r = base + lane;
-            const bool isr = r < pnr, isw = r >= pnr && r < total;
-            int ctx = 0, pre = 0, dec = 0, id = -1;
-            if (isr) {
-                ctx = rc[r];
-                pre = rp[r];
-                dec = rd[r];
-                id = ri[r];
-            } else if (isw) {
-                int pos = wh2 + (r - pnr);
-                if (pos >= Wc) pos -= Wc;
-                pre = wp[pos];
-                dec = wd[pos];
-                id = wi[pos];
-            }
-            const long long inr = isr ? (pre > 0 ? pre : 1) : 0;
-            const long long incl_r = rused + warp_incl_sum64(inr, lane);
-            const long long inw = isw ? pre : 0;
-            const long long incl_w = wst + warp_incl_sum64(inw, lane);
-            long long x = 0;
-            if (isr && r < rend) x = max(0LL, min(inr, (long long)B - (incl_r - inr)));
-            if (isw) x = min(inw, budget - (incl_w - inw));
-            if (x > 0) {
-                if (pre > 0) {
-                    ctx += (int)x;
-                    pre -= (int)x;
-                    if (pre == 0 && c.mode == 1) {
-                        dec -= 1;  // first token with the last chunk
-                        if (track) id = emit_first(a, id, true, t + (double)T);
+        // 3. execute it: a request with no decode token left, or whose context reached the
+        //    limit, ends
+        nd = pnd;
+        csx = pcsx;
+        pf = ppf;
+        fresh = min(fresh, nd);
+        freeb = fb - ablk;
+        emit_fresh(t1);
+        t = t1;
+        if (emin <= G || kq > 0) freeb += drop_ended(G);
+        if (pf) {
+            pC += px;
+            pP -= px;
+            pH = pnew;
+            if (pP == 0) {
+                pf = false;
+                const int dec = pD - off;
+                if (track && off) pI = lane == 0 ? emit_first(a, pI, true, t1) : -1;
+                if (dec > 0 && (long long)pC < mctx) {
+                    const int x = pC - (G + 1), z = dec + (G + 1);
+                    if (lane == 0) {
+                        rx[nd] = x;
+                        rz[nd] = z;
+                        ri[nd] = pI;
                     }
+                    csx += x;
+                    emin = min(emin, last_batch(x, z));
+                    ++nd;
                 } else {
-                    ctx += 1;
-                    dec -= 1;
-                    if (track) id = emit_first(a, id, c.mode == 0, t + (double)T);
+                    freeb += pH;
                 }
+                pH = 0;
             }
-            if (pre == 0 && (long long)ctx >= mctx) dec = 0;  // the context limit
-            const bool keep = (isr || isw) && dec > 0;
+        } else {
+            pH = 0;
+        }
+        long long left = budget;
+        for (int base = 0; base < na; base += 32) {
+            const int q = base + lane;
+            int pos = wh2 + q;
+            if (pos >= Wc) pos -= Wc;
+            const bool in = q < na;
+            const int p = in ? wp[pos] : 0, d = in ? wd[pos] : 0;
+            int id = in ? wi[pos] : -1;
+            const long long incl = warp_incl_sum64(p, lane);
+            const bool whole = in && incl <= left;
+            if (track && off && whole) id = emit_first(a, id, true, t1);
+            const bool keep = whole && d - off > 0 && (long long)p < mctx;
             const unsigned bal = __ballot_sync(kFull, keep);
+            const int x = p - (G + 1), z = d - off + (G + 1);
             if (keep) {
-                const int pos = kept + __popc(bal & lanemask_lt());
-                nc[pos] = ctx;
-                np[pos] = pre;
-                nd[pos] = dec;
-                ni[pos] = id;
+                const int r = nd + __popc(bal & lanemask_lt());
+                rx[r] = x;
+                rz[r] = z;
+                ri[r] = id;
             }
-            kept += __popc(bal);
-            rused = __shfl_sync(kFull, incl_r, 31);
-            wst = __shfl_sync(kFull, incl_w, 31);
+            if (bal) {
+                csx += warp_sum64(keep ? (long long)x : 0);
+                emin = min(emin, __reduce_min_sync(kFull, keep ? last_batch(x, z) : kBig));
+                nd += __popc(bal);
+            }
+            freeb += warp_sum64(whole && !keep ? (long long)dblk(dv, p) : 0);  // ended with its prompt
+            // the last admitted prompt may continue in later batches
+            const unsigned part = __ballot_sync(kFull, in && !whole);
+            if (part) {
+                const int l = __ffs(part) - 1;
+                pf = true;
+                pC = (int)(left - (__shfl_sync(kFull, incl, l) - __shfl_sync(kFull, p, l)));
+                pP = __shfl_sync(kFull, p, l) - pC;
+                pD = __shfl_sync(kFull, d, l);
+                pI = __shfl_sync(kFull, id, l);
+                pH = dblk(dv, pC);
+            }
+            left -= __shfl_sync(kFull, incl, 31);
         }
         __syncwarp();
-        int32_t *x0 = rc, *x1 = rp, *x2 = rd, *x3 = ri;
-        rc = nc;
-        rp = np;
-        rd = nd;
-        ri = ni;
-        nc = x0;
-        np = x1;
-        nd = x2;
-        ni = x3;
-        nr = kept;
         wh = wh2 + na;
         if (wh >= Wc) wh -= Wc;
         nw = nw2 - na;
-        t += (double)T;
+        ++G;
         if (nw > capW) {
             err = kECapacity;
             break;
@@ -726,11 +806,13 @@ __device__ void advance_instance_kv(const K3Launch &a, const StateBuf &src, cons
         fail3(a.ctl, err, lane);
         return;
     }
+    const int nr = nd + (pf ? 1 : 0);
     for (int q = lane; q < capR; q += 32) {
-        dst.run_ctx[rrow + q] = q < nr ? rc[q] : 0;
-        dst.run_pre[rrow + q] = q < nr ? rp[q] : 0;
-        dst.run_dec[rrow + q] = q < nr ? rd[q] : 0;
-        if (track) idst.run_id[rrow + q] = q < nr ? ri[q] : -1;
+        const bool d = q < nd, p = pf && q == nd;
+        dst.run_ctx[rrow + q] = d ? rx[q] + G : p ? pC : 0;
+        dst.run_pre[rrow + q] = p ? pP : 0;
+        dst.run_dec[rrow + q] = d ? rz[q] - G : p ? pD : 0;
+        if (track) idst.run_id[rrow + q] = d ? ri[q] : p ? pI : -1;
     }
     for (int q = lane; q < capW; q += 32) {
         int pos = wh + q;

@@ -53,6 +53,7 @@ struct lr_ctx {
     int kv_warps = 0;
     size_t kv_smem = 0;
     size_t k3_kv_smem = 0;  // the KV stream step's shared memory (all warps of a CTA)
+    bool k3_kv_ok = false;  // the queue capacities are within what it takes
     int32_t *kv_order = nullptr;  // [max_queries] the estimate's query order
     int32_t *kv_leaders = nullptr, *kv_sort = nullptr;  // [max_queries]; [4][kKvBuckets] + 4 + [2][tiles] + [ceil(I/8)]
     float *kv_mat = nullptr;  // [max_queries][I] the KV estimate matrix a route scores
@@ -809,7 +810,10 @@ int lr_set_kv_limits(lr_ctx *c, const int32_t *block_size, const int64_t *num_bl
     c->kv_warps = warps;
     c->kv_smem = warps * per_warp;
     c->k3_kv_smem = lr::kK3Warps * lr::advance_kv_smem_per_warp(c->cfg);
-    if (c->k3_kv_smem <= 200 * 1024) {
+    // capacities it takes: 44 B a running and 12 B a waiting request within 200 KB for four
+    // instances (it needs less)
+    c->k3_kv_ok = lr::kK3Warps * sizeof(int32_t) * ((size_t)11 * c->cfg.capR + (size_t)3 * c->cfg.capW + 32) <= 200 * 1024;
+    if (c->k3_kv_ok) {
         e = lr::set_k3_kv_smem(c->k3_kv_smem);
         if (e != cudaSuccess) {
             free_kv(c);
@@ -868,7 +872,7 @@ int lr_advance_tracked(lr_ctx *c, int32_t Q, const int32_t *assign, const int32_
     if (dec_cols != 1 && dec_cols != c->cfg.M) return fail(c, LR_EINVAL, "dec_cols must be 1 or num_models");
     if (!std::isfinite(t_now)) return fail(c, LR_EINVAL, "t_now must be finite");
     if (c->cfg.capR < c->max_seqs) return fail(c, LR_ECAPACITY, "advancing needs cap_running >= every max_seqs");
-    if (c->kv_on ? c->k3_kv_smem > 200 * 1024 : !c->k3_ok)
+    if (c->kv_on ? !c->k3_kv_ok : !c->k3_ok)
         return fail(c, LR_ECAPACITY, "queue capacities too large for one advance warp");
     lr::K3Launch k;
     std::memset(&k, 0, sizeof(k));

@@ -206,6 +206,39 @@ __device__ __forceinline__ long long warp_sum64(long long v) {
     return (long long)(s0 + ((unsigned long long)s1 << 22) + ((unsigned long long)s2 << 44));
 }
 
+// Division by an instance's block size, which the KV kernels repeat many times a batch:
+// unsigned n / d for any 32-bit n as a multiply-high and shifts (Granlund and
+// Montgomery's method for invariant divisors: l = ceil(log2 d), m = floor(2^32 (2^l - d)
+// / d) + 1, q = (t + ((n - t) >> 1)) >> (l - 1) with t = mulhi(m, n); d = 1 takes
+// shifts of 0).
+struct Div32 {
+    unsigned d, m;
+    int s1, s2;
+};
+__device__ __forceinline__ Div32 make_div32(int d) {
+    const unsigned ud = (unsigned)d;
+    const int l = ud <= 1u ? 0 : 32 - __clz((int)(ud - 1u));
+    Div32 v;
+    v.d = ud;
+    v.m = (unsigned)((((1ull << 32) * ((1ull << l) - ud)) / ud) + 1ull);
+    v.s1 = min(l, 1);
+    v.s2 = max(l - 1, 0);
+    return v;
+}
+__device__ __forceinline__ unsigned udiv32(const Div32 &v, unsigned n) {
+    const unsigned t = __umulhi(v.m, n);
+    return (t + ((n - t) >> v.s1)) >> v.s2;
+}
+// ceil(c / d) for 0 <= c < 2^31
+__device__ __forceinline__ int dblk(const Div32 &v, int c) { return (int)udiv32(v, (unsigned)c + v.d - 1u); }
+// x mod d in [0, d) for any int x
+__device__ __forceinline__ int dres(const Div32 &v, int x) {
+    if (x >= 0) return (int)((unsigned)x - udiv32(v, (unsigned)x) * v.d);
+    const unsigned ax = (unsigned)(-(long long)x);
+    const unsigned r = ax - udiv32(v, ax) * v.d;
+    return r == 0u ? 0 : (int)(v.d - r);
+}
+
 // Candidate-kernel tile block: everything one CTA of the candidate kernel needs about
 // its tile of 4 * tgp instances, laid out as that CTA's shared memory so that a single
 // bulk copy brings it in.  Instance j0 + 4g + u of the tile sits in column u * tgp + g:
@@ -434,9 +467,9 @@ __host__ __device__ inline size_t advance_smem_per_warp(const DevConfig &c) {
     return (sizeof(int32_t) * ((size_t)3 * c.capR + (size_t)3 * c.capW + 96) + 15) & ~(size_t)15;
 }
 // The KV stream step's waiting queue is a ring of capW + capR entries: preempted
-// requests return to its front.
+// requests return to its front.  (A window's words, the decoders, the ring; 16-byte aligned.)
 __host__ __device__ inline size_t advance_kv_smem_per_warp(const DevConfig &c) {
-    return sizeof(int32_t) * ((size_t)8 * c.capR + (size_t)3 * ((size_t)c.capW + c.capR) + 32);
+    return (sizeof(int32_t) * ((size_t)3 * c.capR + (size_t)3 * ((size_t)c.capW + c.capR) + 160) + 15) & ~(size_t)15;
 }
 cudaError_t launch_advance(const K3Launch &a, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_advance_kv(const K3Launch &a, int grid, size_t smem, cudaStream_t st);

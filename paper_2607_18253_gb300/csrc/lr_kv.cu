@@ -81,39 +81,6 @@ __device__ __forceinline__ void kv_cal_push(int32_t *head, int32_t *nxt, int32_t
 __device__ __forceinline__ long long kv_end(const int4 &q, long long mctx) {
     return min((long long)q.z - 1, mctx - 1 - q.x);
 }
-// Division by an instance's block size, which the load repeats many times a batch:
-// unsigned n / d for any 32-bit n as a multiply-high and shifts (Granlund and
-// Montgomery's method for invariant divisors: l = ceil(log2 d), m = floor(2^32 (2^l - d)
-// / d) + 1, q = (t + ((n - t) >> 1)) >> (l - 1) with t = mulhi(m, n); d = 1 takes
-// shifts of 0).
-struct Div32 {
-    unsigned d, m;
-    int s1, s2;
-};
-__device__ __forceinline__ Div32 make_div32(int d) {
-    const unsigned ud = (unsigned)d;
-    const int l = ud <= 1u ? 0 : 32 - __clz((int)(ud - 1u));
-    Div32 v;
-    v.d = ud;
-    v.m = (unsigned)((((1ull << 32) * ((1ull << l) - ud)) / ud) + 1ull);
-    v.s1 = min(l, 1);
-    v.s2 = max(l - 1, 0);
-    return v;
-}
-__device__ __forceinline__ unsigned udiv32(const Div32 &v, unsigned n) {
-    const unsigned t = __umulhi(v.m, n);
-    return (t + ((n - t) >> v.s1)) >> v.s2;
-}
-// ceil(c / d) for 0 <= c < 2^31
-__device__ __forceinline__ int dblk(const Div32 &v, int c) { return (int)udiv32(v, (unsigned)c + v.d - 1u); }
-// x mod d in [0, d) for any int x
-__device__ __forceinline__ int dres(const Div32 &v, int x) {
-    if (x >= 0) return (int)((unsigned)x - udiv32(v, (unsigned)x) * v.d);
-    const unsigned ax = (unsigned)(-(long long)x);
-    const unsigned r = ax - udiv32(v, ax) * v.d;
-    return r == 0u ? 0 : (int)(v.d - r);
-}
-
 // One instance's residents alone, batch by batch, from the snapshot.  Every lane
 // holds the same scalar state.
 //

@@ -235,3 +235,43 @@ def test_a_query_that_could_never_run_keeps_the_live_snapshot():
     w2, c2 = oracle.advance(wl, np.zeros(wl.num_instances), [], [], [], 0.5, kv=limits)
     check_state(read(rt), w2, c2)
     rt.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("bs", [1, 16, 64])
+def test_decode_windows_under_limits(mode, bs):
+    # long decode-only stretches with requests ending inside them, by their length or at the
+    # context limit, block needs that preempt, and a head held back by blocks or by seats;
+    # arrivals in the middle of a window and exactly at a batch's end
+    import dataclasses
+    I, cap = 13, 64
+    rng = np.random.default_rng(78 + bs)
+    wl = W.small_workload(6, num_instances=I, num_models=3, num_queries=8, cap_running=cap, cap_waiting=128,
+                          first_token_mode=mode, wait_max=20, budget_range=(64, 300), min_gap=8)
+    S = rng.integers(3, 50, I).astype(np.int32)
+    n_run = np.minimum(S, rng.integers(0, 40, I)).astype(np.int32)
+    col = np.arange(cap)[None, :] < n_run[:, None]
+    wl = dataclasses.replace(
+        wl, max_seqs=S, n_run=n_run, run_pre=np.zeros((I, cap), np.int32),
+        run_ctx=np.where(col, rng.integers(0, 900, (I, cap)), 0).astype(np.int32),
+        run_dec=np.where(col, rng.integers(1, 300, (I, cap)), 0).astype(np.int32))
+    bsz, nb, mctx = W.kv_limits(wl, 3, block_sizes=(bs,), tightness=(0.05, 0.6), ctx_slack=(60, 300), max_new=60)
+    rt = R().LatencyRouter.from_workload(wl)
+    rt.set_kv_limits(bsz, nb, mctx, horizon=4096)
+    rt.load_state(*R().state_tensors(wl))
+    N = 64
+    ftt = torch.full((N,), float("nan"), dtype=torch.float64, device="cuda")
+    rt.track_first_tokens(ftt)
+    rt.load_state(*R().state_tensors(wl))
+    track, clk, kv = oracle.new_track(wl, N), np.zeros(I), (bsz, nb, mctx)
+    for step, t_now in enumerate((0.011, 0.4, -1.0, 2.1, 9.0, 3e5)):
+        a = rng.integers(-1, I, 8).astype(np.int32)
+        p, d = rng.integers(1, 160, 8).astype(np.int32), rng.integers(1, 60, 8).astype(np.int32)
+        if t_now < 0:  # exactly where some instance's batch ends
+            t_now = float(np.median(oracle.advance(wl, clk, a, p, d, 1.1, kv=kv)[1]))
+        rt.advance(*(torch.from_numpy(x).cuda() for x in (a, p, d)), t_now, id_base=8 * step)
+        wl, clk, track = oracle.advance(wl, clk, a, p, d, t_now, track=track, id_base=8 * step, kv=kv)
+        check_state(read(rt), wl, clk, f"step {step}")
+        assert rt.status() == R().LR_OK, step
+        np.testing.assert_array_equal(ftt.cpu().numpy().view(np.uint64), track["first_token_time"].view(np.uint64))
+    rt.close()
