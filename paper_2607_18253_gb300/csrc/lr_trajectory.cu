@@ -374,6 +374,7 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
         int n = n0;  // decoders alive at the start of batch l
         int l = 1, head = 0, iters = 0;
         int ph = 0;  // prompt prefix sum at the waiting head
+        const int ptot = lds(sP + 4u * nw);
         int fnext = tr.next_end(1);
         int la = 0, r0 = 0;
 
@@ -505,7 +506,7 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
             const unsigned dcm = __ballot_sync(kFull, dc);
             const int nent = __popc(__ballot_sync(kFull, valid));
             const int last_end = __shfl_sync(kFull, en, max(nent - 1, 0));
-            const int total_left = base + lds(sP + 4u * nw) - ph;
+            const int total_left = base + ptot - ph;
             const int lb = l + lane;
             const int calw = lb < kCalendar ? lds(tr.cal + 4u * lb) : -1;
             const unsigned calok = __ballot_sync(kFull, calw >= 0);
@@ -517,20 +518,22 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
                 // decoders ending in batch lw: the calendar's and this window's (off the chain)
                 const int ecal = __shfl_sync(kFull, calw, w);
                 const int ewin = __popc(__ballot_sync(kFull, dn >= 0 && fl == lw) & dcm);
+                // (one test for every reason to stop: a branch costs as much as the batch's
+                // arithmetic)
                 const int freeseats = S - nn - (ip ? 1 : 0);
-                if (freeseats <= 0 && !ip) break;  // every slot holds a decoder
+                const bool seats = freeseats > 0;
                 const int budget = B - nn;
-                if (budget <= 0) break;
                 int T2 = T + budget;
-                if (T2 >= total_left) break;  // the queue could run out in this batch
-                if (freeseats > 0) {
-                    const int kl = ndone + (ip ? 1 : 0) + freeseats - 1;  // last entry a free slot lets start
-                    const int lim = __shfl_sync(kFull, en, min(kl, 31));
-                    if (kl < nent) T2 = min(T2, lim);
-                    else if (T2 > last_end) break;  // beyond the lanes
-                } else {
-                    T2 = min(T2, __shfl_sync(kFull, en, ndone & 31));  // only the prefill in progress advances
-                }
+                // the last entry a free slot lets start, or the prefill in progress alone
+                const int kl = ndone + (seats ? (ip ? 1 : 0) + freeseats - 1 : 0);
+                const int lim = __shfl_sync(kFull, en, min(kl, 31));
+                const bool within = kl < nent;
+                const bool stop = (!seats && !ip)              // every slot holds a decoder
+                                  | (budget <= 0)
+                                  | (T2 >= total_left)         // the queue could run out in this batch
+                                  | (!within && T2 > last_end);  // beyond the lanes
+                if (stop) break;
+                if (within) T2 = min(T2, lim);
                 const bool nd = valid && dn < 0 && en <= T2;
                 if (nd) {
                     dn = lw;
@@ -589,7 +592,8 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
         while (iters < c.max_iters && l < (1 << 30)) {
             ++iters;
             int cnt = n + (pf ? 1 : 0);  // requests running in batch l
-            if (pf || cnt < S) {
+            // (no window if the queue could run out in its first batch)
+            if ((pf || cnt < S) && B - n < (pf ? pfR : 0) + ptot - ph) {
                 const int wt = window();  // every batch of a window counts against max_iters
                 if (wt > 0) {
                     iters += wt - 1;
