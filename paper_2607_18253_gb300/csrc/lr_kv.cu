@@ -36,6 +36,10 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr long long kHuge = 1LL << 62;
 constexpr int kBigKv = 0x7fffffff;
+// A condition that is the same on every lane, as a vote: the compiler then knows it and
+// branches without setting up a reconvergence point (which costs the scalar code of a warp
+// more than the vote).
+__device__ __forceinline__ bool uni(bool c) { return __any_sync(kFull, c) != 0; }
 __device__ __forceinline__ int clamp32(long long x) { return (int)min(x, (long long)kBigKv); }
 
 __device__ __forceinline__ long long kv_blocks(long long c, long long bs) { return (c + bs - 1) / bs; }
@@ -541,14 +545,14 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 }
                 if (G >= Gstop) break;
                 slack = nr > 0 ? fa : kHuge;
-                if (fa < 0) {
+                if (uni(fa < 0)) {
                     // preemption from the tail (see the general form)
                     const int excess = -fa;
                     int acc = 0;
-                    for (int top = tl - 1; top >= 0 && acc < excess; top -= 32) {
+                    for (int top = tl - 1; uni((top >= 0) & (acc < excess)); top -= 32) {
                         const int s2 = top - lane;
                         unsigned live = __ballot_sync(kFull, s2 >= 0 && reinterpret_cast<const int *>(rq + s2)[1] >= 0);
-                        while (live != 0u && acc < excess) {
+                        while (uni((live != 0u) & (acc < excess))) {
                             const int r = top - (__ffs(live) - 1);
                             live &= live - 1u;
                             const int4 q = rq[r];
@@ -578,14 +582,13 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 budget = B - nd;
                 const int bar_ = budget, far_ = fa;
                 f1 = f4 = 0;
-                if (fa >= hm) {
+                if (uni(fa >= hm)) {
                     do {
                         const int x = min(hp, budget);
-                        if ((x == hp ? hb : dblk(dv, x)) > fa) break;
-                        if (x < hp || wc == 1 || hfin <= hp || ne == C) {
-                            scanned = true;  // the general form admits it
-                            break;
-                        }
+                        const bool fits = (x == hp ? hb : dblk(dv, x)) <= fa;
+                        // (the general form admits it)
+                        scanned = fits & ((x < hp) | (wc == 1) | (hfin <= hp) | (ne == C));
+                        if (uni(!fits | scanned)) break;
                         // whole: a decoder from the next batch on, ending in batch G + hfin - hp
                         const int xs = hp - (G + 1), E = G + (hfin - hp);
                         int res = hrem + ridx - 1;  // xs mod bs
@@ -616,9 +619,9 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                         hp = wv.x;
                         hd = wv.y;
                         derive();
-                    } while (budget > 0 && nr < S);
+                    } while (uni((budget > 0) & (nr < S)));
                 }
-                if (scanned) {  // this batch goes on below
+                if (uni(scanned)) {  // this batch goes on below
                     fb = fa;
                     s_end = s;
                     f3 = t3;
@@ -631,13 +634,13 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                 r2 += ndb;
                 r3 += t3;
                 r4 += f4;
-                if (la0 != 0) record(slack, far_, bar_, budget);
-                if (s >= 0) {  // the decoders whose last batch this is return their blocks
+                if (uni(la0 != 0)) record(slack, far_, bar_, budget);
+                if (uni(s >= 0)) {  // the decoders whose last batch this is return their blocks
                     do {
                         const int ns = nxt[s];
                         const int4 q = rq[s];
                         const int ebs = eb[s];
-                        if (q.y == 0) {  // a hole is a request preempted after it was filed
+                        if (uni(q.y == 0)) {  // a hole is a request preempted after it was filed
                             fb += ebs;
                             src -= q.x;
                             --nd;
@@ -645,7 +648,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
                             if (lane == 0) reinterpret_cast<int *>(rq + s)[1] = -1;
                         }
                         s = ns;
-                    } while (s >= 0);
+                    } while (uni(s >= 0));
                     if (lane == 0) head[G & (kKvCal - 1)] = -1;
                     nr = nd;
                 }
@@ -841,7 +844,7 @@ __device__ void kv_instance(const KvLoad &a, const StateBuf &out, int j, int lan
         }
         // 2. Admission from the waiting front while budget, a seat and the first chunk's
         //    blocks allow; one that prefills whole decodes from the next batch.
-        while (budget > 0 && wc > 0 && nr < S) {
+        while ((budget > 0) & (wc > 0) & (nr < S)) {
             const int x = min(hp, budget);
             const int qt = (int)udiv32(dv, (unsigned)x), rem = x - qt * bs;
             const int nb1 = qt + (rem > 0 ? 1 : 0);
