@@ -286,7 +286,7 @@ constexpr int kCalConsumerWarps = kCalThreads / 32 - 1;  // the last warp issues
 constexpr int kCalTile = 2 * 32 * kCalConsumerWarps;     // rows per staged tile, two a consumer lane (16-byte copies)
 constexpr int kCalStagesMax = 3;                    // tiles in flight per CTA
 constexpr int kCalFlushRows = 128;                  // rows a lane sums in 64 bits between flushes
-constexpr size_t kCalSmemMax = 227 * 1024;
+constexpr size_t kCalSmemMax = 223 * 1024;           // (the kernel's static words need 4 KB)
 constexpr size_t kCalStageBytes = (size_t)kCalTile * (kCalCols * 8 + 8 + 4);
 constexpr int kCalFlushSums = 26;  // a warp flush's sums: 15 of G, 5 + 5 halves of b, the row count
 // the CTA's shared sums: 128-bit [M][kCalAcc] and the flushes' carry-save words [M][kCalFlushSums]

@@ -150,3 +150,26 @@ def test_long_slices_flush_within_128_rows():
     got = rt.calibrate(dev(F), dev(m), dev(t), shared_beta1=True).cpu().numpy()
     assert rt.status() == R().LR_OK
     np.testing.assert_allclose(got, oracle.calibrate(F, m, t, M, shared_beta1=True), rtol=RTOL)
+
+
+@pytest.mark.parametrize("M,N,drift", [(2, 63, False), (15, 959, False), (16, 50_001, False), (3, 145_923, True),
+                                       (7, 300_002, False), (12, 150_001, True), (40, 200_003, False),
+                                       (128, 160_000, True)])
+def test_mixed_models(M, N, drift):
+    # rows of several models in the order they ran: the tiles are listed by model, the models
+    # shared out over the warps (up to 15 a warp or more each, beyond that several to a warp),
+    # again when the log's mix drifts.  The sums are exact, so the fit is the same, bit for
+    # bit, as that of the same rows grouped by model.
+    F, m, t = W.batch_log(N, M, seed=M, coef=coef_of(M, M), noise=0.03, grouped=False)
+    if drift:  # from mostly the first models to mostly the last
+        rng = np.random.default_rng(M)
+        m = np.sort(m)[np.argsort(np.arange(N) + rng.normal(0.0, N / 16, N))].astype(m.dtype)
+    rt = router_for(M)
+    order = np.argsort(m, kind="stable")
+    for shared in (True, False):
+        got = rt.calibrate(dev(F), dev(m), dev(t), shared_beta1=shared).cpu().numpy()
+        assert rt.status() == R().LR_OK
+        ref = rt.calibrate(dev(F[order]), dev(m[order]), dev(t[order]), shared_beta1=shared).cpu().numpy()
+        np.testing.assert_array_equal(got, ref)
+        if N // M > 100:
+            np.testing.assert_allclose(got, oracle.calibrate(F, m, t, M, shared_beta1=shared), rtol=RTOL)
