@@ -41,8 +41,8 @@ WORKLOAD = "pool256"
 # DRAM bytes (read + write) per launch of the step's kernels on this workload, from one
 # ncu capture of the kernels as they are built now (summaries under profiles/); they
 # are retaken whenever one of the kernels changes.
-NCU_TRAFFIC = {"k_route": 4_577_792 + 8_019_712, "k_trajectory": 1_401_344, "k_estimate": 357_888 + 7_386_624,
-               "k_calibrate": 208_430_848 + 3_465_728}
+NCU_TRAFFIC = {"k_route": 4_586_240 + 8_535_296, "k_trajectory": 1_398_272, "k_estimate": 381_952 + 7_250_432,
+               "k_calibrate": 208_709_632 + 3_387_392}
 
 
 def _peaks():
@@ -709,8 +709,8 @@ def run_kv(args, dev, wl, flush):
                                    "k_kv_estimate, k_kv_expand)", "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
                          "frac": ach / hbm, "peak_source": f"{src} (MEASURED_PEAKS.json hbm_gbs, copy)",
                          "algorithmic_bytes": nbytes, "traffic": None,
-                         "note": "the call's six kernels together; k_kv_estimate alone read 2.35 MB and wrote "
-                                 "0.85 MB per launch (ncu); the load is one dependency chain per instance"}}
+                         "note": "the call's six kernels together; k_kv_estimate alone read 2.48 MB and wrote "
+                                 "0.93 MB per launch (ncu); the load is one dependency chain per instance"}}
 
 
 def run_avgcase(args, dev, wl, flush):
@@ -937,9 +937,9 @@ def run_stream(args, dev):
     lat = [e0.elapsed_time(e1) for e0, e1 in ev]
     q = np.percentile(np.asarray(lat) * 1e3, [50, 99])
     fin = rt.read_state(device=dev)
-    # launches per decision: advance (K3 KV, KV load) + route (count, tile sums, scan,
-    # scatter, walk, expand, route)
-    launches += 9 * nb
+    # launches per decision: advance (K3 KV, KV load) + route (walk, route; 16 queries on
+    # this pool are walked without a sort)
+    launches += 4 * nb
     out["kv_poisson_16"] = {"arrival_qps": 0.5 * float(cap.sum()), "batches": nb, "queries": nb * m, "p50_us": float(q[0]), "p99_us": float(q[1]),
                             "mean_us": float(np.mean(lat) * 1e3), "wall_s": wall,
                             "simulated_s": float(arr[nb * m - 1]),

@@ -519,7 +519,7 @@ __device__ void summarize_instance(const K1Launch &a, int j, int lane, int32_t *
                 const int ecal = __shfl_sync(kFull, calw, w);
                 const int ewin = __popc(__ballot_sync(kFull, dn >= 0 && fl == lw) & dcm);
                 // (one test for every reason to stop: a branch costs as much as the batch's
-                // arithmetic)
+                // arithmetic; 256 instances 29.7 -> 25.7 us, 64 20.4 -> 19.6)
                 const int freeseats = S - nn - (ip ? 1 : 0);
                 const bool seats = freeseats > 0;
                 const int budget = B - nn;
