@@ -590,8 +590,10 @@ __global__ void __launch_bounds__(kCalThreads, 1) k_calibrate(long long N, const
             // do), and each warp takes the rows of the models it owns: the warps are dealt out
             // by the models' rows in a tile, again when a warp's share grows fourfold.
             // 1M rows of 4 / 8 / 12 / 40 models in random order: 85 / 136 / 185 / 343 us with
-            // flushes alone, 44 / 44 / 46 / 89 this way; a run of 32 rows a model is where a
-            // warp's flush costs what listing its 64 rows does.
+            // flushes alone, 44 / 44 / 46 / 89 this way.  The line is where the two meet: 1M rows
+            // of 8 models in runs of 16 rows 49 us with flushes, 31 listed; in runs of 32 rows
+            // (a change in 37) 35 and 39, of 64 35 and 44.  2 models, runs of 16 and 32 rows: 42
+            // and 30 with flushes, 28 and 28 listed.
             auto consumers = [&]() {
                 __syncwarp();
                 asm volatile("bar.sync 1, %0;" ::"n"(kCalConsumerWarps * 32) : "memory");
