@@ -101,8 +101,8 @@ __device__ __forceinline__ double u128_to_double(const U128 &v, int p, int e2) {
 // enters fp64 once, already scaled by the powers of two that bring the diagonal into
 // [1, 4) (regressor p scaled by 2^-h_p with h_p half the leading-bit position of G_pp),
 // so the conditioning that the raw feature magnitudes take away is restored without a
-// rounding.  The code runs once per call from cold instruction caches, and the fp64
-// pipe is narrow on this part: a warp forms the 20 scaled entries of a model,
+// rounding.  The solve is a chain of dependent integer and fp64 work on one CTA, and the
+// fp64 pipe is narrow on this part: a warp forms the 20 scaled entries of a model,
 // a lane each (integer pipes only), then a warp factors five models' systems with
 // straight-line code in registers, whose only fp64 divisions are the pivot reciprocals.
 constexpr int kCalSolveWords = 24;  // per model in shared memory: 15 + 5 scaled entries, 5 exponents
