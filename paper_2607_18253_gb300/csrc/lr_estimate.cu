@@ -865,12 +865,14 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                     const f32x2 nm = pack2(lm.y, lm.y);
                     const float4 *tr4 = s_t + rr * Gp;
                     const float2 *carow = s_ca + rr * M;
+                    // the best of a group of four, and the first group that has it: an objective of
+                    // -inf (a product beyond fp32) is a value like any other, NaN (no estimate, or
+                    // beyond the pool) is none
                     float best = -INFINITY, U = 0.f;
-                    int bj = -1, cur = -1;
-                    for (int gg = 0; 4 * gg < I; ++gg) {
+                    int bg = -1, cur = -1;
+                    auto objectives = [&](int gg, float U4[4], float J[4]) {
                         const float4 t4 = tr4[gg];
                         const int m = s_m4[gg];
-                        float U4[4], J[4];
                         if (m >= 0) {
                             if (m != cur) {
                                 const float2 ca = carow[m];
@@ -887,18 +889,22 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                         }
                         unpack2(fma2(nm, pack2(t4.x, t4.y), pack2(U4[0], U4[1])), J[0], J[1]);
                         unpack2(fma2(nm, pack2(t4.z, t4.w), pack2(U4[2], U4[3])), J[2], J[3]);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (J[u] > best) {  // NaN (no estimate, or beyond the pool) never is
-                                best = J[u];
-                                bj = 4 * gg + u;
-                            }
+                    };
+                    float U4[4], J[4];
+                    for (int gg = 0; 4 * gg < I; ++gg) {
+                        objectives(gg, U4, J);
+                        const float m1 = fmaxf(fmaxf(J[0], J[1]), fmaxf(J[2], J[3]));  // NaN only if all are
+                        if (m1 > best || (bg < 0 && m1 == m1)) {
+                            best = m1;
+                            bg = gg;
+                        }
                     }
                     if (act) {
                         Cand w = {0u, 0, 0.f, 0.f};
-                        if (bj >= 0) {
-                            const float2 ca = carow[s_m4[Gp + bj]];
-                            w = Cand{1u, bj, reinterpret_cast<const float *>(tr4)[bj], __fmaf_rn(-lm.x, ca.x, ca.y)};
+                        if (bg >= 0) {
+                            objectives(bg, U4, J);
+                            const int u = first4(J, best);
+                            w = Cand{1u, 4 * bg + u, reinterpret_cast<const float *>(tr4)[4 * bg + u], pick4(U4, u)};
                         }
                         write_pick(a, (size_t)pp * a.Q + q0 + row, w);
                     }

@@ -110,6 +110,31 @@ def test_sweep_lane_splits(P):
           sweep=P)
 
 
+@pytest.mark.parametrize("I", [5, 45, 200])
+@pytest.mark.parametrize("P", [1, 2, 5, 33])
+def test_objectives_beyond_fp32(I, P):
+    # a finite mu or lambda whose product with the time or the cost overflows: the objective is
+    # -inf on some instances or on all, and the lowest instance wins the tie, alone or in a sweep
+    wl = W.small_workload(50 + P, num_instances=I, num_models=3, num_queries=101, budget_range=(16, 96), min_gap=8)
+    wl = dataclasses.replace(wl, coef=wl.coef * np.float32(100.0), price_in=(wl.price_in * 1e6).astype(np.float32))
+    rt = R().LatencyRouter.from_workload(wl, max_pairs=P)
+    rt.load_state(*R().state_tensors(wl))
+    p, dh, acc, _ = R().query_tensors(wl)
+    _, _, t32, _ = oracle.estimate_matrix(wl)
+    mid = np.float32(np.finfo(np.float32).max / np.median(t32))  # overflows on about half of the candidates
+    for lam1, mu1 in ((1.0, 3e38), (1.0, mid), (3e38, 0.0)):
+        lam, mu = np.linspace(0.5, 2.0, P).astype(np.float32), np.geomspace(1e-2, 1.0, P).astype(np.float32)
+        lam[P // 2], mu[P // 2] = lam1, mu1
+        a, u, tc = oracle.route(wl, t32, lam=lam, mu=mu)
+        o = rt.route(p, dh, acc, lam, mu, frontier=True)
+        np.testing.assert_array_equal(o["assign"].cpu().numpy(), a)
+        np.testing.assert_array_equal(bits(o["util"].cpu().numpy()), bits(u))
+        np.testing.assert_array_equal(bits(o["ttft_chosen"].cpu().numpy()), bits(tc))
+        np.testing.assert_allclose(o["frontier"].cpu().numpy(), oracle.frontier(wl, a, tc), rtol=1e-12)
+    assert rt.status() == R().LR_OK
+    rt.close()
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 def test_prefill_totals_beyond_fp32(mode):
     # one instance whose residents hold more than 2^24 prompt tokens: the whole tile leaves the
