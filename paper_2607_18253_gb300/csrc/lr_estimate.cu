@@ -809,7 +809,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                                 float4 *part = reinterpret_cast<float4 *>(s_part + 2 * (rr * WPR + wrow));
                                 part[0] = make_float4(t[0], t[1], t[2], t[3]);
                                 part[1] = make_float4(w, U[0], __int_as_float(jb), 0.f);
-                            } else if (best == 0u && lane == 0) {  // an invalid prompt
+                            } else if (best == 0u && lane == 0) {  // every objective is NaN
                                 reinterpret_cast<float *>(s_part + 2 * (rr * WPR + wrow) + 1)[0] = kNaN;
                             }
                             break;
@@ -910,8 +910,10 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                     }
                 }
             } else if (DEFER) {
-                // one thread per row: the best warp of the row (the first among equals), then
-                // the first of the winning thread's four instances with that value
+                // one thread per row: the best warp of the row (the first among equals; a warp whose
+                // objectives are all NaN -- an invalid prompt, or a cost that overflows times a
+                // lambda of 0 -- yields to any), then the first of the winning thread's four
+                // instances with that value
                 __syncthreads();
                 for (int r2 = threadIdx.x; r2 < nrows; r2 += blockDim.x) {
                     const float4 *part = reinterpret_cast<const float4 *>(s_part + 2 * (size_t)(r2 * WPR));
@@ -919,7 +921,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                     float w = part[1].x;
                     for (int wi = 1; wi < WPR; ++wi) {
                         const float x = part[2 * wi + 1].x;
-                        if (x > w) {
+                        if (x > w || w != w) {
                             w = x;
                             wb = wi;
                         }
@@ -929,7 +931,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                     const float J[4] = {__fmaf_rn(nm, tt[0], d.y), __fmaf_rn(nm, tt[1], d.y), __fmaf_rn(nm, tt[2], d.y),
                                         __fmaf_rn(nm, tt[3], d.y)};
                     const int u = first4(J, w);
-                    // (an invalid prompt's row is NaN in every warp)
+                    // (w is NaN only if it is in every warp)
                     write_pick(a, (size_t)(q0 + r2), Cand{w == w ? 1u : 0u, __float_as_int(d.z) + u, pick4(tt, u), d.y});
                 }
             } else if (ROUTE && Gp > 32) {

@@ -135,6 +135,34 @@ def test_objectives_beyond_fp32(I, P):
     rt.close()
 
 
+@pytest.mark.parametrize("I", [64, 256, 512])
+@pytest.mark.parametrize("first", [0, 1])
+def test_a_model_without_objective(I, first):
+    # a cost that overflows times a lambda of 0 is no objective (NaN) on every instance of one
+    # model, here whole warps of a wide pool, the first of a row's or its last: the others compete
+    wl = W.small_workload(6, num_instances=I, num_models=2, num_queries=200, budget_range=(64, 64), min_gap=8)
+    moi = (np.arange(I) * 2 // I).astype(np.int32)
+    wl = dataclasses.replace(wl, model_of_instance=moi, max_seqs=np.full(I, 8, np.int32), n_run=np.minimum(wl.n_run, 8),
+                             prompt_len=np.maximum(wl.prompt_len, 2))
+    wl.price_in[first] = np.finfo(np.float32).max
+    rt = R().LatencyRouter.from_workload(wl, max_pairs=2)
+    rt.load_state(*R().state_tensors(wl))
+    p, dh, acc, _ = R().query_tensors(wl)
+    t32 = oracle.estimate_matrix(wl)[2]
+    mine = np.flatnonzero(moi != first)
+    zero, mu = np.zeros(2, np.float32), np.float32(0.1)
+    # U = acc (lambda 0), J = U - mu t (rounded to 64 bits, then to 32: no winner hangs on it here)
+    J = (wl.acc[:, 1 - first, None].astype(np.float64) - np.float64(mu) * t32[:, mine]).astype(np.float32)
+    want = mine[np.argmax(J, 1)]
+    for lam, m in ((zero[:1], [mu]), (zero, [mu, mu])):
+        o = rt.route(p, dh, acc, lam, np.array(m, np.float32))
+        for k in range(len(lam)):
+            np.testing.assert_array_equal(o["assign"][k].cpu().numpy(), want)
+            np.testing.assert_array_equal(bits(o["util"][k].cpu().numpy()), bits(wl.acc[:, 1 - first]))
+            np.testing.assert_array_equal(bits(o["ttft_chosen"][k].cpu().numpy()), bits(t32[np.arange(len(want)), want]))
+    rt.close()
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 def test_prefill_totals_beyond_fp32(mode):
     # one instance whose residents hold more than 2^24 prompt tokens: the whole tile leaves the
