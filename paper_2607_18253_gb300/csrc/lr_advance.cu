@@ -906,7 +906,7 @@ cudaError_t launch_advance(const K3Launch &a, int grid, size_t smem, cudaStream_
 }
 
 cudaError_t set_k3_smem(size_t bytes) {
-    return cudaFuncSetAttribute(k_advance, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return allow_smem(k_advance, bytes);
 }
 
 cudaError_t launch_advance_kv(const K3Launch &a, int grid, size_t smem, cudaStream_t st) {
@@ -914,7 +914,7 @@ cudaError_t launch_advance_kv(const K3Launch &a, int grid, size_t smem, cudaStre
 }
 
 cudaError_t set_k3_kv_smem(size_t bytes) {
-    return cudaFuncSetAttribute(k_advance_kv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return allow_smem(k_advance_kv, bytes);
 }
 
 }  // namespace lr

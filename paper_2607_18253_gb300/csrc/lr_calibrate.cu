@@ -811,11 +811,8 @@ cudaError_t launch_calibrate(long long N, const long long *F, const int32_t *mod
 
 cudaError_t set_calib_smem(int M) {
     const size_t fixed = cal_sums_bytes(M);
-    cudaError_t e = cudaFuncSetAttribute(k_calibrate<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(fixed + kCalStageBytes * calib_stages(M)));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_calibrate<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(fixed + solve_bytes(M)));
+    cudaError_t e = allow_smem(k_calibrate<true>, fixed + kCalStageBytes * calib_stages(M));
+    if (e == cudaSuccess) e = allow_smem(k_calibrate<false>, fixed + solve_bytes(M));
     return e;
 }
 

@@ -1060,18 +1060,13 @@ cudaError_t launch_cand_mode(const K2Launch &a, int out, dim3 grid, int block, s
     }
 }
 
-template <typename F>
-cudaError_t set_attr(F f, size_t bytes) {
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <int MODE>
 cudaError_t set_mode_attrs(size_t bytes) {
     const cudaError_t es[] = {
-        set_attr(k_cand<MODE, kOutMatrix>, bytes), set_attr(k_cand<(MODE == 2 ? 0 : MODE), kOutMatrix | kOutIters>, bytes),
-        set_attr(k_cand<MODE, kOutLag>, bytes), set_attr(k_cand<MODE, kOutLag | kOutMatrix>, bytes),
-        set_attr(k_cand<MODE, kOutCon>, bytes), set_attr(k_cand<MODE, kOutCon | kOutMatrix>, bytes),
-        set_attr(k_cand<MODE, kOutSweep>, bytes), set_attr(k_cand<MODE, kOutSweep | kOutMatrix>, bytes)};
+        allow_smem(k_cand<MODE, kOutMatrix>, bytes), allow_smem(k_cand<(MODE == 2 ? 0 : MODE), kOutMatrix | kOutIters>, bytes),
+        allow_smem(k_cand<MODE, kOutLag>, bytes), allow_smem(k_cand<MODE, kOutLag | kOutMatrix>, bytes),
+        allow_smem(k_cand<MODE, kOutCon>, bytes), allow_smem(k_cand<MODE, kOutCon | kOutMatrix>, bytes),
+        allow_smem(k_cand<MODE, kOutSweep>, bytes), allow_smem(k_cand<MODE, kOutSweep | kOutMatrix>, bytes)};
     for (cudaError_t x : es)
         if (x != cudaSuccess) return x;
     return cudaSuccess;
@@ -1375,8 +1370,8 @@ cudaError_t launch_on_time(int Q, const float *util, const float *ttft, const fl
 }
 
 cudaError_t set_baseline_smem(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_baseline<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_baseline<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(k_baseline<0>, bytes);
+    if (e == cudaSuccess) e = allow_smem(k_baseline<1>, bytes);
     return e;
 }
 

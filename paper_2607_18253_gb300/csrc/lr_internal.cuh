@@ -143,6 +143,22 @@ cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, 
     return cudaLaunchKernelEx(&cfg, k, P(args)...);
 }
 
+// Lets kernel f be launched with `bytes` of dynamic shared memory.  The limit belongs to the
+// process's kernel, not to one lr_ctx, so it is always set to all that the device gives a CTA:
+// the same value whatever a context needs, and no context takes away what another launches with.
+template <typename F>
+cudaError_t allow_smem(F *f, size_t bytes) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, (const void *)f);
+    if (e != cudaSuccess) return e;
+    most -= (int)fa.sharedSizeBytes;
+    if (bytes > (size_t)most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute((const void *)f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // The live-buffer index with acquire ordering: reads of the buffer it names see
 // everything the load that published it wrote (it may have finished on another stream).
 __device__ __forceinline__ int32_t load_acquire(const int32_t *p) {

@@ -1510,10 +1510,10 @@ cudaError_t launch_kv_load(const KvLoad &a, int grid, int warps, size_t smem, cu
 }
 
 cudaError_t set_kv_smem(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_kv_load<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_kv_load<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(k_kv_load<0>, bytes);
+    if (e == cudaSuccess) e = allow_smem(k_kv_load<1>, bytes);
     auto est = [&](auto f, size_t n) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+        if (e == cudaSuccess) e = allow_smem(f, n);
     };
     est(k_kv_estimate<0, false>, EstShape<false>::kSmem);
     est(k_kv_estimate<1, false>, EstShape<false>::kSmem);

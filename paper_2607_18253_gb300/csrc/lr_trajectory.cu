@@ -1003,8 +1003,8 @@ cudaError_t launch_trajectory(const K1Launch &a, int grid, int block, size_t sme
 }
 
 cudaError_t set_k1_smem(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_trajectory<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_trajectory<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(k_trajectory<0>, bytes);
+    if (e == cudaSuccess) e = allow_smem(k_trajectory<1>, bytes);
     return e;
 }
 

@@ -386,3 +386,42 @@ def test_load_overlapping_estimates_sees_whole_snapshots():
         assert np.all(is_old | is_new)
     # after both streams finished, the new snapshot is live everywhere
     np.testing.assert_array_equal(bits(rt.estimate_ttft(p).cpu().numpy()), b_new)
+
+
+@pytest.mark.parametrize("kv", [False, True])
+def test_a_small_context_beside_a_large_one(kv):
+    # contexts of one process share the kernels: what a later, smaller one asks of them takes
+    # nothing away from the first, whose calls give what they gave before
+    wl = W.make_workload("pool256", num_queries=500)
+    rt = R().LatencyRouter.from_workload(wl, max_pairs=8)
+    if kv:
+        rt.set_kv_limits(*W.kv_limits(wl, 1, block_sizes=(16, 64)), horizon=512)
+    p, dh, acc, tau = R().query_tensors(wl)
+    lam, mu = np.linspace(0.5, 2.0, 8).astype(np.float32), np.geomspace(1e-2, 1.0, 8).astype(np.float32)
+    F, m, t = W.batch_log(3000, wl.num_models, seed=1, coef=wl.coef.astype(np.float64))
+    log = [torch.from_numpy(x).cuda() for x in (F, m, t)]
+    i32 = torch.int32
+
+    def calls():
+        out = []
+        rt.load_state(*R().state_tensors(wl))
+        out.append(rt.estimate_ttft(p))
+        for o in (rt.route(p, dh, acc, lam[:1], mu[:1]), rt.route(p, dh, acc, lam[:1], tau=tau),
+                  rt.route(p, dh, acc, lam, mu, frontier=True), rt.route_baseline(1, p, dh, acc, 1.0)):
+            out += [o[k] for k in sorted(o)]
+        out.append(rt.calibrate(*log))
+        rt.advance(torch.arange(16, dtype=i32, device="cuda"), p[:16], torch.full((16,), 20, dtype=i32, device="cuda"), 0.5)
+        out.append(rt.estimate_ttft(p))
+        assert rt.status() == R().LR_OK
+        return [x.cpu().numpy().view(np.uint8) for x in out]
+
+    before = calls()
+    small = W.small_workload(1, num_instances=2)
+    rt2 = make_router(small)
+    if kv:
+        rt2.set_kv_limits(*W.kv_limits(small, 1, block_sizes=(4,)), horizon=64)
+    after = calls()
+    rt2.close()
+    for a, b in zip(before, after):
+        np.testing.assert_array_equal(a, b)
+    rt.close()
