@@ -180,8 +180,7 @@ lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep) {
     // the tile block (tables and per-instance scalars), brought in by one bulk copy
     lr::DevConfig dt = d;
     dt.tgp = s.Gp;
-    // (and the buffers in which a warp orders the stores of rows that are not whole 16-byte words)
-    const size_t tables = lr::tile_bytes(dt) + (d.I % 4 ? (size_t)s.block * 32 : 0);
+    const size_t tables = lr::k2_head_bytes(dt, s.block);
     // wide-row partials; a sweep keeps the row's times, and once the models and the pairs
     const size_t part = sweep ? 16 * (size_t)s.Gp : s.Gp > 32 ? 2 * (size_t)wpr * 16 : 0;
     const size_t fixed = tables + (sweep ? 20 * (size_t)s.Gp + 4 + 8 * lr::kMaxPairs : 0);
@@ -528,6 +527,7 @@ static int estimate_common(lr_ctx *c, int32_t Q, const int32_t *p, float *ttft, 
     a.QS = c->est.QS;
     a.QT = c->est.QT;
     a.vec_ok = (c->cfg.I % 4 == 0) && ((uintptr_t)ttft % 16 == 0);
+    a.vec_first = (c->cfg.I % 4 == 0) && ((uintptr_t)iters % 16 == 0);
     dim3 grid(std::min(c->sms * c->est.occ, (Q + a.QS - 1) / a.QS), c->est.tiles);
     set_row_split(a, c, (int)grid.x, (int)grid.y, c->est.occ, stream);
     e = lr::launch_cand(a, lr::cand_out_flags(true, iters != nullptr, false, false, 1), grid, c->est.block,

@@ -31,9 +31,12 @@
 // 8.3 M, 15.0 us; route 20.2 M, 27.0 -> 15.1 M, 23.0 us; with the matrix 27.6 -> 24.5 us.
 //
 // The estimate matrix is write-only (4 bytes per candidate) and leaves as one
-// 16-byte evict-first store per thread and row.  Where rows are not whole 16-byte words
-// (I % 4 != 0) each warp puts its 128 elements of a row in order in shared memory first:
-// 4-byte stores 16 bytes apart wrote every sector in pieces (50,001 x 250: 26.6 -> 15.6 us).
+// 16-byte evict-first store per thread and row, the batch indices too.  Where rows are not
+// whole 16-byte words (I % 4 != 0) a thread stores its four values one by one, under
+// predicates (in a loop that could not be unrolled they took 27.3 us for 50,001 x 250, now
+// 12.3).  The average-case sources have little else to do than to store: there each warp puts
+// its 128 elements of a row in order in shared memory first (15.0 -> 10.7 us for 50,001 x 250;
+// the SFS estimate, bound by issue, loses by it: 12.3 -> 13.6).
 // Routing reduces each row with redux.sync over the objective (the value itself, or an
 // order-preserving integer key): the lowest lane (lowest instance) among the maximal wins,
 // as in a first-max scan.
@@ -373,10 +376,9 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
     // targets and the raw query rows (route with one pair stages (U, cost) per row
     // and model, sweeps (cost, acc)).
     const int WPR = Gp > 32 ? Gp / 32 : 1;  // warps per row
-    // (and, if rows are not whole 16-byte words, two 128-float buffers a warp in which its
-    // stores are put in order)
-    float *s_tr = reinterpret_cast<float *>(smem + tb);
-    QRec *s_q = reinterpret_cast<QRec *>(smem + tb + (I % 4 ? (size_t)blockDim.x * 32 : 0));  // [QT]
+    // (an affine source needs no tables: in their place each warp has two 128-float buffers in
+    // which its stores are put in order, if rows are not whole 16-byte words)
+    QRec *s_q = reinterpret_cast<QRec *>(smem + k2_head_bytes(c, blockDim.x));         // [QT]
     int4 *s_part = reinterpret_cast<int4 *>(s_q + QT);                                 // [NP][QT][WPR][2]
     // a sweep keeps the chunk's times [QT][4 Gp] instead of row partials, and per thread group
     // and instance the model (s_m4: -1 if the group's four differ)
@@ -535,11 +537,9 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
     const uint32_t ecst = 8u * (uint32_t)Gp;
     const uint32_t erow = 8u * 4u * (uint32_t)Gp, brow = 4u * 4u * (uint32_t)Gp;
     const uint32_t ebofs = (uint32_t)tile_enta_bytes(c);
-    // rows that are not whole 16-byte words: a warp puts its 128 elements of a row in order
-    // in shared memory and stores them coalesced; ntr of this lane's four lie in the pool
-    const bool tr = I % 4 != 0 && Gp >= 32;
-    const uint32_t trb = (uint32_t)__cvta_generic_to_shared(s_tr) + (threadIdx.x >> 5) * 1024u;
-    const int ntr = min(4, max(0, (I - (jb - 4 * lane) - lane + 31) >> 5));
+    const bool tr = AFF && I % 4 != 0 && Gp >= 32;
+    const uint32_t trb = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x >> 5) * 1024u;
+    const int ntr = min(4, max(0, (I - (jb - 4 * lane) - lane + 31) >> 5));  // of this lane's four, those in the pool
     if (SWEEP) {
         if (threadIdx.x < Gp) {
             bool one = true;
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
         // warps is described once per row, after the chunk, instead of by a lane of every warp
         constexpr bool DEFER = ROUTE && UNI && WIDE && !CON && !SWEEP;
         Inst4 r;
-        int r0[4], shift[4];
+        int r0[4], shift[4], la[4] = {0, 0, 0, 0};
         float T0[4], T1[4], X0[4], X1[4];  // entries 0 and 1 of the thread's instances (see the tile block)
         if (!AFF) {
             auto two = [&](int f, int v) { return pack2(__int_as_float(scal(f, 2 * v)), __int_as_float(scal(f, 2 * v + 1))); };
@@ -583,6 +583,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 shift[u] = scal(kScShift, u);
+                if (OUT & kOutIters) la[u] = scal(kScLa, u);
                 r0[u] = scal(kScR0, u);
                 const float2 e0 = lds_float2(ecol + u * ecst), e1 = lds_float2(ecol + u * ecst + (c.kph > 1 ? erow : 0u));
                 T0[u] = e0.x;
@@ -636,6 +637,7 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
             __syncthreads();
             float *orow = (OUT & kOutMatrix) ? a.ttft + (size_t)(q0 + qs) * I + jb : nullptr;
             const size_t ostep = (size_t)QS * I;
+            float *frow = (OUT & kOutIters) ? reinterpret_cast<float *>(a.first_batch) + (size_t)(q0 + qs) * I + jb : nullptr;
             const bool mat = AFF && a.src == kSrcMatrix;
             // a given matrix: its row is read one row ahead
             float tn[4];
@@ -654,7 +656,25 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                 }
             };
             if (AFF) read_row(qs);
-            uint32_t trw = trb;  // this row's buffer of the two
+            uint32_t trw = trb;  // the buffer of the two that is next
+            // four values of a row at p (v4: as one 16-byte word)
+            auto store4 = [&](float *p, bool v4, const float v[4]) {
+                if (v4) {
+                    __stcs(reinterpret_cast<float4 *>(p), make_float4(v[0], v[1], v[2], v[3]));
+                } else if (tr) {
+                    sts_f4(trw + 16u * lane, v[0], v[1], v[2], v[3]);
+                    __syncwarp();
+                    p -= 3 * lane;  // element `lane` of the warp's block
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (u < ntr) __stcs(p + 32 * u, lds_f32(trw + 4u * lane + 128u * u));
+                    trw ^= 512u;  // the other buffer: the next row's writes need not wait for these reads
+                } else if (nv > 0) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (u < nv) __stcs(p + u, v[u]);
+                }
+            };
             for (int rr = qs; rr < nrows; rr += QS) {
                 struct {
                     f32x2 fp2, ph2, pl2;
@@ -733,25 +753,16 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                     }
                 }
                 if (OUT & kOutMatrix) {
-                    if (UNI ? a.vec_ok != 0 : vec) {
-                        __stcs(reinterpret_cast<float4 *>(orow), make_float4(t[0], t[1], t[2], t[3]));
-                    } else if (tr) {
-                        sts_f4(trw + 16u * lane, t[0], t[1], t[2], t[3]);
-                        __syncwarp();
-                        float *ob = orow - 3 * lane;  // element `lane` of the warp's block
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (u < ntr) __stcs(ob + 32 * u, lds_f32(trw + 4u * lane + 128u * u));
-                        trw ^= 512u;  // the other buffer: the next row's writes need not wait for these reads
-                    } else {
-                        for (int u = 0; u < nv; ++u) __stcs(orow + u, t[u]);
-                    }
+                    store4(orow, UNI ? a.vec_ok != 0 : vec, t);
                     orow += ostep;
                 }
                 if (OUT & kOutIters) {
                     const bool bad = q.fp != q.fp;
-                    const size_t o = (size_t)(q0 + rr) * I + jb;
-                    for (int u = 0; u < nv; ++u) a.first_batch[o + u] = bad ? -1 : scal(kScLa, u) + kk[u] + off;
+                    float f[4];  // (the indices' bits)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) f[u] = __int_as_float(bad ? -1 : la[u] + kk[u] + off);
+                    store4(frow, UNI ? a.vec_first != 0 : a.vec_first && nv == 4, f);
+                    frow += ostep;
                 }
                 if (SWEEP) {
                     if (!UNI) {

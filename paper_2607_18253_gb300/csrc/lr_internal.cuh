@@ -281,6 +281,12 @@ __host__ __device__ inline size_t tile_bkt_bytes(const DevConfig &c) {
 __host__ __device__ inline size_t tile_bytes(const DevConfig &c) {
     return tile_ent_bytes(c) + tile_bkt_bytes(c) + (size_t)kScal * 4 * c.tgp * 4;
 }
+// The head of the candidate kernel's shared memory: the tile block, or (an affine source with
+// rows that are not whole 16-byte words) 1 KB a warp in which stores are put in order.
+__host__ __device__ inline size_t k2_head_bytes(const DevConfig &c, int block) {
+    const size_t tb = tile_bytes(c), ord = c.I % 4 != 0 && c.tgp >= 32 ? (size_t)block * 32 : 0;
+    return tb > ord ? tb : ord;
+}
 __host__ __device__ inline int tile_count(const DevConfig &c) { return (c.I + 4 * c.tgp - 1) / (4 * c.tgp); }
 // Byte offset of instance j's column within its tile block, and the tile's base.
 __host__ __device__ inline size_t tile_base(const DevConfig &c, int j) { return (size_t)(j / (4 * c.tgp)) * tile_bytes(c); }
@@ -424,6 +430,7 @@ struct K2Launch {
     // launch shape: Gp thread groups of four instances per row (a power of two up
     // to 32, else a multiple of 32), QS rows in flight, QT rows per staged chunk
     int32_t Gp, QS, QT, vec_ok;
+    int32_t vec_first;  // first_batch rows are whole, aligned 16-byte words
     int32_t pg;  // sweep: lanes per row (a power of two, the pairs up to 32)
     // TTFT source (kSrc*) and, for the average-case ones, the instance constants
     int32_t src;

@@ -48,9 +48,12 @@ def check(wl, sweep=5):
         rt.estimate_ttft(p, out=out)
         np.testing.assert_array_equal(bits(out.cpu().numpy()), bits(t32).ravel())
         assert (guard[:4 + shift] == -7.0).all() and (guard[4 + shift + Q * I:] == -7.0).all()
-    fb = torch.empty((Q, I), dtype=torch.int32, device="cuda")
-    rt.estimate_ttft(p, first_batch=fb)
-    np.testing.assert_array_equal(fb.cpu().numpy(), lt)
+    for shift in (0, 1):
+        guard = torch.full((Q * I + 8,), -7, dtype=torch.int32, device="cuda")
+        fb = guard[4 + shift:4 + shift + Q * I]
+        rt.estimate_ttft(p, first_batch=fb)
+        np.testing.assert_array_equal(fb.cpu().numpy(), lt.ravel())
+        assert (guard[:4 + shift] == -7).all() and (guard[4 + shift + Q * I:] == -7).all()
     if I > 1024:
         rt.close()
         return
