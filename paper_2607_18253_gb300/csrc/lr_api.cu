@@ -159,13 +159,15 @@ int pow2_ceil(int x) {
     return p;
 }
 
+constexpr size_t kK2SmemMax = 224 * 1024;
+
 // Launch shape of the candidate kernel: threads own four consecutive instances;
 // Gp groups per row (power of two up to 32, else a multiple of 32); the
-// summary tables of the tile and QT staged query rows fit the shared-memory
-// target.  Routing runs three 256-thread CTAs per SM (one of them fits beside a
-// snapshot load's CTA); the estimate alone runs one 512-thread CTA per SM, so
-// that each SM copies its tile block once.
-lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep) {
+// summary tables of the tile and QT staged query rows fit the shared memory.
+// Routing runs up to three CTAs of at most 256 threads per SM (one of them fits beside a
+// snapshot load's CTA); the estimate alone runs one of at most 512, so that each SM copies
+// its tile block once.
+lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep, size_t sm_smem) {
     lr_ctx::Shape s;
     s.block = route ? lr::kK2Block : lr::kK2EstBlock;
     const int G = (d.I + 3) / 4;
@@ -176,6 +178,7 @@ lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep) {
     }
     s.tiles = (d.I + 4 * s.Gp - 1) / (4 * s.Gp);
     s.QS = s.block / s.Gp;
+    s.block = s.QS * s.Gp;  // (threads beyond these would repeat rows)
     const int wpr = s.Gp > 32 ? s.Gp / 32 : 1;
     // the tile block (tables and per-instance scalars), brought in by one bulk copy
     lr::DevConfig dt = d;
@@ -187,14 +190,29 @@ lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep) {
     // staged row (32 B) and two raw copies of its prompt; routing adds the wide-row partials,
     // (cost, acc) per model, tau, and two raw copies of tau, dec_hat and acc
     const size_t per_row = 32 + 8 + (route ? part + (size_t)d.M * 8 + 4 + 8 + (size_t)d.M * 16 : 0);
-    const size_t target = route ? lr::kK2SmemTarget : lr::kK2EstSmemTarget;
-    const size_t room = target > fixed ? target - fixed : 0;
-    int qt = (int)std::min<size_t>(route ? 256 : 1024, room / per_row);
-    if (route && (size_t)qt * per_row + fixed > 200 * 1024) qt = 0;
+    // CTAs on an SM against rows in a chunk: the most CTAs (three to route, one to estimate) that
+    // hold eight rows each.  A chunk costs its CTA four barriers and the round trip of its rows'
+    // copies, so the row or two that the target leaves a pool of more than 256 instances are
+    // bound by those; past eight rows another CTA is worth more, above all beside a load.
+    // 16,384 queries x 384 / 512 / 576 / 1,024 instances, one pair, chunks of 2 / 2 / 1 / 1 rows ->
+    // these: 16.1 / 41.5 / 161 / 147 -> 14.1 / 12.9 / 43.7 / 31.4 us; estimates of 50,001 x 577
+    // / 1,021: 92.6 / 139 -> 26.4 / 36.0.  Three CTAs of 16 rows or two of 130 at 384 instances:
+    // 14.1 and 12.6 us alone, 23.6 and 26.1 beside a load; at 576 with wider budgets, three of
+    // 11 or two of 67: 28.5 and 29.0, 39.7 and 65.5.
+    constexpr int kLeastRows = 8;
+    int qt = 0;
+    for (int n = route ? 3 : 1; n >= 1 && qt < kLeastRows; --n) {
+        auto rows = [&](size_t bytes) {
+            return (int)std::min<size_t>(route ? 256 : 1024, bytes > fixed ? (bytes - fixed) / per_row : 0);
+        };
+        qt = n == (route ? 3 : 1) ? rows(route ? lr::kK2SmemTarget : lr::kK2EstSmemTarget) : 0;
+        // an SM's share of the shared memory, less what the system and the static words take
+        if (qt < 64) qt = rows(std::min<size_t>(kK2SmemMax, sm_smem / n - 1280));
+    }
     qt = std::max(s.QS, (qt / s.QS) * s.QS);
     s.QT = qt;
     s.smem = fixed + (size_t)qt * per_row;
-    s.ok = s.smem <= 224 * 1024;
+    s.ok = s.smem <= kK2SmemMax;
     return s;
 }
 
@@ -397,10 +415,14 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     // K1: one warp per instance.
     c->k1_smem = lr::kK1Warps * lr::trajectory_smem_per_warp(d);
     if (c->k1_smem > 200 * 1024) return bail(LR_ECAPACITY, "snapshot capacities too large for one K1 warp");
-    c->est = make_shape(d, false, false);
-    c->rt = make_shape(d, true, false);
-    c->sw = make_shape(d, true, true);
-    if (!c->est.ok) return bail(LR_ECAPACITY, "summary tables too large for shared memory");
+    int sm_smem = 0, dev = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    auto shape = [&](lr_ctx::Shape &s, bool route, bool sweep) {
+        s = make_shape(d, route, sweep, (size_t)sm_smem);
+        if (e == cudaSuccess && s.ok) e = lr::cand_occupancy(d.mode, route, s.block, s.smem, &s.occ);
+        s.occ = std::max(1, s.occ);
+    };
     c->k3_smem = lr::kK3Warps * lr::advance_smem_per_warp(d);
     // capacities lr_advance takes: 32 B a running and 12 B a waiting request within 200 KB
     // for four instances (it needs less)
@@ -408,17 +430,14 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     e = lr::set_k1_smem(c->k1_smem);
     if (e == cudaSuccess && c->k3_ok) e = lr::set_k3_smem(c->k3_smem);
     if (e == cudaSuccess && M <= lr::kCalMaxModels) e = lr::set_calib_smem(M);
-    if (e == cudaSuccess) e = lr::set_k2_smem(std::max({c->est.smem, c->rt.ok ? c->rt.smem : 0, c->sw.ok ? c->sw.smem : 0}));
+    if (e == cudaSuccess) e = lr::set_k2_smem(kK2SmemMax);
     c->bl_ok = lr::baseline_smem(d) <= 200 * 1024;
     if (e == cudaSuccess && c->bl_ok) e = lr::set_baseline_smem(lr::baseline_smem(d));
-    if (e == cudaSuccess) e = lr::cand_occupancy(d.mode, false, c->est.block, c->est.smem, &c->est.occ);
-    if (e == cudaSuccess && c->rt.ok) e = lr::cand_occupancy(d.mode, true, c->rt.block, c->rt.smem, &c->rt.occ);
+    shape(c->est, false, false);
+    shape(c->rt, true, false);
+    shape(c->sw, true, true);
     if (e != cudaSuccess) return bail(LR_ECUDA, cudaGetErrorString(e));
-    c->est.occ = std::max(1, c->est.occ);
-    c->rt.occ = std::max(1, c->rt.occ);
-    if (c->sw.ok) e = lr::cand_occupancy(d.mode, true, c->sw.block, c->sw.smem, &c->sw.occ);
-    if (e != cudaSuccess) return bail(LR_ECUDA, cudaGetErrorString(e));
-    c->sw.occ = std::max(1, c->sw.occ);
+    if (!c->est.ok) return bail(LR_ECAPACITY, "summary tables too large for shared memory");
     *out = c;
     return LR_OK;
 }
@@ -564,6 +583,8 @@ int lr_route(lr_ctx *c, int32_t Q, const int32_t *prompt_len, const int32_t *dec
     }
     if (Q == 0) return LR_OK;
     if (!prompt_len || !dec_hat || !acc || !assign_out || !util_out) return fail(c, LR_EINVAL, "null array");
+    const lr_ctx::Shape &sh = P > 1 ? c->sw : c->rt;
+    if (!sh.ok) return fail(c, LR_ECAPACITY, "routing needs num_instances <= 1024 and its tiles in shared memory");
     float *kv_matrix = nullptr;
     bool leaders = false;
     if (c->kv_on) {
@@ -598,8 +619,6 @@ int lr_route(lr_ctx *c, int32_t Q, const int32_t *prompt_len, const int32_t *dec
             a.lead_order = c->kv_order;
         }
     }
-    const lr_ctx::Shape &sh = P > 1 ? c->sw : c->rt;
-    if (!sh.ok) return fail(c, LR_ECAPACITY, "routing needs num_instances <= 1024 and its tiles in shared memory");
     a.Gp = sh.Gp;
     a.QS = sh.QS;
     a.QT = sh.QT;

@@ -93,6 +93,62 @@ def test_instance_counts(I, mode):
     check(wl)
 
 
+@pytest.mark.parametrize("I,Q", [(33, 9000), (257, 5000), (384, 4001), (513, 3000), (640, 2500), (1000, 1500), (1023, 700),
+                                 (1024, 65), (3001, 300)])
+def test_chunks_and_claims_of_wide_pools(I, Q):
+    # calls of several chunks of rows a CTA and of less than one, on the load's stream (equal
+    # parts) and on another one (parts and claims): the same results, those of the oracle where
+    # sampled, and the average-case source's, whose ragged rows are put in order in shared memory
+    wl = W.small_workload(7 + I, num_instances=I, num_models=3, num_queries=Q, budget_range=(64, 128), min_gap=48)
+    rt = R().LatencyRouter.from_workload(wl)
+    rt.load_state(*R().state_tensors(wl))
+    p, dh, acc, tau = R().query_tensors(wl)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def calls(stream):
+        with torch.cuda.stream(stream):
+            fb = torch.empty((Q, I), dtype=torch.int32, device="cuda")
+            o = [rt.estimate_ttft(p, first_batch=fb), fb]
+            if I <= 1024:
+                for mu, tt, m in ((wl.mu, None, None), (wl.mu, None, torch.empty((Q, I), device="cuda")), (None, tau, None)):
+                    r = rt.route(p, dh, acc, wl.lam, mu, tau=tt, ttft_matrix=m)
+                    o += [r[k] for k in sorted(r)]
+        torch.cuda.synchronize()
+        return [x.cpu().numpy() for x in o]
+
+    one, two = calls(torch.cuda.current_stream()), calls(side)
+    for a, b in zip(one, two):
+        np.testing.assert_array_equal(a.view(np.uint8), b.view(np.uint8))
+    t = one[0]
+    rng = np.random.default_rng(I)
+    cq, cj = rng.integers(0, Q, 2000), rng.integers(0, I, 2000)
+    _, lt, t32, _ = oracle.estimate_candidates(wl, cq, cj)
+    np.testing.assert_array_equal(bits(t[cq, cj]), bits(t32))
+    np.testing.assert_array_equal(one[1][cq, cj], lt)
+    if I <= 1024:
+        for k, tt in ((2, None), (5, None), (9, wl.tau)):
+            a, u, tc = oracle.route(wl, t, tau=tt)
+            got = dict(zip(("assign", "ttft_chosen", "util") if k != 5 else ("assign", "ttft_chosen", "ttft_matrix", "util"),
+                           one[k:k + 4]))
+            np.testing.assert_array_equal(got["assign"], a)
+            np.testing.assert_array_equal(bits(got["util"]), bits(u))
+            np.testing.assert_array_equal(bits(got["ttft_chosen"]), bits(tc))
+            if k == 5:
+                np.testing.assert_array_equal(bits(got["ttft_matrix"]), bits(t))
+    service = rng.uniform(2.0, 4.0, I)
+    theta, tdec, alpha = rng.uniform(3e3, 4e4, I), rng.uniform(0.004, 0.06, I), service * rng.uniform(0.3, 0.95, I)
+    k = rng.integers(1, 64, I).astype(np.int32)
+    rt.set_queue_params(theta, tdec, alpha, service, k)
+    rt.set_ttft_source(R().LR_TTFT_LPS)
+    want = oracle.avgcase_matrix(wl, np.array([oracle.lps_wait(*x) for x in zip(alpha, service, k.tolist())]), theta, tdec)[0]
+    guard = torch.full((Q * I + 8,), -7.0, device="cuda")
+    rt.estimate_ttft(p, out=guard[4:4 + Q * I])
+    assert rt.status() == R().LR_OK and (guard[:4] == -7.0).all() and (guard[4 + Q * I:] == -7.0).all()
+    np.testing.assert_array_equal(bits(guard[4:4 + Q * I].cpu().numpy()), bits(want).ravel())
+    rt.close()
+
+
 @pytest.mark.parametrize("I", [12, 128, 256])
 @pytest.mark.parametrize("grouped", [False, True])
 def test_models_of_a_thread(I, grouped):
