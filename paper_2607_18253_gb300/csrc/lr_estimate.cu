@@ -295,14 +295,16 @@ struct Flag {
 // at a time.  CTA b < first_ctas starts with the static range [b F, (b + 1) F)
 // (F = first_rows, most of its share of the rows): those CTAs fit beside a snapshot
 // load's CTAs running on another stream and start at once.  The remaining rows are
-// claimed from the tile's counter, which counts the rows past the static ones: QT
-// rows while many are left, down to 4 QS at the end (a claim's atomic still returns
-// well within the chunk before it).  So CTAs that start late (their SM busy with the
+// claimed from the tile's counter, which counts the rows past the static ones: an equal
+// share of those left, to route half of one (65,536 x 256 beside a load 33.0 -> 30.8 us, with
+// deadlines 47 -> 40; an estimate of 16,384, with fewer and wider CTAs, takes 14.4 us with
+// whole shares and 16.1 with halves), at most QT, down to a.least at the end (a claim's
+// atomic still returns well within the chunk before it).  So CTAs that start late (their SM busy with the
 // load) or run slower take less, and all finish at about the same time.  `seen` is
 // a row index recently reached.
 __device__ __forceinline__ int claim_size(const K2Launch &a, int seen) {
-    const int n = (a.Q - seen) / (int)gridDim.x;
-    return min(a.QT, max(4 * a.QS, n - n % a.QS));
+    const int n = (a.Q - seen) / (a.share * (int)gridDim.x);
+    return min(a.QT, max(a.least, n - n % a.QS));
 }
 __device__ __forceinline__ int static_rows(const K2Launch &a) { return min(a.Q, a.first_ctas * a.first_rows); }
 // Every row of the launch lies in a static range: no CTA claims, and the counters stay
