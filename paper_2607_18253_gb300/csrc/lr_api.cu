@@ -200,7 +200,10 @@ lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep, size_t 
     // / 1,021: 92.6 / 139 -> 26.4 / 36.0.  Three CTAs of 16 rows or two of 130 at 384 instances:
     // 14.1 and 12.6 us alone, 23.6 and 26.1 beside a load; at 576 with wider budgets, three of
     // 11 or two of 67: 28.5 and 29.0, 39.7 and 65.5.
-    constexpr int kLeastRows = 8;
+    // (A sweep's rows hold their times as well, and its chunks have more work: four rows.  512
+    // instances x 32,768 queries x 2 / 8 / 64 pairs, two CTAs of 6 rows or one of 56: 63 and 47 us,
+    // 107 and 112, 429 and 561; beside a load's stream 68 and 55, 111 and 132, 432 and 653.)
+    const int kLeastRows = sweep ? 4 : 8;
     int qt = 0;
     for (int n = route ? 3 : 1; n >= 1 && qt < kLeastRows; --n) {
         auto rows = [&](size_t bytes) {
@@ -242,6 +245,34 @@ int set_row_split(lr::K2Launch &a, const lr_ctx *c, int ctas, int tiles, int occ
     const int f = (int)((long long)a.Q * 9 / (10LL * std::max(1, ctas)));
     a.first_rows = std::max(a.QS, f - f % a.QS);
     return ctas;
+}
+
+// How a sweep's warps share the (row, pair, instance) work of a chunk: pg lanes by pair, sp
+// lanes that split a row's instances (and exchange their best in log2(sp) rounds), the other
+// lanes by row.  Lanes by pair read a word together, lanes by instance neighbouring words, lanes
+// by row the same banks; but pg lanes store as many pieces of the outputs.  The split of the
+// least cost is taken, in steps of four candidates: the longer of the units that a warp takes
+// one after the other (a step waits for 14 times its issue) and of what the SM's warps issue
+// together.  Fitted to all splits of 28 calls of 2 to 64 pairs on 8 to 1,024 instances, of
+// which it takes the fastest or one within 5%.  One lane per (row, pair) whatever the call left
+// a chunk of few pairs to one warp in eight: 32,768 queries x 2 pairs on 256 / 512 / 1,024
+// instances 40 / 576 / 4,197 us, now 23 / 45 / 110.
+void set_sweep_lanes(lr::K2Launch &a, int I, int warps, int ctas, int ctas_sm) {
+    const int rows = std::min(a.QT, (a.Q + ctas - 1) / ctas), G = (I + 3) / 4;
+    double least = 0.0;
+    for (int pg = 1; pg <= std::min(32, pow2_ceil(a.P)); pg *= 2)
+        for (int sp = 1, lg = 0; pg * sp <= 32 && sp <= pow2_ceil(G); sp *= 2, ++lg) {
+            const int rw = 32 / (pg * sp);
+            const double units = (double)((rows + rw - 1) / rw) * ((a.P + pg - 1) / pg);
+            const int conflicts = std::max(0, std::min(a.Gp, 8) / (pg * sp) - 1);
+            const double steps = (G + sp - 1) / sp * (1.0 + 0.1 * conflicts);
+            const double cost = std::max(14.0 * std::ceil(units / warps) * (steps + 4.0 + 0.25 * lg),
+                                         ctas_sm * units * (steps + 2.0 + 0.5 * lg + 0.1 * pg));
+            if (least > 0.0 && cost >= least) continue;
+            least = cost;
+            a.pg = pg;
+            a.sp = sp;
+        }
 }
 
 lr::K2Launch k2_base(const lr_ctx *c) {
@@ -635,10 +666,10 @@ int lr_route(lr_ctx *c, int32_t Q, const int32_t *prompt_len, const int32_t *dec
     a.QT = sh.QT;
     a.least = sh.least;
     a.share = 2;
-    a.pg = std::min(32, pow2_ceil(P));
     a.vec_ok = (c->cfg.I % 4 == 0) && ((uintptr_t)(kv_matrix ? kv_matrix : a.ttft) % 16 == 0);
     dim3 grid(std::min(c->sms * sh.occ, (Q + a.QS - 1) / a.QS), 1);
     grid.x = set_row_split(a, c, (int)grid.x, 1, sh.occ, stream);
+    if (P > 1) set_sweep_lanes(a, c->cfg.I, sh.block / 32, (int)grid.x, std::min(sh.occ, ((int)grid.x + c->sms - 1) / c->sms));
     cudaError_t e = lr::launch_cand(a, lr::cand_out_flags(a.ttft != nullptr, false, true, tau != nullptr, P), grid,
                                     sh.block, sh.smem, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "route launch");

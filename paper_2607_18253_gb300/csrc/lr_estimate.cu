@@ -861,18 +861,26 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                 }
             }
             if (SWEEP) {
-                // A lane per (row, pair): each follows the pool's times of its row in instance
-                // order, so a candidate of a pair costs a packed multiply-add and a running
-                // maximum, with no reduction across lanes and no row-by-row winner (a lane per
-                // four instances and one pair after the other took about 120 warp instructions
-                // per row and pair).  32 pairs x 4,096 queries x 64 instances: kernel 17.3 -> 12.0 us.
+                // A lane per (row, pair), or several that split the row's instances (set_sweep_lanes):
+                // each follows the pool's times of its row in instance order, so a candidate of a
+                // pair costs a packed multiply-add and a running maximum, with no reduction per
+                // row (a lane per four instances and one pair after the other took about 120 warp
+                // instructions per row and pair).  32 pairs x 4,096 queries x 64 instances: kernel
+                // 17.3 -> 12.0 us.
                 __syncthreads();
-                const int pg = a.pg, rw = 32 / pg, np = (a.P + 31) / 32;
-                const int pl = lane & (pg - 1), rs = lane / pg;
-                const int units = (nrows + rw - 1) / rw * np;
-                for (int un = threadIdx.x >> 5; un < units; un += blockDim.x >> 5) {
-                    const int row = un / np * rw + rs, pp = un % np * 32 + pl;
-                    const bool act = row < nrows && pp < a.P;
+                const int pg = a.pg, sp = a.sp, rw = 32 / (pg * sp), np = (a.P + pg - 1) / pg;
+                const int pl = lane & (pg - 1), sl = lane / pg & (sp - 1), rs = lane / (pg * sp);
+                const int nw = blockDim.x >> 5, w0 = threadIdx.x >> 5;
+                const int drow = nw / np * rw, dpr = nw % np;  // the next unit: rows and blocks of pairs on
+                for (int r0 = w0 / np * rw, pb = w0 % np; r0 < nrows;) {
+                    const int row = r0 + rs, pp = pb * pg + pl;
+                    r0 += drow;
+                    pb += dpr;
+                    if (pb >= np) {
+                        pb -= np;
+                        r0 += rw;
+                    }
+                    const bool act = row < nrows && pp < a.P && sl == 0;
                     const int rr = min(row, nrows - 1);
                     const float2 lm = s_lm[min(pp, a.P - 1)];
                     const f32x2 nm = pack2(lm.y, lm.y);
@@ -904,14 +912,37 @@ __global__ void __launch_bounds__((OUT & (kOutLag | kOutCon | kOutSweep)) ? kK2B
                         unpack2(fma2(nm, pack2(t4.z, t4.w), pack2(U4[2], U4[3])), J[2], J[3]);
                     };
                     float U4[4], J[4];
-                    for (int gg = 0; 4 * gg < I; ++gg) {
-                        objectives(gg, U4, J);
-                        const float m1 = fmaxf(fmaxf(J[0], J[1]), fmaxf(J[2], J[3]));  // NaN only if all are
-                        if (m1 > best || (bg < 0 && m1 == m1)) {
-                            best = m1;
-                            bg = gg;
+                    auto walk = [&](int first, int step) {
+                        for (int gg = first; 4 * gg < I; gg += step) {
+                            objectives(gg, U4, J);
+                            const float m1 = fmaxf(fmaxf(J[0], J[1]), fmaxf(J[2], J[3]));  // NaN only if all are
+                            if (m1 > best) {
+                                best = m1;
+                                bg = gg;
+                            }
+                        }
+                    };
+                    if (sp == 1) {
+                        walk(0, 1);  // (a step the compiler knows: 32,768 x 256 x 64 pairs 170 -> 153 us)
+                    } else {
+                        walk(sl, sp);
+                        // the best of the lanes that share the instances, the lowest group among equals
+                        for (int o = pg; o < pg * sp; o <<= 1) {
+                            const float b2 = __shfl_xor_sync(kFull, best, o);
+                            const int g2 = __shfl_xor_sync(kFull, bg, o);
+                            if (b2 > best || (b2 == best && (unsigned)g2 < (unsigned)bg)) {
+                                best = b2;
+                                bg = g2;
+                            }
                         }
                     }
+                    if (bg < 0)  // none above -inf: the first that is not NaN, if any
+                        for (int gg = 0; 4 * gg < I && bg < 0; ++gg) {
+                            objectives(gg, U4, J);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (J[u] == J[u]) bg = gg;
+                        }
                     if (act) {
                         Cand w = {0u, 0, 0.f, 0.f};
                         if (bg >= 0) {

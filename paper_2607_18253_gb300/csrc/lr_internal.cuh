@@ -432,7 +432,7 @@ struct K2Launch {
     int32_t Gp, QS, QT, vec_ok;
     int32_t vec_first;  // first_batch rows are whole, aligned 16-byte words
     int32_t least, share;  // a claim: the fewest rows, and 1 / share of an equal part of those left
-    int32_t pg;  // sweep: lanes per row (a power of two, the pairs up to 32)
+    int32_t pg, sp;  // sweep: lanes by pair and lanes that share a row's instances (powers of two)
     // TTFT source (kSrc*) and, for the average-case ones, the instance constants
     int32_t src;
     const QueueDev *qd;

@@ -169,6 +169,38 @@ def test_sweep_lane_splits(P):
           sweep=P)
 
 
+@pytest.mark.parametrize("I", [1, 9, 66, 130, 256, 700, 1024])
+@pytest.mark.parametrize("Q", [3, 300, 4000])
+def test_sweep_splits_the_instances(I, Q):
+    # calls of few and many pairs and rows, whose warps split rows, pairs and a row's instances in
+    # different ways; equal replicas (ties go to the lowest instance, across lanes too) and an
+    # invalid prompt
+    if I * Q > 1_200_000:
+        Q = 1100
+    wl = W.small_workload(9 + I, num_instances=I, num_models=3, num_queries=Q, budget_range=(64, 64), min_gap=48)
+    wl = dataclasses.replace(wl, max_seqs=np.full(I, 8, np.int32), n_run=np.minimum(wl.n_run, 8),
+                             model_of_instance=(np.arange(I) // 2 * 2 % 3).astype(np.int32))
+    for a in (wl.n_run, wl.run_ctx, wl.run_pre, wl.run_dec, wl.n_wait, wl.wait_pre, wl.wait_dec):
+        a[1::2] = a[0::2][:a[1::2].shape[0]]
+    wl.prompt_len[Q // 2] = 0
+    rt = R().LatencyRouter.from_workload(wl, max_pairs=64)
+    rt.load_state(*R().state_tensors(wl))
+    p, dh, acc, _ = R().query_tensors(wl)
+    t = rt.estimate_ttft(p).cpu().numpy()
+    assert rt.status() == R().LR_EINVAL and np.isnan(t[Q // 2]).all()
+    for P in (2, 3, 16, 64):
+        lam, mu = np.linspace(0.0, 3.0, P).astype(np.float32), np.geomspace(1e-3, 1.0, P).astype(np.float32)
+        o = rt.route(p, dh, acc, lam, mu)
+        a, u, tc = oracle.route(wl, t, lam=lam, mu=mu)
+        assert rt.status() == R().LR_EINVAL
+        np.testing.assert_array_equal(o["assign"].cpu().numpy(), a)
+        ok = a >= 0
+        np.testing.assert_array_equal(bits(o["util"].cpu().numpy()[ok]), bits(u[ok]))
+        np.testing.assert_array_equal(bits(o["ttft_chosen"].cpu().numpy()[ok]), bits(tc[ok]))
+        assert np.isnan(o["util"].cpu().numpy()[~ok]).all() and np.isnan(o["ttft_chosen"].cpu().numpy()[~ok]).all()
+    rt.close()
+
+
 @pytest.mark.parametrize("I", [5, 45, 200])
 @pytest.mark.parametrize("P", [1, 2, 5, 33])
 def test_objectives_beyond_fp32(I, P):
