@@ -317,11 +317,12 @@ __global__ void __launch_bounds__(kCalThreads, 1) k_calibrate(long long N, const
     const int lane = threadIdx.x & 31;
     unsigned char *stages = cal_smem + cal_sums_bytes(M);
     __shared__ __align__(8) unsigned long long s_mbar[kCalStagesMax];
-    __shared__ int s_last;
+    __shared__ int s_last, s_work;
     __shared__ long long s_none[kCalCols + 1];  // a row that adds nothing: constant 1, then zeros
     unsigned int *done = reinterpret_cast<unsigned int *>(acc + 2 * (size_t)M * kCalAcc);
     for (int i = threadIdx.x; i < M * (kCalAcc + kCalFlushSums) * 2; i += blockDim.x) sacc[i] = 0ull;
     if (threadIdx.x < kCalCols + 1) s_none[threadIdx.x] = threadIdx.x == 0 ? 1 : 0;
+    if (threadIdx.x == 0) s_work = 0;
     unsigned long long g[15], bl[5], bh[5];  // 64-bit sums since the last flush
     int nfast = 0, cur = -1;
     bool bad = false;
@@ -584,16 +585,25 @@ __global__ void __launch_bounds__(kCalThreads, 1) k_calibrate(long long N, const
             }
         } else {
             // A log whose rows are in the order they ran mixes the models, and a lane that
-            // meets another model has its warp flush.  The first tile's model changes decide
-            // for the slice: with one in 32 rows or more, each tile's rows are first listed by
-            // model (a counting sort of their indexes; the sums are exact, so any order will
-            // do), and each warp takes the rows of the models it owns: the warps are dealt out
-            // by the models' rows in a tile, again when a warp's share grows fourfold.
-            // 1M rows of 4 / 8 / 12 / 40 models in random order: 85 / 136 / 185 / 343 us with
-            // flushes alone, 44 / 44 / 46 / 89 this way.  The line is where the two meet: 1M rows
-            // of 8 models in runs of 16 rows 49 us with flushes, 31 listed; in runs of 32 rows
-            // (a change in 37) 35 and 39, of 64 35 and 44.  2 models, runs of 16 and 32 rows: 42
-            // and 30 with flushes, 28 and 28 listed.
+            // meets another model has its warp flush, once for each model its lanes hold.  Where
+            // that is much, each tile's rows are first listed by model (a counting sort of their
+            // indexes; the sums are exact, so any order will do), and each warp takes the rows of
+            // the models it owns: the warps are dealt out by the models' rows in a tile, again
+            // when a warp's share grows fourfold.  2M rows of 8 / 12 / 40 models in random order:
+            // 260 / 360 / 679 us with flushes alone, 56 / 57 / 145 this way.
+            // The slice's first tile decides.  `per` is the flushes a warp would make in a tile,
+            // about a microsecond each: for each of its two rows a lane as many as the models of
+            // the warp's rows, if a lane's two rows differ (rows that take turns, so that each
+            // lane meets one model, cost none but the last), and those of the end.  Listing costs
+            // two to three, or, with more models than warps, flushes as well, of every model in
+            // the tile by some warp, and the more so where one model has most rows and the others
+            // crowd the last warps.  (The slowest slice sets the time, so the lines keep clear of
+            // what chance moves a tile by.)  2M rows, flushes / listed: 2 models in runs of 16 rows
+            // (per 2.3) 76 / 50 us, 8 in runs of 32 (2.0) 66 / 49, 12 in random runs of 64 (1.9)
+            // 65 / 106; 40 models in turn (0.1) 58 / 139, runs of 8 in turn (8) 154 / 121, random runs
+            // of 16 (4) 98 / 159; 64 and 128 models in runs of 8 and 4 (8, 16) 157 / 247, 279 /
+            // 445, of 2 (32) 491 / 206, 501 / 359; skewed counts of 16 / 40 / 128 models (16 to
+            // 18) 276 / 179, 308 / 419, 330 / 802.
             auto consumers = [&]() {
                 __syncwarp();
                 asm volatile("bar.sync 1, %0;" ::"n"(kCalConsumerWarps * 32) : "memory");
@@ -622,13 +632,25 @@ __global__ void __launch_bounds__(kCalThreads, 1) k_calibrate(long long N, const
             // are bounded too)
             failed = !__all_sync(kFull, landed());
             const int32_t *m0 = reinterpret_cast<const int32_t *>(stages + kFeat + kTime);
-            const unsigned change = !failed && ja + 1 < left && m0[ja] != m0[ja + 1];
-            unsigned changes;
-            asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %1, 0;\n bar.red.popc.u32 %0, 1, %2, p;\n}"
-                         : "=r"(changes)
-                         : "r"(change), "n"(kCalConsumerWarps * 32)
-                         : "memory");
-            const bool mixed = (int)changes * 32 > min(kCalConsumerWarps * 32, left);
+            const bool va = !failed && ja < left;
+            const int xa = va ? m0[ja] : -1, xb = va && jb < left ? m0[jb] : xa;
+            const unsigned same = __match_any_sync(kFull, xa);
+            const int kinds = __popc(__ballot_sync(kFull, va && (same & lt) == 0u));
+            const bool moves = __any_sync(kFull, xa != xb);
+            if (lane == 0) atomicAdd(&s_work, moves ? 2 * ntiles * kinds : kinds);
+            consumers();
+            const float per = (float)s_work / (float)(min(kCalConsumerWarps, (left + 31) / 32) * ntiles);
+            bool mixed = per >= (M > kCalConsumerWarps ? 4.f : 2.5f);
+            if (mixed && M > kCalConsumerWarps) {
+                if (va && xa >= 0 && xa < M) atomicAdd(&s_cnt[1][xa], 1);
+                if (va && jb < left && xb >= 0 && xb < M) atomicAdd(&s_cnt[1][xb], 1);
+                consumers();
+                const int4 c = reinterpret_cast<const int4 *>(s_cnt[1])[lane];  // (cleared with the first tile)
+                const int n = __reduce_add_sync(kFull, (c.x > 0) + (c.y > 0) + (c.z > 0) + (c.w > 0));
+                const int most = __reduce_max_sync(kFull, max(max(c.x, c.y), max(c.z, c.w)));
+                const bool skewed = most * kCalConsumerWarps > 4 * min(left, kCalTile);
+                if (n > kCalConsumerWarps) mixed = per >= (0.7f + 0.18f * (float)n) * (skewed ? 3.5f : 1.f);
+            }
             if (!mixed) {
                 for (; left > 0 && !failed; release()) {
                     if (!landed()) {

@@ -173,3 +173,25 @@ def test_mixed_models(M, N, drift):
         np.testing.assert_array_equal(got, ref)
         if N // M > 100:
             np.testing.assert_allclose(got, oracle.calibrate(F, m, t, M, shared_beta1=shared), rtol=RTOL)
+
+
+@pytest.mark.parametrize("M,N,run", [(2, 200_000, 1), (8, 150_001, 4), (8, 961, 8), (12, 2_000, 16), (15, 480, 1), (16, 300_002, 4),
+                                     (16, 300_002, 1), (40, 150_000, 8), (40, 300_001, 1), (64, 200_001, 2), (128, 1_000, 8),
+                                     (128, 160_003, 16), (128, 500_000, 2)])
+@pytest.mark.parametrize("skewed", [False, True])
+def test_models_in_turn(M, N, run, skewed):
+    # runs of a model in turn (with runs that divide the rows a step takes, every lane meets one
+    # model alone), on both sides of the rule that lists a tile by model, and counts in which one
+    # model has half of the rows.  Bit for bit the fit of the same rows grouped by model.
+    F, _, t = W.batch_log(N, M, seed=M + run, coef=coef_of(M, M), noise=0.03)
+    m = (np.arange(N) // run % M).astype(np.int32)
+    if skewed:
+        rng = np.random.default_rng(M + run)
+        m = np.repeat(np.minimum(rng.pareto(1.0, N // run + 1).astype(np.int32), M - 1), run)[:N]
+    rt = router_for(M)
+    order = np.argsort(m, kind="stable")
+    got = rt.calibrate(dev(F), dev(m), dev(t), shared_beta1=True).cpu().numpy()
+    assert rt.status() == R().LR_OK
+    ref = rt.calibrate(dev(F[order]), dev(m[order]), dev(t[order]), shared_beta1=True).cpu().numpy()
+    np.testing.assert_array_equal(got, ref)
+    rt.close()
