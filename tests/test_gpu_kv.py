@@ -414,24 +414,38 @@ def test_full_size_sampled(name):
     assert not np.isnan(t).any()
 
 
+def check_sampled(got, wl, limits, cq, cj):
+    st, eF, elt, et, _ = oracle.estimate_matrix_kv(wl, *limits, cand_q=cq, cand_j=cj)
+    t, fb, F = got
+    compare((t[cq, cj], fb[cq, cj], F[cq, cj]), (eF, elt, et), st == 0)
+    assert np.isnan(t[cq, cj][st != 0]).all()
+
+
 def test_prompt_bound_beyond_exact_buckets():
     # a prompt bound above 2^16 - 2: the sort buckets group several lengths, so
-    # every query is estimated (in sorted order) instead of one per length
-    wl = W.small_workload(65, num_instances=10, num_models=2, num_queries=60, max_prompt_len=150_000,
+    # every query is estimated (in sorted order) instead of one per length.  20,000 queries on 10
+    # instances: more than a call walks without the sort.
+    wl = W.small_workload(65, num_instances=10, num_models=2, num_queries=20_000, max_prompt_len=150_000,
                           budget_range=(6000, 8192), min_gap=4096)
     p = wl.prompt_len.copy()
     p[:6] = (1, 1, 150_000, 150_000, 65_535, 65_536)  # duplicates and bucket edges
     wl.prompt_len = p
     limits = W.kv_limits(wl, 12, block_sizes=(16, 64))
-    check(wl, limits)
+    rt = make(wl, limits)
+    got = gpu_estimate(rt, wl)
+    rt.close()
+    rng = np.random.default_rng(3)
+    cq = np.concatenate([np.repeat(np.arange(6), 10), rng.integers(0, 20_000, 1500)])
+    cj = np.concatenate([np.tile(np.arange(10), 6), rng.integers(0, 10, 1500)])
+    check_sampled(got, wl, limits, cq, cj)
 
 
 def test_many_duplicate_lengths():
-    # 2,000 queries over 40 distinct prompt lengths: most rows are copies of the
-    # row of the first query with the same length
-    wl = W.small_workload(66, num_instances=12, num_models=2, num_queries=2000, budget_range=(8, 96), min_gap=8)
+    # 20,000 queries over 40 distinct prompt lengths (sorted: more than a call walks directly):
+    # most rows are copies of the row of the first query with the same length
+    wl = W.small_workload(66, num_instances=12, num_models=2, num_queries=20_000, budget_range=(8, 96), min_gap=8)
     rng = np.random.default_rng(0)
-    wl.prompt_len = rng.choice(np.arange(1, 161, 4, dtype=np.int32), 2000)
+    wl.prompt_len = rng.choice(np.arange(1, 161, 4, dtype=np.int32), 20_000)
     limits = W.kv_limits(wl, 13, block_sizes=(4,))
     rt = make(wl, limits)
     p = torch.from_numpy(np.ascontiguousarray(wl.prompt_len, np.int32)).cuda()
@@ -440,13 +454,53 @@ def test_many_duplicate_lengths():
     assert rt.status() == R().LR_OK
     rt.close()
     np.testing.assert_array_equal(bits(t_only), bits(got[0]))
-    st, eF, elt, et, _ = oracle.estimate_matrix_kv(wl, *limits)
-    compare(got, (eF, elt, et), st == 0)
+    # every length on every instance against the oracle, and every row equal to its length's first
+    lengths, first, inverse = np.unique(wl.prompt_len, return_index=True, return_inverse=True)
+    check_sampled(got, wl, limits, np.repeat(first, 12), np.tile(np.arange(12), len(lengths)))
+    for x in got:
+        np.testing.assert_array_equal(x, x[first[inverse]])
+
+
+@pytest.mark.parametrize("I", [11, 12])
+@pytest.mark.parametrize("bound", [160, 100_000])
+def test_route_without_a_matrix_reads_one_row_per_length(I, bound):
+    # enough queries for the sort: a route that returns no matrix reads the row of the first query
+    # of each length (with a prompt bound above 2^16 - 2, its own), with duplicate and invalid
+    # lengths among them; the same picks as with the matrix, which the oracle routes on
+    Q, P = 20_000, 5
+    wl = W.small_workload(68 + I, num_instances=I, num_models=3, num_queries=Q, max_prompt_len=bound,
+                          budget_range=(8, 96) if bound == 160 else (6000, 8192), min_gap=8 if bound == 160 else 4096)
+    limits = W.kv_limits(wl, 14, block_sizes=(4, 16))
+    wl.prompt_len[7::97] = wl.prompt_len[3]
+    wl.prompt_len[[0, 11, 500, Q - 1]] = (0, -5, bound + 1, 0)
+    rt = make(wl, limits, max_pairs=P)
+    p, dh, acc, tau = R().query_tensors(wl)
+    lam, mu = np.linspace(0.2, 2.0, P).astype(np.float32), np.geomspace(1e-2, 1.0, P).astype(np.float32)
+    for l, m, tt in ((lam[:1], mu[:1], None), (lam[:1], None, tau), (lam, mu, None)):
+        mat = torch.empty((Q, I), device="cuda")
+        a = rt.route(p, dh, acc, l, m, tau=tt)
+        b = rt.route(p, dh, acc, l, m, tau=tt, ttft_matrix=mat)
+        assert rt.status() == R().LR_EINVAL
+        for k in ("assign", "util", "ttft_chosen"):
+            np.testing.assert_array_equal(a[k].cpu().numpy().view(np.uint32), b[k].cpu().numpy().view(np.uint32))
+        ea, eu, et = oracle.route(wl, mat.cpu().numpy(), lam=l, mu=m, tau=None if tt is None else wl.tau)
+        np.testing.assert_array_equal(a["assign"].cpu().numpy(), ea)
+        ok = ea >= 0
+        assert not ok[:, [0, 11, 500, Q - 1]].any()
+        np.testing.assert_array_equal(bits(a["util"].cpu().numpy()[ok]), bits(eu[ok]))
+        np.testing.assert_array_equal(bits(a["ttft_chosen"].cpu().numpy()[ok]), bits(et[ok]))
+    # the matrix itself at sampled candidates
+    t = mat.cpu().numpy()
+    rng = np.random.default_rng(I)
+    cq, cj = rng.integers(1, 400, 600), rng.integers(0, I, 600)
+    st, _, _, want, _ = oracle.estimate_matrix_kv(wl, *limits, cand_q=cq, cand_j=cj)
+    np.testing.assert_array_equal(bits(t[cq, cj][st == 0]), bits(want[st == 0]))
+    rt.close()
 
 
 def test_hand_trace_with_residents_preempting_each_other():
     # the worked trace of tests/golden/kv_hand_trace_residents.json on the GPU: one
-    # instance, the query of the trace twice (one walk, a copied row) and a longer one
+    # instance, the query of the trace twice and a longer one
     import json
     import os
     g = json.load(open(os.path.join(os.path.dirname(__file__), "golden", "kv_hand_trace_residents.json")))
