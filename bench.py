@@ -16,7 +16,8 @@ e2e        = same metric through the public API from pinned host buffers, with t
 roofline   = the SFS estimate call (lr_estimate_ttft, the full Q x I matrix) on the same
              workload against measured HBM bandwidth; per-kernel figures of the step
              (route, K1) under "kernels"
-configs    = the other single-GPU configurations (tiny, pool64, the 32-pair sweep)
+configs    = the other single-GPU configurations (tiny, pool64, the 32-pair sweep); these and the
+             further measurements are on stderr, the line on stdout holds the headline
 cpu_baseline / --impl reference = the CPU oracle (literal per-candidate simulation) on
              every host core (and one core), with the host's core count and CPU model
 """
@@ -146,6 +147,21 @@ class Clocks:
             pass
         return {"sm_mhz": statistics.median(sm) if sm else None, "sm_max_mhz": smax, "samples": len(sm),
                 "reasons": sorted(reasons)}
+
+
+def _emit(line):
+    """One short JSON line on stdout (a reader that keeps the last few kB of the output still gets all
+    of it); every measurement, the other workloads' among them, as one line on stderr."""
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    pick = lambda d, *keys: None if d is None else {k: d[k] for k in keys if k in d}  # noqa: E731
+    short = {k: v for k, v in line.items() if not isinstance(v, (dict, list)) or k == "config"}
+    short["roofline"] = pick(line["roofline"], "kernel", "bound", "achieved", "peak", "unit", "frac", "peak_source",
+                             "algorithmic_bytes", "traffic", "target_met")
+    short["cpu_baseline"] = pick(line["cpu_baseline"], "value", "unit", "cores", "kind")
+    short["e2e"] = pick(line["e2e"], "value", "unit", "ms_per_step", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps",
+                        "p50_latency_ms", "p99_latency_ms")
+    short["clocks"] = pick(line["clocks"], "sm_mhz", "sm_max_mhz", "reasons")
+    print(json.dumps(short), flush=True)
 
 
 def run_gpu(args):
@@ -449,7 +465,7 @@ def run_gpu(args):
             "stream": stream,
             "policy_eval": policy_eval,
         }
-        print(json.dumps(line), flush=True)
+        _emit(line)
     rt.close()
     if world > 1:
         dist.destroy_process_group()
