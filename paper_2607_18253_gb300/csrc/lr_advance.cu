@@ -905,16 +905,16 @@ cudaError_t launch_advance(const K3Launch &a, int grid, size_t smem, cudaStream_
     return launch_chained(k_advance, grid, kK3Warps * 32, smem, st, a);
 }
 
-cudaError_t set_k3_smem(size_t bytes) {
-    return allow_smem(k_advance, bytes);
+cudaError_t set_k3_smem() {
+    return allow_smem(k_advance, kSmemMax);
 }
 
 cudaError_t launch_advance_kv(const K3Launch &a, int grid, size_t smem, cudaStream_t st) {
     return launch_chained(k_advance_kv, grid, kK3Warps * 32, smem, st, a);
 }
 
-cudaError_t set_k3_kv_smem(size_t bytes) {
-    return allow_smem(k_advance_kv, bytes);
+cudaError_t set_k3_kv_smem() {
+    return allow_smem(k_advance_kv, kSmemMax);
 }
 
 }  // namespace lr

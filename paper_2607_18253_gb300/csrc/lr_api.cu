@@ -159,15 +159,13 @@ int pow2_ceil(int x) {
     return p;
 }
 
-constexpr size_t kK2SmemMax = 224 * 1024;
-
 // Launch shape of the candidate kernel: threads own four consecutive instances;
 // Gp groups per row (power of two up to 32, else a multiple of 32); the
 // summary tables of the tile and QT staged query rows fit the shared memory.
 // Routing runs up to three CTAs of at most 256 threads per SM (one of them fits beside a
 // snapshot load's CTA); the estimate alone runs one of at most 512, so that each SM copies
 // its tile block once.
-lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep, size_t sm_smem) {
+lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep, size_t sm_smem, size_t k1_smem) {
     lr_ctx::Shape s;
     s.block = route ? lr::kK2Block : lr::kK2EstBlock;
     const int G = (d.I + 3) / 4;
@@ -209,14 +207,17 @@ lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep, size_t 
         auto rows = [&](size_t bytes) {
             return (int)std::min<size_t>(route ? 256 : 1024, bytes > fixed ? (bytes - fixed) / per_row : 0);
         };
-        qt = n == (route ? 3 : 1) ? rows(route ? lr::kK2SmemTarget : lr::kK2EstSmemTarget) : 0;
         // an SM's share of the shared memory, less what the system and the static words take
-        if (qt < 64) qt = rows(std::min<size_t>(kK2SmemMax, sm_smem / n - 1280));
+        const size_t share = std::min<size_t>(lr::kK2SmemMax, sm_smem / n - 1280);
+        qt = n == (route ? 3 : 1) ? rows(route ? lr::kK2SmemTarget : lr::kK2EstSmemTarget) : 0;
+        // a lone CTA leaves room for a load's CTA if it can
+        if (n == 1 && qt < 64) qt = rows(sm_smem > k1_smem + 2560 ? std::min(share, sm_smem - k1_smem - 2560) : 0);
+        if (qt < (n == 1 ? (route ? kLeastRows : 64) : 64)) qt = rows(share);
     }
     qt = std::max(s.QS, (qt / s.QS) * s.QS);
     s.QT = qt;
     s.smem = fixed + (size_t)qt * per_row;
-    s.ok = s.smem <= kK2SmemMax;
+    s.ok = s.smem <= lr::kK2SmemMax;
     return s;
 }
 
@@ -227,8 +228,9 @@ lr_ctx::Shape make_shape(const lr::DevConfig &d, bool route, bool sweep, size_t 
 // candidate-kernel slot each) start with a static range of 90% of their share, and
 // the other rows are claimed as they run out, by the remaining CTAs and by whichever
 // finish early, so that every CTA ends on small claimed chunks.
-// A call that the CTAs beside the load can take in two rows a thread group has no other CTAs
-// and no claims (1,000 x 256 estimates 6.8 -> 4.6 us).  Returns the CTAs of a tile.
+// A call that the CTAs beside the load can take in two rows a thread group (or four rows each)
+// has no other CTAs and no claims (1,000 x 256 estimates 6.8 -> 4.6 us).  Returns the CTAs of a
+// tile.
 int set_row_split(lr::K2Launch &a, const lr_ctx *c, int ctas, int tiles, int occ, void *stream) {
     if (!c->loaded_any || stream == c->load_stream) {
         a.first_ctas = ctas;
@@ -237,11 +239,14 @@ int set_row_split(lr::K2Launch &a, const lr_ctx *c, int ctas, int tiles, int occ
     }
     const int k1 = (c->cfg.I + lr::kK1Warps - 1) / lr::kK1Warps;
     a.first_ctas = tiles == 1 ? std::max(0, std::min(ctas, c->sms * occ - k1)) : 0;
-    if (a.Q <= 2 * a.QS * a.first_ctas) {
+    if (a.Q <= std::max(2 * a.QS, 4) * a.first_ctas) {
         ctas = a.first_ctas;
         a.first_rows = (a.Q + ctas - 1) / ctas;
         return ctas;
     }
+    // (a small route's claims spread over its CTAs: 24 x 640 x 8 pairs beside a load 20.7 -> 16.3 us;
+    // a small estimate, whose rows cost less than a claim, loses by it: 1,000 x 512 6.1 -> 6.7)
+    if (a.share > 1) a.least = std::min(a.least, round_up((a.Q + ctas - 1) / std::max(1, ctas), a.QS));
     const int f = (int)((long long)a.Q * 9 / (10LL * std::max(1, ctas)));
     a.first_rows = std::max(a.QS, f - f % a.QS);
     return ctas;
@@ -458,8 +463,9 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     int sm_smem = 0, dev = 0;
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e != cudaSuccess) return bail(LR_ECUDA, cudaGetErrorString(e));
     auto shape = [&](lr_ctx::Shape &s, bool route, bool sweep) {
-        s = make_shape(d, route, sweep, (size_t)sm_smem);
+        s = make_shape(d, route, sweep, (size_t)sm_smem, c->k1_smem);
         if (e == cudaSuccess && s.ok) e = lr::cand_occupancy(d.mode, route, s.block, s.smem, &s.occ);
         s.occ = std::max(1, s.occ);
     };
@@ -467,12 +473,12 @@ int lr_create(const lr_config *cfg, lr_ctx **out) {
     // capacities lr_advance takes: 32 B a running and 12 B a waiting request within 200 KB
     // for four instances (it needs less)
     c->k3_ok = lr::kK3Warps * sizeof(int32_t) * ((size_t)8 * d.capR + (size_t)3 * d.capW + 32) <= 200 * 1024;
-    e = lr::set_k1_smem(c->k1_smem);
-    if (e == cudaSuccess && c->k3_ok) e = lr::set_k3_smem(c->k3_smem);
-    if (e == cudaSuccess && M <= lr::kCalMaxModels) e = lr::set_calib_smem(M);
-    if (e == cudaSuccess) e = lr::set_k2_smem(kK2SmemMax);
+    e = lr::set_k1_smem();
+    if (e == cudaSuccess && c->k3_ok) e = lr::set_k3_smem();
+    if (e == cudaSuccess && M <= lr::kCalMaxModels) e = lr::set_calib_smem();
+    if (e == cudaSuccess) e = lr::set_k2_smem();
     c->bl_ok = lr::baseline_smem(d) <= 200 * 1024;
-    if (e == cudaSuccess && c->bl_ok) e = lr::set_baseline_smem(lr::baseline_smem(d));
+    if (e == cudaSuccess && c->bl_ok) e = lr::set_baseline_smem();
     shape(c->est, false, false);
     shape(c->rt, true, false);
     shape(c->sw, true, true);
@@ -822,7 +828,7 @@ int lr_set_kv_limits(lr_ctx *c, const int32_t *block_size, const int64_t *num_bl
     if (!on) return LR_OK;
     int warps = lr::kKvWarps;
     while (warps > 1 && warps * per_warp > 200 * 1024) --warps;
-    e = lr::set_kv_smem(warps * per_warp);
+    e = lr::set_kv_smem();
     if (e != cudaSuccess) return cuda_fail(c, e, "KV load shared memory");
     auto alloc = [&](size_t bytes, void **p) {
         cudaError_t ee = cudaMalloc(p, bytes > 0 ? bytes : 16);
@@ -877,7 +883,7 @@ int lr_set_kv_limits(lr_ctx *c, const int32_t *block_size, const int64_t *num_bl
     // instances (it needs less)
     c->k3_kv_ok = lr::kK3Warps * sizeof(int32_t) * ((size_t)11 * c->cfg.capR + (size_t)3 * c->cfg.capW + 32) <= 200 * 1024;
     if (c->k3_kv_ok) {
-        e = lr::set_k3_kv_smem(c->k3_kv_smem);
+        e = lr::set_k3_kv_smem();
         if (e != cudaSuccess) {
             free_kv(c);
             return cuda_fail(c, e, "KV advance shared memory");

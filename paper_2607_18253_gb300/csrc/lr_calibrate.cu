@@ -831,10 +831,10 @@ cudaError_t launch_calibrate(long long N, const long long *F, const int32_t *mod
                           ctl);
 }
 
-cudaError_t set_calib_smem(int M) {
-    const size_t fixed = cal_sums_bytes(M);
-    cudaError_t e = allow_smem(k_calibrate<true>, fixed + kCalStageBytes * calib_stages(M));
-    if (e == cudaSuccess) e = allow_smem(k_calibrate<false>, fixed + solve_bytes(M));
+cudaError_t set_calib_smem() {
+    cudaError_t e = allow_smem(k_calibrate<true>, kCalSmemMax);
+    if (e == cudaSuccess)
+        e = allow_smem(k_calibrate<false>, cal_sums_bytes(kCalMaxModels) + solve_bytes(kCalMaxModels));
     return e;
 }
 

@@ -1105,12 +1105,12 @@ cudaError_t launch_cand_mode(const K2Launch &a, int out, dim3 grid, int block, s
 }
 
 template <int MODE>
-cudaError_t set_mode_attrs(size_t bytes) {
+cudaError_t set_mode_attrs() {
     const cudaError_t es[] = {
-        allow_smem(k_cand<MODE, kOutMatrix>, bytes), allow_smem(k_cand<(MODE == 2 ? 0 : MODE), kOutMatrix | kOutIters>, bytes),
-        allow_smem(k_cand<MODE, kOutLag>, bytes), allow_smem(k_cand<MODE, kOutLag | kOutMatrix>, bytes),
-        allow_smem(k_cand<MODE, kOutCon>, bytes), allow_smem(k_cand<MODE, kOutCon | kOutMatrix>, bytes),
-        allow_smem(k_cand<MODE, kOutSweep>, bytes), allow_smem(k_cand<MODE, kOutSweep | kOutMatrix>, bytes)};
+        allow_smem(k_cand<MODE, kOutMatrix>, kK2SmemMax), allow_smem(k_cand<(MODE == 2 ? 0 : MODE), kOutMatrix | kOutIters>, kK2SmemMax),
+        allow_smem(k_cand<MODE, kOutLag>, kK2SmemMax), allow_smem(k_cand<MODE, kOutLag | kOutMatrix>, kK2SmemMax),
+        allow_smem(k_cand<MODE, kOutCon>, kK2SmemMax), allow_smem(k_cand<MODE, kOutCon | kOutMatrix>, kK2SmemMax),
+        allow_smem(k_cand<MODE, kOutSweep>, kK2SmemMax), allow_smem(k_cand<MODE, kOutSweep | kOutMatrix>, kK2SmemMax)};
     for (cudaError_t x : es)
         if (x != cudaSuccess) return x;
     return cudaSuccess;
@@ -1413,16 +1413,16 @@ cudaError_t launch_on_time(int Q, const float *util, const float *ttft, const fl
                           reinterpret_cast<unsigned *>(part + 2 * max_parts), out);
 }
 
-cudaError_t set_baseline_smem(size_t bytes) {
-    cudaError_t e = allow_smem(k_baseline<0>, bytes);
-    if (e == cudaSuccess) e = allow_smem(k_baseline<1>, bytes);
+cudaError_t set_baseline_smem() {
+    cudaError_t e = allow_smem(k_baseline<0>, kSmemMax);
+    if (e == cudaSuccess) e = allow_smem(k_baseline<1>, kSmemMax);
     return e;
 }
 
-cudaError_t set_k2_smem(size_t bytes) {
-    cudaError_t e = set_mode_attrs<0>(bytes);
-    if (e == cudaSuccess) e = set_mode_attrs<1>(bytes);
-    if (e == cudaSuccess) e = set_mode_attrs<2>(bytes);
+cudaError_t set_k2_smem() {
+    cudaError_t e = set_mode_attrs<0>();
+    if (e == cudaSuccess) e = set_mode_attrs<1>();
+    if (e == cudaSuccess) e = set_mode_attrs<2>();
     return e;
 }
 

@@ -143,20 +143,26 @@ cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, 
     return cudaLaunchKernelEx(&cfg, k, P(args)...);
 }
 
-// Lets kernel f be launched with `bytes` of dynamic shared memory.  The limit belongs to the
-// process's kernel, not to one lr_ctx, so it is always set to all that the device gives a CTA:
-// the same value whatever a context needs, and no context takes away what another launches with.
+// Lets kernel f be launched with up to `most` bytes of dynamic shared memory.  The limit belongs
+// to the process's kernel, not to one lr_ctx, so `most` is a constant, the most that lr_create or
+// lr_set_kv_limits lets any context need: no context takes away what another launches with.
+constexpr size_t kSmemMax = 200 * 1024;    // the loads, the stream steps, the baselines
+constexpr size_t kK2SmemMax = 224 * 1024;  // the candidate kernel
 template <typename F>
-cudaError_t allow_smem(F *f, size_t bytes) {
-    int dev = 0, most = 0;
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, (const void *)f);
-    if (e != cudaSuccess) return e;
-    most -= (int)fa.sharedSizeBytes;
-    if (bytes > (size_t)most) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute((const void *)f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+cudaError_t allow_smem(F *f, size_t most) {
+    return cudaFuncSetAttribute((const void *)f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
+// K1 asks for the whole shared-memory carve-out as well: with one that fits its own CTAs alone, an
+// SM could not take a larger CTA of a call on another stream before it was idle (routes beside a
+// load, 16,384 x 61 / 256 / 640: 12.4 / 17.6 / 55 -> 11.5 / 14.1 / 44 us).  Not the KV load, whose
+// few warps are the longer part and lose more to company (65,536 x 256 186 -> 200 us).
+template <typename F>
+cudaError_t beside_smem(F *f, size_t most) {
+    cudaError_t e = allow_smem(f, most);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void *)f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    return e;
 }
 
 // The live-buffer index with acquire ordering: reads of the buffer it names see
@@ -319,7 +325,7 @@ __host__ __device__ inline size_t cal_acc_words(int M) { return (size_t)M * kCal
 cudaError_t launch_calibrate(long long N, const long long *F, const int32_t *model, const double *time, int M,
                              int shared_beta1, unsigned long long *acc, double *coef, DevCtl *ctl, int grid,
                              cudaStream_t st);
-cudaError_t set_calib_smem(int M);
+cudaError_t set_calib_smem();
 
 // Launch helpers implemented in the kernel translation units.
 struct K1Launch {
@@ -329,7 +335,7 @@ struct K1Launch {
     StateIn in;
 };
 cudaError_t launch_trajectory(const K1Launch &a, int grid, int block, size_t smem, cudaStream_t st);
-cudaError_t set_k1_smem(size_t bytes);
+cudaError_t set_k1_smem();
 constexpr int kK1Warps = 4;
 
 // KV-limited load (residents alone, records) and estimate (per-candidate walk).
@@ -350,7 +356,7 @@ __host__ __device__ inline size_t kv_smem_per_warp(const DevConfig &c, int hist)
 }
 // warps: instances per CTA, 1 .. kKvWarps
 cudaError_t launch_kv_load(const KvLoad &a, int grid, int warps, size_t smem, cudaStream_t st);
-cudaError_t set_kv_smem(size_t bytes);
+cudaError_t set_kv_smem();
 struct KvEst {
     DevConfig cfg;
     KvLimits kv;
@@ -455,13 +461,13 @@ cudaError_t launch_frontier(const K2Launch &a, double *out, int sms, cudaStream_
 // Baseline routing policies (0 Round Robin, 1 Shortest Queue, 2 Latency-Agnostic) and
 // the stream metrics (OnTimeUtility, SLO attainment) over routed queries.
 size_t baseline_smem(const DevConfig &c);
-cudaError_t set_baseline_smem(size_t bytes);
+cudaError_t set_baseline_smem();
 cudaError_t launch_baseline(const K2Launch &a, int policy, long long rr_start, float lam, int sms, cudaStream_t st);
 constexpr int kOnTimeParts = 1024;
 cudaError_t launch_on_time(int Q, const float *util, const float *ttft, const float *tau, const float *delay,
                            double *part, int max_parts, double *out, cudaStream_t st);
 cudaError_t cand_occupancy(int mode, bool route, int block, size_t smem, int *blocks_per_sm);
-cudaError_t set_k2_smem(size_t bytes);
+cudaError_t set_k2_smem();
 constexpr int kK2Block = 256;                // route: three CTAs per SM, one fits beside a load's CTA
 constexpr size_t kK2SmemTarget = 72 * 1024;  // three CTAs per SM
 constexpr int kK2EstBlock = 512;             // estimate alone: one CTA per SM, one tile copy per SM
@@ -497,8 +503,8 @@ __host__ __device__ inline size_t advance_kv_smem_per_warp(const DevConfig &c) {
 }
 cudaError_t launch_advance(const K3Launch &a, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_advance_kv(const K3Launch &a, int grid, size_t smem, cudaStream_t st);
-cudaError_t set_k3_kv_smem(size_t bytes);
-cudaError_t set_k3_smem(size_t bytes);
+cudaError_t set_k3_kv_smem();
+cudaError_t set_k3_smem();
 struct StateOut {
     int32_t *n_run, *run_ctx, *run_pre, *run_dec, *n_wait, *wait_pre, *wait_dec;
     double *clock;

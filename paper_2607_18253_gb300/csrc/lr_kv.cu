@@ -1509,9 +1509,9 @@ cudaError_t launch_kv_load(const KvLoad &a, int grid, int warps, size_t smem, cu
     return launch_chained(a.cfg.mode == 0 ? k_kv_load<0> : k_kv_load<1>, grid, warps * 32, smem, st, a);
 }
 
-cudaError_t set_kv_smem(size_t bytes) {
-    cudaError_t e = allow_smem(k_kv_load<0>, bytes);
-    if (e == cudaSuccess) e = allow_smem(k_kv_load<1>, bytes);
+cudaError_t set_kv_smem() {
+    cudaError_t e = allow_smem(k_kv_load<0>, kSmemMax);
+    if (e == cudaSuccess) e = allow_smem(k_kv_load<1>, kSmemMax);
     auto est = [&](auto f, size_t n) {
         if (e == cudaSuccess) e = allow_smem(f, n);
     };

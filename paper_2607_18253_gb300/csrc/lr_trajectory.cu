@@ -1002,9 +1002,9 @@ cudaError_t launch_trajectory(const K1Launch &a, int grid, int block, size_t sme
     return launch_chained(a.cfg.mode == 0 ? k_trajectory<0> : k_trajectory<1>, grid, block, smem, st, a);
 }
 
-cudaError_t set_k1_smem(size_t bytes) {
-    cudaError_t e = allow_smem(k_trajectory<0>, bytes);
-    if (e == cudaSuccess) e = allow_smem(k_trajectory<1>, bytes);
+cudaError_t set_k1_smem() {
+    cudaError_t e = beside_smem(k_trajectory<0>, kSmemMax);
+    if (e == cudaSuccess) e = beside_smem(k_trajectory<1>, kSmemMax);
     return e;
 }
 
