@@ -42,8 +42,8 @@ WORKLOAD = "pool256"
 # DRAM bytes (read + write) per launch of the step's kernels on this workload, from one
 # ncu capture of the kernels as they are built now (summaries under profiles/); they
 # are retaken whenever one of the kernels changes.
-NCU_TRAFFIC = {"k_route": 4_586_240 + 8_535_296, "k_trajectory": 1_398_272, "k_estimate": 381_952 + 7_250_432,
-               "k_calibrate": 208_709_632 + 3_387_392}
+NCU_TRAFFIC = {"k_route": 4_579_840 + 7_786_496, "k_trajectory": 1_398_272, "k_estimate": 376_576 + 7_384_320,
+               "k_calibrate": 208_710_912 + 3_696_896}
 
 
 def _peaks():
@@ -725,8 +725,8 @@ def run_kv(args, dev, wl, flush):
                                    "k_kv_estimate, k_kv_expand)", "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
                          "frac": ach / hbm, "peak_source": f"{src} (MEASURED_PEAKS.json hbm_gbs, copy)",
                          "algorithmic_bytes": nbytes, "traffic": None,
-                         "note": "the call's six kernels together; k_kv_estimate alone read 2.48 MB and wrote "
-                                 "0.93 MB per launch (ncu); the load is one dependency chain per instance"}}
+                         "note": "the call's six kernels together; k_kv_estimate alone read 2.58 MB and wrote "
+                                 "1.03 MB per launch (ncu); the load is one dependency chain per instance"}}
 
 
 def run_avgcase(args, dev, wl, flush):

@@ -254,9 +254,10 @@ LR_API int lr_set_ttft_source(lr_ctx *ctx, int32_t source);
  * With limits on, lr_route and lr_route_frontier_static first write the KV-limited
  * estimate matrix (to ttft_matrix_out if given, else to library memory) and score
  * and pick over it; lr_route_baseline reports the chosen instance's KV-limited time;
- * lr_advance executes the same rule; the average-case sources return LR_EINVAL.  Each estimate call
- * runs one walk per distinct prompt length (the queries are counting-sorted by
- * length in library memory sized by max_queries).  Memory taken here: per buffer
+ * lr_advance executes the same rule; the average-case sources return LR_EINVAL.  An estimate
+ * call of few queries walks each of them; a larger one runs one walk per distinct prompt
+ * length (the queries are counting-sorted by length in library memory sized by
+ * max_queries).  Memory taken here: per buffer
  * 68 B x I x horizon of records, and max_queries x (8 B + 4 B x I) for the sort
  * and the routed matrix (LR_ENOMEM if it cannot be had; nothing is allocated
  * later, so routing stays allocation-free).  Device errors: a snapshot in which a running request other than the last is
@@ -305,8 +306,9 @@ LR_API int lr_calibrate(lr_ctx *ctx, int64_t N, const int64_t *features, const i
  * those limits.  There a query whose prompt is not below max_ctx, or whose whole context
  * (capped at max_ctx) needs more blocks than the instance has, records LR_EINVAL; a
  * waiting queue that preemptions grow past cap_waiting records LR_ECAPACITY; either keeps
- * the previous snapshot live.  The KV step needs 4 x (11 cap_running + 3 cap_waiting + 32)
- * bytes of shared memory per instance, at most 200 KB for 4 (LR_ECAPACITY otherwise). */
+ * the previous snapshot live.  The KV step takes capacities of which four instances'
+ * 4 x (11 cap_running + 3 cap_waiting + 32) bytes are at most 200 KB (LR_ECAPACITY
+ * otherwise; the shared memory it uses is less). */
 LR_API int lr_advance(lr_ctx *ctx, int32_t Q, const int32_t *assign, const int32_t *prompt_len,
                       const int32_t *dec, int32_t dec_cols, double t_now, void *cuda_stream);
 

@@ -1373,7 +1373,7 @@ cudaError_t launch_features(const K2Launch &a, int sms, cudaStream_t st) {
 
 cudaError_t launch_frontier(const K2Launch &a, double *out, int sms, cudaStream_t st) {
     // CTAs per pair: a power of two up to 8 (the portable cluster size), while the pairs
-    // leave SMs free and each CTA still has 512 queries
+    // leave SMs free and each CTA still has more than 256 queries
     int cs = 1;
     while (cs < 8 && 2 * cs * a.P <= sms && 512 * cs < a.Q) cs *= 2;
     cudaLaunchConfig_t cfg = {};

@@ -1,7 +1,8 @@
 """The candidate kernel's paths against the CPU oracle, bit for bit: instance counts around the
-warp and tile edges (rows that are not whole 16-byte words are put in order in shared memory),
-prompts around the bound up to which a candidate's two table entries stay in registers, sweeps
-with every lane split, and instances whose prefill total is not exact in fp32.
+warp and tile edges (rows that are not whole 16-byte words: stored value by value, by the
+average-case sources in order through shared memory), prompts around the bound up to which a
+candidate's two table entries stay in registers, sweeps with every lane split, and instances
+whose prefill total is not exact in fp32.
 
 Times, utilities and assignments are compared exactly (both sides evaluate the same sequence
 of IEEE operations)."""
