@@ -261,7 +261,7 @@ int set_row_split(lr::K2Launch &a, const lr_ctx *c, int ctas, int tiles, int occ
 // together.  Fitted to all splits of 28 calls of 2 to 64 pairs on 8 to 1,024 instances, of
 // which it takes the fastest or one within 5%.  One lane per (row, pair) whatever the call left
 // a chunk of few pairs to one warp in eight: 32,768 queries x 2 pairs on 256 / 512 / 1,024
-// instances 40 / 576 / 4,197 us, now 23 / 45 / 110.
+// instances 40 / 576 / 4,197 us, now 23 / 63 / 110.
 void set_sweep_lanes(lr::K2Launch &a, int I, int warps, int ctas, int ctas_sm) {
     const int rows = std::min(a.QT, (a.Q + ctas - 1) / ctas), G = (I + 3) / 4;
     double least = 0.0;
